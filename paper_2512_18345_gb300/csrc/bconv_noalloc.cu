@@ -140,7 +140,7 @@ extern "C" int fhe_bconv_noalloc(fhe_ctx *c, const uint32_t *in, const int *in_i
   SegList sl;
   memset(&sl, 0, sizeof sl);
   for (int j = 0; j < n_in; j++) {
-    Seg &x = sl.seg[sl.nseg++];
+    Seg x{};
     x.src = in + (size_t)j * N;
     x.dst = y + (size_t)j * N;
     x.n = 1;
@@ -149,7 +149,7 @@ extern "C" int fhe_bconv_noalloc(fhe_ctx *c, const uint32_t *in, const int *in_i
     x.src_prime = -1;
     x.scale = dPre + j;
     x.galois = 1;
-    sl.total += 1;
+    seg_push(sl, x);
   }
   e = launch_ew(c->tabs, EW_SCALE, sl, s);
   if (e != cudaSuccess) return fhe_fail(FHE_ECUDA, "fhe_bconv_noalloc: scale: %s", cudaGetErrorString(e));

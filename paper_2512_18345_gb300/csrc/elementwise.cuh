@@ -29,22 +29,18 @@ __global__ void __launch_bounds__(kEwThreads) k_ew(const __grid_constant__ SegLi
   const int blocks_per_limb = (int)(N / (4 * kEwThreads));
   const int v = blockIdx.x / blocks_per_limb;
   const uint32_t j0 = (uint32_t)((blockIdx.x % blocks_per_limb) * 4 * kEwThreads + threadIdx.x * 4);
-  int within;
-  const Seg &sg = seg_at(sl, seg_find(sl, v, within));
-  const KsArgs &ks = item_ks(sl, sg);
-  const int prime = sg.prime + within;
-  const PrimeC P = pc[prime];
+  const Limb lb = limb_at<OP == EW_COMBINE>(sl, v, nullptr, logn);
+  const PrimeC P = pc[lb.prime];
   const uint32_t q = P.q;
-  const uint32_t *src = sg.src ? sg.src + (size_t)within * sg.src_stride * N : nullptr;
-  const uint32_t *src2 = sg.src2 ? sg.src2 + (size_t)within * N : nullptr;
-  uint32_t *dst = sg.dst + (size_t)within * N;
+  const uint32_t *src = lb.src, *src2 = lb.src2;
+  uint32_t *dst = lb.dst;
   uint32_t o[4];
   if (OP == EW_TENSOR) {  // the segment covers one ciphertext's limbs; n = level is the poly stride
-    const size_t poly = (size_t)sg.n * N, off = (size_t)within * N + j0;
-    const uint4 A0 = __ldg(reinterpret_cast<const uint4 *>(sg.src + off));
-    const uint4 A1 = __ldg(reinterpret_cast<const uint4 *>(sg.src + poly + off));
-    const uint4 B0 = __ldg(reinterpret_cast<const uint4 *>(sg.src2 + off));
-    const uint4 B1 = __ldg(reinterpret_cast<const uint4 *>(sg.src2 + poly + off));
+    const size_t poly = (size_t)lb.n * N;
+    const uint4 A0 = __ldg(reinterpret_cast<const uint4 *>(src + j0));
+    const uint4 A1 = __ldg(reinterpret_cast<const uint4 *>(src + poly + j0));
+    const uint4 B0 = __ldg(reinterpret_cast<const uint4 *>(src2 + j0));
+    const uint4 B1 = __ldg(reinterpret_cast<const uint4 *>(src2 + poly + j0));
     const uint32_t a0[4] = {A0.x, A0.y, A0.z, A0.w}, a1[4] = {A1.x, A1.y, A1.z, A1.w};
     const uint32_t b0[4] = {B0.x, B0.y, B0.z, B0.w}, b1[4] = {B1.x, B1.y, B1.z, B1.w};
     uint32_t d0[4], d1[4], d2[4];
@@ -54,7 +50,7 @@ __global__ void __launch_bounds__(kEwThreads) k_ew(const __grid_constant__ SegLi
       d1[x] = reduce_u64((uint64_t)a0[x] * b1[x] + (uint64_t)a1[x] * b0[x], P);  // < 2^63
       d2[x] = mul_mod(a1[x], b1[x], P);
     }
-    uint32_t *d = sg.dst + off;
+    uint32_t *d = dst + j0;
     *reinterpret_cast<uint4 *>(d) = make_uint4(d0[0], d0[1], d0[2], d0[3]);
     *reinterpret_cast<uint4 *>(d + poly) = make_uint4(d1[0], d1[1], d1[2], d1[3]);
     *reinterpret_cast<uint4 *>(d + 2 * poly) = make_uint4(d2[0], d2[1], d2[2], d2[3]);
@@ -62,7 +58,7 @@ __global__ void __launch_bounds__(kEwThreads) k_ew(const __grid_constant__ SegLi
   }
   if (OP == EW_GATHER) {
 #pragma unroll
-    for (int e = 0; e < 4; e++) o[e] = __ldg(src + galois_src(j0 + e, sg.galois, logn));
+    for (int e = 0; e < 4; e++) o[e] = __ldg(src + galois_src(j0 + e, lb.galois, logn));
   } else {
     const uint4 a = __ldg(reinterpret_cast<const uint4 *>(src + j0));
     const uint32_t av[4] = {a.x, a.y, a.z, a.w};
@@ -72,8 +68,7 @@ __global__ void __launch_bounds__(kEwThreads) k_ew(const __grid_constant__ SegLi
       bv[0] = b.x; bv[1] = b.y; bv[2] = b.z; bv[3] = b.w;
     }
     uint2 sc = make_uint2(0, 0);
-    if (OP == EW_SCALE) sc = sg.scale[within];
-    if (OP == EW_COMBINE) sc = ks.pinv[prime];
+    if (OP == EW_SCALE || OP == EW_COMBINE) sc = __ldg(lb.scale);
 #pragma unroll
     for (int e = 0; e < 4; e++) {
       if (OP == EW_SCALE) o[e] = shoup(av[e], sc.x, sc.y, q);

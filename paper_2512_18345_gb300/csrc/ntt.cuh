@@ -41,7 +41,7 @@ struct NttTables {
 // Prologue modes (how pass 1 reads an element)
 enum : int {
   PRO_PLAIN = 0,   // src[j]
-  PRO_GATHER = 1,  // src[sigma(j)], sigma = ks.galois_own (NTT form input)
+  PRO_GATHER = 1,  // src[sigma(j)], sigma = the limb's galois (NTT form input)
   PRO_REDUCE = 2,  // src[j] reduced from another prime (rescale: src_prime)
 };
 // Epilogue modes (how the last pass writes an element)
@@ -112,15 +112,16 @@ constexpr int kOtfSmall = 8;
 //     xfer[(r & 15) * 256 + col];
 // and the second pass reads the value of (r, col) from the CTA that owns it.
 template <int LOGN, bool COLUMN, bool FWD, int PRO, int EPI, bool OTF, int SRCM, int DSTM>
-__device__ __forceinline__ void ntt_pass(const Seg &sg, const KsArgs &ks, int within, int prime, const NttTables &tb,
-                                         int tile, uint32_t *sm, uint2 *tws, uint32_t *xfer) {
+__device__ __forceinline__ void ntt_pass(const Limb &lb, const NttTables &tb, int tile,
+                                         uint32_t *sm, uint2 *tws, uint32_t *xfer) {
   using G = NttGeom<LOGN, COLUMN>;
   constexpr int R = G::R, N = G::N, S0 = COLUMN ? 0 : LOGN - 8;
+  const int prime = lb.prime;
   const PrimeC P = tb.pc[prime];
   const uint32_t q = P.q;
   const uint2 *tw = (FWD ? tb.tw_fwd : tb.tw_inv) + (size_t)prime * N;
-  const uint32_t *src = sg.src + (size_t)within * sg.src_stride * N;
-  uint32_t *dst = sg.dst + (size_t)within * N;
+  const uint32_t *src = lb.src;
+  uint32_t *dst = lb.dst;
   const int tid = threadIdx.x;
 
   if (COLUMN) {
@@ -213,7 +214,7 @@ __device__ __forceinline__ void ntt_pass(const Seg &sg, const KsArgs &ks, int wi
     for (int e = 0; e < 16; e++) {
       const uint32_t j = G::gidx(tile, c, kmap<R>(hi0, e, tau));
       if (PRO == PRO_GATHER)
-        x[e] = __ldg(src + galois_src(j, ks.galois_own, LOGN));
+        x[e] = __ldg(src + galois_src(j, lb.galois, LOGN));
       else if (PRO == PRO_REDUCE)  // value of another prime's limb, reduced exactly mod q
         x[e] = reduce_u64(__ldg(src + j), P);
       else
@@ -317,14 +318,12 @@ __device__ __forceinline__ void ntt_pass(const Seg &sg, const KsArgs &ks, int wi
     return;
   }
   uint2 scale = make_uint2(0, 0);
-  if (EPI == EPI_SCALE || EPI == EPI_RESCALE) scale = sg.scale ? sg.scale[within] : tb.ninv[prime];
-  uint2 pinv = make_uint2(0, 0);
-  if (EPI == EPI_COMBINE) pinv = ks.pinv[prime];
+  if (EPI == EPI_SCALE || EPI == EPI_RESCALE || EPI == EPI_COMBINE) scale = __ldg(lb.scale);
   const bool contiguous = !COLUMN && !hiL;  // forward block pass: 16 consecutive elements per thread
   const uint32_t j0 = G::gidx(tile, c, kmap<R>(hiL, 0, tau));
   uint32_t a[16];  // second operand of the combine / rescale epilogues
   if (EPI == EPI_RESCALE || EPI == EPI_COMBINE) {
-    const uint32_t *s2 = sg.src2 + (size_t)within * N;
+    const uint32_t *s2 = lb.src2;
     if (contiguous) {
 #pragma unroll
       for (int e4 = 0; e4 < 4; e4++) {
@@ -352,7 +351,7 @@ __device__ __forceinline__ void ntt_pass(const Seg &sg, const KsArgs &ks, int wi
     } else if (EPI == EPI_RESCALE) {
       o = shoup(a[e] + q - red2(val, q), scale.x, scale.y, q);
     } else {  // EPI_COMBINE: a = inner product u (with P times the pass-through term folded in)
-      o = shoup(a[e] + q - red2(val, q), pinv.x, pinv.y, q);
+      o = shoup(a[e] + q - red2(val, q), scale.x, scale.y, q);
     }
     x[e] = o;
   }
@@ -389,12 +388,8 @@ __global__ void __launch_bounds__(kNttThreads, ntt_min_blocks<COLUMN, FWD, PRO, 
   extern __shared__ __align__(16) uint2 tws[];  // dynamic: ntt_twiddle_smem(COLUMN, S) bytes (+ the small table)
 
   const int v = blockIdx.x / G::TILES, tile = blockIdx.x % G::TILES;
-  int within;
-  const int si = seg_find(sl, v, within);
-  const Seg &sg = seg_at(sl, si);
-  const KsArgs &ks = item_ks(sl, sg);
-  ntt_pass<LOGN, COLUMN, FWD, PRO, EPI, OTF, SRC_GLOBAL, DST_GLOBAL>(sg, ks, within, sg.prime + within, tb, tile, sm,
-                                                                     tws, nullptr);
+  const Limb lb = limb_at<EPI == EPI_COMBINE>(sl, v, tb.ninv, LOGN);
+  ntt_pass<LOGN, COLUMN, FWD, PRO, EPI, OTF, SRC_GLOBAL, DST_GLOBAL>(lb, tb, tile, sm, tws, nullptr);
 }
 
 // Both passes of a 2^16-point transform in one launch: a cluster of 16 CTAs per limb, CTA
@@ -412,20 +407,16 @@ __global__ void __cluster_dims__(16, 1, 1) __launch_bounds__(kNttThreads)
   __shared__ uint32_t xfer[kTile];
   extern __shared__ __align__(16) uint2 tws[];  // the larger of the two passes' staged twiddles
   const int v = blockIdx.x / 16, tile = blockIdx.x % 16;
-  int w1, w2;
-  const Seg &s1 = seg_at(first, seg_find(first, v, w1));
-  const Seg &s2 = seg_at(second, seg_find(second, v, w2));
-  const KsArgs &k1 = item_ks(first, s1);
-  const KsArgs &k2 = item_ks(second, s2);
-  const int prime = s1.prime + w1;
+  const Limb l1 = limb_at<false>(first, v, nullptr, LOGN);
+  const Limb l2 = limb_at<EPI == EPI_COMBINE>(second, v, tb.ninv, LOGN);
   // forward: column pass then block pass; inverse: block pass then column pass
   // (the passes pair a split cluster barrier: pass 1 arrives after publishing its tile and
   // pass 2 waits just before reading the cluster, so pass 2's twiddle loads overlap the
   // wait; pass 2 arrives after its reads and the CTA waits before exiting, so no CTA's
   // shared memory goes away while another reads it)
-  ntt_pass<LOGN, FWD, FWD, PRO, EPI_LAZY, OTF, SRC_GLOBAL, DST_LOCAL>(s1, k1, w1, prime, tb, tile, sm, tws, xfer);
+  ntt_pass<LOGN, FWD, FWD, PRO, EPI_LAZY, OTF, SRC_GLOBAL, DST_LOCAL>(l1, tb, tile, sm, tws, xfer);
   __syncthreads();  // pass 1's last reads of the staged twiddles come before pass 2 restages them
-  ntt_pass<LOGN, !FWD, FWD, PRO_PLAIN, EPI, OTF, SRC_CLUSTER, DST_GLOBAL>(s2, k2, w2, prime, tb, tile, sm, tws, xfer);
+  ntt_pass<LOGN, !FWD, FWD, PRO_PLAIN, EPI, OTF, SRC_CLUSTER, DST_GLOBAL>(l2, tb, tile, sm, tws, xfer);
   cluster_wait();
 }
 
@@ -469,10 +460,8 @@ __global__ void __launch_bounds__(kNttThreads)
   extern __shared__ __align__(16) uint2 tws[];     // the larger of the two passes' staged twiddles
   const int units = first.total * 16;
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
-    int w;
-    const Seg &sg = seg_at(first, seg_find(first, u >> 4, w));
-    ntt_pass<LOGN, FWD, FWD, PRO, EPI_LAZY, false, SRC_GLOBAL, DST_GLOBAL>(sg, item_ks(first, sg), w, sg.prime + w, tb,
-                                                                         u & 15, sm, tws, nullptr);
+    const Limb lb = limb_at<false>(first, u >> 4, nullptr, LOGN);
+    ntt_pass<LOGN, FWD, FWD, PRO, EPI_LAZY, false, SRC_GLOBAL, DST_GLOBAL>(lb, tb, u & 15, sm, tws, nullptr);
     __syncthreads();  // the tile and the staged twiddles are reused by the next unit
   }
   if (!grid_barrier_bounded(ctr, gridDim.x)) {
@@ -480,10 +469,8 @@ __global__ void __launch_bounds__(kNttThreads)
     return;
   }
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
-    int w;
-    const Seg &sg = seg_at(second, seg_find(second, u >> 4, w));
-    ntt_pass<LOGN, !FWD, FWD, PRO_PLAIN, EPI, false, SRC_GLOBAL, DST_GLOBAL>(sg, item_ks(second, sg), w, sg.prime + w,
-                                                                           tb, u & 15, sm, tws, nullptr);
+    const Limb lb = limb_at<EPI == EPI_COMBINE>(second, u >> 4, tb.ninv, LOGN);
+    ntt_pass<LOGN, !FWD, FWD, PRO_PLAIN, EPI, false, SRC_GLOBAL, DST_GLOBAL>(lb, tb, u & 15, sm, tws, nullptr);
     __syncthreads();
   }
 }

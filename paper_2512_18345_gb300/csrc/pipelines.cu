@@ -52,8 +52,7 @@ struct SegBuilder {
   }
   void add(const Seg &s) {
     if (s.n <= 0) return;
-    l.seg[l.nseg++] = s;
-    l.total += s.n;
+    seg_push(l, s);
   }
 };
 
@@ -329,9 +328,9 @@ static int transform(fhe_ctx *c, uint32_t *a, const int *idx, int n, bool fwd, f
   int i = 0;
   while (i < n) {
     SegBuilder sb;
-    while (i < n && sb.l.nseg < kMaxSeg) {
+    while (i < n && sb.l.nseg < kMaxSeg && sb.l.total + kMaxPrimes <= kMaxInlineLimbs) {
       int j = i + 1;
-      while (j < n && idx[j] == idx[j - 1] + 1) j++;
+      while (j < n && idx[j] == idx[j - 1] + 1) j++;  // at most kMaxPrimes limbs
       sb.add(mkseg(a + (size_t)i * N, a + (size_t)i * N, j - i, idx[i]));
       i = j;
     }

@@ -167,7 +167,9 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, Progra
       add(gather, gs);
       src = S.TMP;
     }
-    add(i1, seg(src, S.Y, level, 0, (int)i));
+    Seg g1 = seg(src, S.Y, level, 0, (int)i);
+    g1.galois = P.ks[i].galois_own;  // read by PRO_GATHER
+    add(i1, g1);
     Seg y = seg(S.Y, S.Y, level, 0, (int)i);
     if (fused) y.scale = c->d_mu_scale + (size_t)(level - 1) * L;
     add(i2, y);
@@ -366,8 +368,12 @@ static cudaError_t launch_stage(fhe_ctx *c, const Stage &st, const SegList &sl, 
 
 bool program_fits_inline(const Program &P) {
   if ((int)P.ks.size() > kMaxInlineItems) return false;
-  for (const Stage &st : P.stages)
+  for (const Stage &st : P.stages) {
     if ((int)st.segs.size() > kMaxSeg || (int)st.groups.size() > kMaxBconvGroups) return false;
+    int limbs = 0;
+    for (const Seg &x : st.segs) limbs += x.n;
+    if (limbs > kMaxInlineLimbs) return false;
+  }
   return true;
 }
 
@@ -379,14 +385,8 @@ int run_program_inline(fhe_ctx *c, const Program &P, cudaStream_t s) {
     memset(&sl, 0, sizeof sl);
     memset(&sl2, 0, sizeof sl2);
     memset(&ba, 0, sizeof ba);
-    for (const Seg &x : st.segs) {
-      sl.seg[sl.nseg++] = x;
-      sl.total += x.n;
-    }
-    for (const Seg &x : st.segs2) {
-      sl2.seg[sl2.nseg++] = x;
-      sl2.total += x.n;
-    }
+    for (const Seg &x : st.segs) seg_push(sl, x);
+    for (const Seg &x : st.segs2) seg_push(sl2, x);
     for (size_t i = 0; i < P.ks.size(); i++) sl.ks[i] = sl2.ks[i] = P.ks[i];
     if (st.kind == Stage::IP && st.gather_ext) {
       // the hoisted inner product takes the limbs limb by limb across runs of like segments
@@ -421,6 +421,7 @@ int upload_program(fhe_ctx *c, const Program &P, DevProgram &D) {
   bytes = align(bytes);
   std::vector<size_t> seg_off(P.stages.size()), map_off(P.stages.size()), grp_off(P.stages.size());
   std::vector<size_t> seg2_off(P.stages.size()), map2_off(P.stages.size());
+  std::vector<size_t> limb_off(P.stages.size()), limb2_off(P.stages.size());
   for (size_t i = 0; i < P.stages.size(); i++) {
     const Stage &st = P.stages[i];
     int total = 0, total2 = 0;
@@ -436,6 +437,10 @@ int upload_program(fhe_ctx *c, const Program &P, DevProgram &D) {
     bytes = align(bytes + sizeof(Seg) * st.segs2.size());
     map2_off[i] = bytes;
     bytes = align(bytes + sizeof(int2) * total2);
+    limb_off[i] = bytes;
+    bytes = align(bytes + sizeof(Limb) * total);
+    limb2_off[i] = bytes;
+    bytes = align(bytes + sizeof(Limb) * total2);
   }
   std::vector<char> host(bytes, 0);
   memcpy(host.data(), P.ks.data(), sizeof(KsArgs) * P.ks.size());
@@ -447,7 +452,7 @@ int upload_program(fhe_ctx *c, const Program &P, DevProgram &D) {
     // does not change any result, and NTT1's two lists get the same permutation (same
     // segment sizes and primes)
     const bool by_prime = st.kind == Stage::NTT || st.kind == Stage::NTT1;
-    auto fill_map = [by_prime](const std::vector<Seg> &segs, int2 *m) {
+    auto fill_map = [&](const std::vector<Seg> &segs, int2 *m, Limb *lb, bool combine) {
       std::vector<int2> v;
       for (size_t sidx = 0; sidx < segs.size(); sidx++)
         for (int w = 0; w < segs[sidx].n; w++) v.push_back(make_int2((int)sidx, w));
@@ -456,11 +461,26 @@ int upload_program(fhe_ctx *c, const Program &P, DevProgram &D) {
           return segs[a.x].prime + a.y < segs[b.x].prime + b.y;
         });
       std::copy(v.begin(), v.end(), m);
+      for (size_t x = 0; x < v.size(); x++) {
+        const Seg &s = segs[v[x].x];
+        const size_t off = (size_t)v[x].y * c->N;
+        Limb d;
+        d.src = s.src ? s.src + s.src_stride * off : nullptr;
+        d.dst = s.dst + off;
+        d.src2 = s.src2 ? s.src2 + off : nullptr;
+        d.prime = s.prime + v[x].y;
+        d.scale = combine ? c->d_pinv + d.prime : s.scale ? s.scale + v[x].y : c->d_ninv + d.prime;
+        d.galois = s.galois;
+        d.n = s.n;
+        lb[x] = d;
+      }
     };
-    fill_map(st.segs, reinterpret_cast<int2 *>(host.data() + map_off[i]));
+    auto limbs = [&](size_t off) { return reinterpret_cast<Limb *>(host.data() + off); };
+    const bool combine = (by_prime && st.epi == EPI_COMBINE) || (st.kind == Stage::EW && st.ewop == EW_COMBINE);
+    fill_map(st.segs, reinterpret_cast<int2 *>(host.data() + map_off[i]), limbs(limb_off[i]), combine);
     memcpy(host.data() + grp_off[i], st.groups.data(), sizeof(BconvGroup) * st.groups.size());
     memcpy(host.data() + seg2_off[i], st.segs2.data(), sizeof(Seg) * st.segs2.size());
-    fill_map(st.segs2, reinterpret_cast<int2 *>(host.data() + map2_off[i]));
+    fill_map(st.segs2, reinterpret_cast<int2 *>(host.data() + map2_off[i]), limbs(limb2_off[i]), combine);
   }
   if (cudaMalloc(&D.buf, bytes) != cudaSuccess) return fhe_fail(FHE_ENOMEM, "program upload: %zu bytes", bytes);
   if (cudaMemcpy(D.buf, host.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess)
@@ -477,6 +497,7 @@ int upload_program(fhe_ctx *c, const Program &P, DevProgram &D) {
     for (const Seg &x : st.segs) sl.total += x.n;
     sl.dev = reinterpret_cast<const Seg *>(base + seg_off[i]);
     sl.vmap = reinterpret_cast<const int2 *>(base + map_off[i]);
+    sl.limbs = reinterpret_cast<const Limb *>(base + limb_off[i]);
     sl.ksdev = reinterpret_cast<const KsArgs *>(base);
     SegList &sl2 = D.lists2[i];
     memset(&sl2, 0, sizeof sl2);
@@ -484,6 +505,7 @@ int upload_program(fhe_ctx *c, const Program &P, DevProgram &D) {
     for (const Seg &x : st.segs2) sl2.total += x.n;
     sl2.dev = reinterpret_cast<const Seg *>(base + seg2_off[i]);
     sl2.vmap = reinterpret_cast<const int2 *>(base + map2_off[i]);
+    sl2.limbs = reinterpret_cast<const Limb *>(base + limb2_off[i]);
     sl2.ksdev = reinterpret_cast<const KsArgs *>(base);
     BconvArgs &ba = D.bargs[i];
     memset(&ba, 0, sizeof ba);
@@ -491,7 +513,6 @@ int upload_program(fhe_ctx *c, const Program &P, DevProgram &D) {
     ba.lazy = 1;  // every conversion of a program feeds a forward NTT
     ba.dev = reinterpret_cast<const BconvGroup *>(base + grp_off[i]);
   }
-  (void)c;
   return FHE_OK;
 }
 
