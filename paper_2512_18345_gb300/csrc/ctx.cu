@@ -156,6 +156,10 @@ static int build_tables(fhe_ctx *c) {
   CUDA_OR_FAIL(upload(&c->d_tw, tw));
   CUDA_OR_FAIL(upload(&c->d_itw, itw));
   CUDA_OR_FAIL(upload(&c->d_ninv, ninv));
+  for (auto d : {&c->d_lo, &c->d_ilo}) {
+    CUDA_OR_FAIL(cudaMalloc(d, sizeof(uint2) * (size_t)NP * N));
+    CUDA_OR_FAIL(fhe::build_lo_table(d == &c->d_lo ? c->d_tw : c->d_itw, *d, c->logn, NP));
+  }
 
   // ModUp tables per level: pre-factor of each q-limb ((D/q_t)^-1 mod q_t, with and
   // without N^-1) and the BConv table of every digit (rows in ext-limb order).
@@ -252,11 +256,13 @@ static int build_tables(fhe_ctx *c) {
     for (int i = 0; i < level - 1; i++) rs[(size_t)(level - 1) * L + i] = h_pair(h_inv(pr[level - 1] % pr[i], pr[i]), pr[i]);
   CUDA_OR_FAIL(upload(&c->d_rs_qinv, rs));
 
-  c->table_bytes = sizeof(PrimeC) * NP + 2 * sizeof(uint2) * (size_t)NP * N + sizeof(uint2) * (size_t)(4 * L * L + 3 * K + 2 * L) +
+  c->table_bytes = sizeof(PrimeC) * NP + 4 * sizeof(uint2) * (size_t)NP * N + sizeof(uint2) * (size_t)(4 * L * L + 3 * K + 2 * L) +
                    sizeof(uint32_t) * (size_t)L * K;
   c->tabs.ntt.pc = c->d_pc;
   c->tabs.ntt.tw_fwd = c->d_tw;
   c->tabs.ntt.tw_inv = c->d_itw;
+  c->tabs.ntt.lo_fwd = c->d_lo;
+  c->tabs.ntt.lo_inv = c->d_ilo;
   c->tabs.ntt.ninv = c->d_ninv;
   c->tabs.pc = c->d_pc;
   c->tabs.logn = c->logn;
@@ -341,6 +347,8 @@ fhe_ctx::~fhe_ctx() {
   cudaFree(d_pc);
   cudaFree(d_tw);
   cudaFree(d_itw);
+  cudaFree(d_lo);
+  cudaFree(d_ilo);
   cudaFree(d_ninv);
   cudaFree(d_mu_scale);
   cudaFree(d_mu_qhinv);

@@ -24,6 +24,7 @@ struct fhe_ctx {
   // device tables
   fhe::PrimeC *d_pc = nullptr;
   uint2 *d_tw = nullptr, *d_itw = nullptr, *d_ninv = nullptr;
+  uint4 *d_lo = nullptr, *d_ilo = nullptr;  // lo-round twiddles of the block passes in thread order
   uint2 *d_mu_scale = nullptr;  // [L][L]: N^-1 (D/q_t)^-1 mod q_t at level l (row l-1)
   uint2 *d_mu_qhinv = nullptr;  // [L][L]: (D/q_t)^-1 mod q_t
   std::vector<uint32_t *> modup_T;  // [(level-1)*dnum + j]: BConv table, rows in ext-limb order

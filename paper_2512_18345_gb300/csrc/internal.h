@@ -89,6 +89,8 @@ struct TraceScope {
   }
 };
 void note_launch();
+// the block passes' lo-round twiddles in thread order, from the bit-reversed table (legacy stream)
+cudaError_t build_lo_table(const uint2 *tw, uint4 *lo, int logn, int nprimes);
 // the byte-digit table of the tensor-core base conversion (host side)
 // K = kt (48 for at most 8 inputs, 64 for at most 12)
 std::vector<uint16_t> bconv_tc_table(const std::vector<uint32_t> &T, int n_in, const std::vector<uint32_t> &p_out,

@@ -70,8 +70,8 @@ __global__ void __launch_bounds__(kIpIttThreads, 3) k_ip_intt(const __grid_const
 
   // the inverse block pass: lo round (register twiddles), exchange, hi round (staged twiddles)
   {
-    uint2 Lw[15];
-    nb_twiddles<false>(tw, tile, c, tau, Lw);
+    uint2 Lw[16];
+    load_lo_twiddles<16>(tb.lo_inv, prime, tile, tid, Lw);
     nb_round<false>(x, [&](int m, int j) { return Lw[(1 << m) - 1 + j]; }, q);
   }
 #pragma unroll

@@ -35,6 +35,8 @@ struct NttTables {
   const PrimeC *pc;
   const uint2 *tw_fwd;  // [primes][N] (w, floor(w 2^32 / q)), w = psi^brv(index)
   const uint2 *tw_inv;  // [primes][N] with psi^-1
+  const uint4 *lo_fwd;  // [primes][N / 2] the block passes' lo-round twiddles in thread order (ntt_blk.cuh)
+  const uint4 *lo_inv;
   const uint2 *ninv;    // [primes] N^-1
 };
 
@@ -95,6 +97,19 @@ __host__ __device__ constexpr int ntt_twiddle_smem(bool column, int S) { return 
 // thread's earlier shared-memory accesses to the cluster, wait acquires the others'.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// four consecutive words <-> registers
+__device__ __forceinline__ void ld4(const uint32_t *p, uint32_t *v) {
+  const uint4 w = *reinterpret_cast<const uint4 *>(p);
+  v[0] = w.x, v[1] = w.y, v[2] = w.z, v[3] = w.w;
+}
+__device__ __forceinline__ void ldg4(const uint32_t *p, uint32_t *v) {
+  const uint4 w = __ldg(reinterpret_cast<const uint4 *>(p));
+  v[0] = w.x, v[1] = w.y, v[2] = w.z, v[3] = w.w;
+}
+__device__ __forceinline__ void st4(uint32_t *p, const uint32_t *v) {
+  *reinterpret_cast<uint4 *>(p) = make_uint4(v[0], v[1], v[2], v[3]);
+}
 
 // Where a pass reads its round-0 elements and writes its results.
 enum : int { SRC_GLOBAL = 0, SRC_CLUSTER = 1 };

@@ -33,7 +33,7 @@
 // pass's runs psi^brv(2^(8 + m) + (16 tile << m) + i), i < 16 2^m, at 16 (2^m - 1).
 #pragma once
 #include "async.cuh"
-#include "ntt.cuh"
+#include "ntt_blk.cuh"
 
 namespace fhe {
 
@@ -54,11 +54,6 @@ struct NbUnit {
 };
 
 __device__ __forceinline__ uint32_t nb_col_addr(int k, int c) { return (uint32_t)(k * 16 + ((k >> 4) << 4) + c); }
-__device__ __forceinline__ uint32_t nb_blk_addr(int c, int k) {
-  const int r = k >> 4;
-  return (uint32_t)(c * 272 + r * 16 + ((((k >> 2) & 3) ^ ((r >> 1) & 3)) << 2) + (k & 3));
-}
-
 // unit u of a launch -> (limb v, tile): column pass limb-major; block pass in runs of
 // kNbRun limbs per tile (the last run may be shorter)
 template <bool COLUMN>
@@ -85,15 +80,12 @@ __device__ __forceinline__ void cp_async_arrive_noinc(uint64_t *bar) {
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ void nb_consumer_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kNbConsumers) : "memory"); }
 
-// The 15 lo-round twiddles of a consumer thread, entry (1 << m) - 1 + j for register bit
-// m = 3 - bit and j = e >> (bit + 1).
-template <bool COLUMN>
-__device__ __forceinline__ void nb_twiddles(const uint2 *tw, int tile, int c, int tau, uint2 (&Lw)[15]) {
-  constexpr int S0 = 8;  // LOGN - 8 at N = 2^16
+// The 15 lo-round twiddles of a consumer thread of the column pass, entry (1 << m) - 1 + j
+// for register bit m = 3 - bit and j = e >> (bit + 1) (the block pass: load_lo_twiddles).
+__device__ __forceinline__ void nb_col_twiddles(const uint2 *tw, int tau, uint2 (&Lw)[16]) {
 #pragma unroll
   for (int m = 0; m < 4; m++) {
-    const uint2 *from = COLUMN ? tw + (16 << m) + (tau << m)
-                               : tw + (1 << (S0 + 4 + m)) + ((tile * 16 + c) << (4 + m)) + (tau << m);
+    const uint2 *from = tw + (16 << m) + (tau << m);
     if (m == 0) {
       Lw[0] = __ldg(from);
     } else {
@@ -102,33 +94,6 @@ __device__ __forceinline__ void nb_twiddles(const uint2 *tw, int tile, int c, in
         const uint4 w = __ldg(reinterpret_cast<const uint4 *>(from) + k2);
         Lw[(1 << m) - 1 + 2 * k2] = make_uint2(w.x, w.y);
         Lw[(1 << m) - 1 + 2 * k2 + 1] = make_uint2(w.z, w.w);
-      }
-    }
-  }
-}
-
-// one radix-16 round (4 butterfly stages on the 16 register values); tw(m, j) is the
-// twiddle of register bit 3 - m for butterfly group j
-template <bool FWD, class TW>
-__device__ __forceinline__ void nb_round(uint32_t (&x)[16], TW tw, uint32_t q) {
-#pragma unroll
-  for (int i = 0; i < 4; i++) {
-    const int bit = FWD ? 3 - i : i;
-    const int m = 3 - bit;
-#pragma unroll
-    for (int e = 0; e < 16; e++) {
-      if (e & (1 << bit)) continue;
-      const int e2 = e | (1 << bit);
-      const uint2 w = tw(m, e >> (bit + 1));
-      if (FWD) {
-        const uint32_t t = red2(shoup_lazy(x[e2], w.x, w.y, q), q);
-        const uint32_t u = red2(x[e], q);
-        x[e] = u + t;
-        x[e2] = u - t + q;
-      } else {
-        const uint32_t u = red2(x[e], q), v = red2(x[e2], q);
-        x[e] = u + v;
-        x[e2] = shoup_lazy(u - v + q, w.x, w.y, q);
       }
     }
   }
@@ -233,7 +198,7 @@ __global__ void __launch_bounds__(kNbThreads, 3)
     c = tid >> 4;
     tau = tid & 15;
   }
-  uint2 Lw[15];
+  uint2 Lw[16];
   int cur_prime = -1, cur_tile = -1;
   bool ok = true;
   int k = 0;
@@ -246,7 +211,8 @@ __global__ void __launch_bounds__(kNbThreads, 3)
     const PrimeC P = tb.pc[d.prime];
     const uint32_t q = P.q;
     if (d.prime != cur_prime || (!COLUMN && d.tile != cur_tile)) {
-      nb_twiddles<COLUMN>((FWD ? tb.tw_fwd : tb.tw_inv) + (size_t)d.prime * N, d.tile, c, tau, Lw);
+      if (COLUMN) nb_col_twiddles((FWD ? tb.tw_fwd : tb.tw_inv) + (size_t)d.prime * N, tau, Lw);
+      else load_lo_twiddles<16>(FWD ? tb.lo_fwd : tb.lo_inv, d.prime, d.tile, tid, Lw);
       cur_prime = d.prime;
       cur_tile = d.tile;
     }
