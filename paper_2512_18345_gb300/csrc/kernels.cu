@@ -9,6 +9,7 @@
 #include "internal.h"
 #include "ntt.cuh"
 #include "ntt_blk.cuh"
+#include "ntt_col.cuh"
 #include "ntt_bulk.cuh"
 #include "ip_intt.cuh"
 #include "ip_hoisted.cuh"
@@ -80,6 +81,17 @@ static cudaError_t ntt_blk_go(const DevTables &t, const SegList &sl, cudaStream_
   return cudaGetLastError();
 }
 
+// Column pass with warp-private twiddles (ntt_col.cuh).
+template <int LOGN, bool FWD, int PRO, int EPI>
+static cudaError_t ntt_col_go(const DevTables &t, const SegList &sl, cudaStream_t s) {
+  const unsigned grid = (unsigned)(sl.total * ((1 << LOGN) / kTile));
+  if (grid == 0) return cudaSuccess;
+  TraceScope ts(t, ntt_name<LOGN, true, FWD, PRO, EPI, false>(), s);
+  k_ntt_col<LOGN, FWD, PRO, EPI><<<grid, kNttThreads, 0, s>>>(sl, t.ntt);
+  g_launches++;
+  return cudaGetLastError();
+}
+
 cudaError_t build_lo_table(const uint2 *tw, uint4 *lo, int logn, int nprimes) {
   const size_t n = (size_t)nprimes << (logn - 1);
   k_lo_table<<<(unsigned)((n + 255) / 256), 256>>>(tw, lo, logn, nprimes);
@@ -130,7 +142,7 @@ static cudaError_t ntt_dispatch(const DevTables &t, bool column, bool fwd, int p
   }
 #define NTT_CASE(COL, FWDV, P, E)                                                              \
   if (column == COL && fwd == FWDV && pro == P && epi == E) {                                  \
-    if constexpr (COL) return ntt_go<LOGN, COL, FWDV, P, E, false>(t, sl, s);                  \
+    if constexpr (COL) return ntt_col_go<LOGN, FWDV, P, E>(t, sl, s);                          \
     else if (otf) return ntt_go<LOGN, COL, FWDV, P, E, true>(t, sl, s);                        \
     else return ntt_blk_go<LOGN, FWDV, P, E>(t, sl, s);                                        \
   }
