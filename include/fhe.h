@@ -133,10 +133,12 @@ FHE_API int fhe_selftest_wait_timeout(fhe_ctx *ctx, fhe_stream stream);
 FHE_API int fhe_ctx_set_memory_limit(fhe_ctx *ctx, size_t bytes);
 /* Fuse stage epilogues (1, default) or run the plain per-kernel pipeline (0).  Same bits. */
 FHE_API int fhe_ctx_set_fused(fhe_ctx *ctx, int fused);
-/* Complementary pipelining (Section IV-B) in the fused pipeline: with `on`
- * (the default) the inner product of the ciphertext limbs runs on an
- * auxiliary branch beside ModDown's special-limb chain; without it, one launch
- * covers all limbs.  Results are identical either way; fhe_autotune sets it. */
+/* Complementary pipelining (Section IV-B) in batched plans: with `on` (the
+ * default) the inner product of the ciphertext limbs runs on an auxiliary
+ * branch beside ModDown's special-limb chain; without it, one launch covers all
+ * limbs.  Results are identical either way; fhe_autotune sets it.  Single calls
+ * run their stages on the caller's stream alone, each launched as a dependent of
+ * the one before it. */
 FHE_API int fhe_ctx_set_pipelining(fhe_ctx *ctx, int on);
 /* NTT kernel variants (flags; 0 = the two-pass kernels, the default):
  *   FHE_NTT_OTF: the block passes (the last eight stages, the paper's second

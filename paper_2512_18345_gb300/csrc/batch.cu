@@ -174,7 +174,7 @@ extern "C" int fhe_batch_plan(fhe_ctx *c, const fhe_ks_item *items, int n, int f
     }
     // copies of identity rotations have level-dependent sizes: handle them as one-item groups
     Program P;
-    if (rc == FHE_OK) rc = build_program(c, its, true, P);
+    if (rc == FHE_OK) rc = build_program(c, its, true, c->comp_pipe != 0, P);
     DevProgram D;
     if (rc == FHE_OK) rc = upload_program(c, P, D);
     p->progs.push_back(P);

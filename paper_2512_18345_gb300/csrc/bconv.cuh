@@ -83,7 +83,7 @@ __device__ __forceinline__ void bconv_out4(const uint32_t (&y)[NIN][4], const ui
   }
 }
 
-template <int NIN>
+template <int NIN, bool DEP>
 __global__ void __launch_bounds__(kBconvThreads) k_bconv(const __grid_constant__ BconvArgs a, const PrimeC *pc,
                                                          int logn) {
   __shared__ uint32_t sT[kBconvOutChunk * NIN];
@@ -102,13 +102,14 @@ __global__ void __launch_bounds__(kBconvThreads) k_bconv(const __grid_constant__
     sM[threadIdx.x] = g.omap[o0 + threadIdx.x];
     sP[threadIdx.x] = pc[sM[threadIdx.x].y];
   }
+  if (DEP) dep_wait();
   __syncthreads();
   const size_t N = (size_t)1 << logn;
   const size_t n = ((size_t)blockIdx.x * kBconvThreads + threadIdx.x) * 4;
   uint32_t y[NIN][4];
 #pragma unroll
   for (int k = 0; k < NIN; k++) {
-    const uint4 v = k < n_in ? __ldg(reinterpret_cast<const uint4 *>(g.in + k * N + n)) : make_uint4(0, 0, 0, 0);
+    const uint4 v = k < n_in ? ld_in4<DEP>(g.in + k * N + n) : make_uint4(0, 0, 0, 0);
     y[k][0] = v.x;
     y[k][1] = v.y;
     y[k][2] = v.z;

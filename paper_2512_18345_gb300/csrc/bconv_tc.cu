@@ -122,7 +122,7 @@ __device__ __forceinline__ void tc_reduce_outputs(uint32_t tbase, int o_beg, int
 // input pairs into A, thread 0 issues the MMAs and commits to the mbarrier
 // (phase = tile parity), all wait (bounded), then each warp reads its lane
 // quarter for half of the outputs and writes the reduced results.
-template <int KT>
+template <int KT, bool DEP>
 __global__ void __launch_bounds__(kTcThreads, 4) k_bconv_tc(const __grid_constant__ BconvArgs a, const PrimeC *pc,
                                                          int logn, unsigned int *status, int npad_max,
                                                          int tiles_per_group) {
@@ -180,11 +180,12 @@ __global__ void __launch_bounds__(kTcThreads, 4) k_bconv_tc(const __grid_constan
 #pragma unroll
     for (int h = 0; h < 2 * kNch; h++) {
       const int j = 2 * (kc0 + 2 * (h >> 1)) + (h & 1);
-      y[h] = j < nin ? __ldg(g->in + (size_t)j * N + m0 + r) : 0u;
+      y[h] = j < nin ? ld_in<DEP>(g->in + (size_t)j * N + m0 + r) : 0u;
     }
   };
 #pragma unroll
   for (int h = 0; h < 2 * kNch; h++) y[h] = 0u;
+  if (DEP) dep_wait();
   bool prefetched = false;  // y holds the current tile's inputs
   bool big_primes = true;   // the current group's output primes all exceed 2^30
   for (int tile = t0; tile < t1 && ok; tile++) {
@@ -483,8 +484,11 @@ static cudaError_t bconv_tc_go(const DevTables &t, const BconvArgs &a, int max_o
   int smem = std::max(need, 233472 / (per_sm + 1) + 1024);  // 228 KB of shared memory per SM
   if (smem > 232448) smem = 232448;
   static PerDeviceOnce configured;
-  const cudaError_t ce = configured.run(
-      [] { return cudaFuncSetAttribute(k_bconv_tc<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448); });
+  const cudaError_t ce = configured.run([] {
+    const cudaError_t e = cudaFuncSetAttribute(k_bconv_tc<KT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+    return e != cudaSuccess ? e
+                            : cudaFuncSetAttribute(k_bconv_tc<KT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+  });
   if (ce != cudaSuccess) return ce;
   int sms = 0, dev = 0;
   cudaGetDevice(&dev);
@@ -506,7 +510,9 @@ static cudaError_t bconv_tc_go(const DevTables &t, const BconvArgs &a, int max_o
     k_bconv_tc_pipe<KT><<<grid2, kTcThreads, smem2, s>>>(a, t.pc, t.logn, t.status, npad, tiles_per_group);
   } else {
     const int grid = std::min(total, std::max(1, sms * per_sm));
-    k_bconv_tc<KT><<<grid, kTcThreads, smem, s>>>(a, t.pc, t.logn, t.status, npad, tiles_per_group);
+    const cudaError_t le = launch_dep(t, t.dep ? k_bconv_tc<KT, true> : k_bconv_tc<KT, false>, grid, kTcThreads, smem, s, a, t.pc, t.logn, t.status, npad,
+                                      tiles_per_group);
+    if (le != cudaSuccess) return le;
   }
   note_launch();
   return cudaGetLastError();

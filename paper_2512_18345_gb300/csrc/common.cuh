@@ -22,6 +22,37 @@ struct PrimeC {
   uint32_t pad1;
 };
 
+// ---------------------------------------------------------------- dependent launches
+// A stage kernel of a single-call program may start before the one it follows has ended
+// (programmatic dependent launch): it stages its constants, then dep_wait() holds it until the
+// previous kernel has completed and its writes are visible, and lets the next kernel start its
+// own prologue (one kernel ahead at most).  What an earlier kernel of the program wrote is read only after dep_wait, with ld_dep (L2;
+// ordered after the wait): ld.global.nc may be moved above it and may hit a line that L1 kept
+// from before the write.  Only the DEP forms of the kernels wait: the wait also holds back the
+// loads behind a CTA's constants, which cost the 8-rotation graph step 512 -> 552 us when every
+// launch had it.
+__device__ __forceinline__ void dep_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t ld_dep(const uint32_t *p) {
+  uint32_t v;
+  asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint4 ld_dep4(const uint32_t *p) {
+  uint4 v;
+  asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
+
+template <bool DEP>
+__device__ __forceinline__ uint32_t ld_in(const uint32_t *p) { return DEP ? ld_dep(p) : __ldg(p); }
+template <bool DEP>
+__device__ __forceinline__ uint4 ld_in4(const uint32_t *p) {
+  return DEP ? ld_dep4(p) : __ldg(reinterpret_cast<const uint4 *>(p));
+}
+
 // ---------------------------------------------------------------- arithmetic
 // [0, 2q) -> [0, q): if x < q then x - q wraps above x and min keeps x.
 __device__ __forceinline__ uint32_t red2(uint32_t x, uint32_t q) { return min(x, x - q); }

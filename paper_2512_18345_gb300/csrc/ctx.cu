@@ -268,6 +268,7 @@ static int build_tables(fhe_ctx *c) {
   c->tabs.logn = c->logn;
   c->tabs.tracer = nullptr;
   c->tabs.ip_ctas_per_sm = 2;
+  c->tabs.dep = 0;
   c->tabs.ntt_otf = 0;
   c->tabs.ntt_single = 0;
   c->tabs.ntt_stream = 0;

@@ -169,8 +169,8 @@ __global__ void __launch_bounds__(kEwThreads) k_ip(const __grid_constant__ SegLi
 // loads one unit ahead.
 constexpr int kIpChunk = 1024;  // coefficients per unit
 constexpr int kIpThreads = 256;
-constexpr int kIpEpt = kIpChunk / kIpThreads;  // coefficients per thread and unit (2 or 4)
-static_assert(kIpEpt == 2 || kIpEpt == 4, "inner product: 2 or 4 coefficients per thread");
+constexpr int kIpEpt = kIpChunk / kIpThreads;  // coefficients per thread and unit
+static_assert(kIpEpt == 4, "inner product: one 16-byte access per row and thread");
 
 // E consecutive words <-> registers (one 8- or 16-byte access)
 template <int E>
@@ -180,16 +180,6 @@ __device__ __forceinline__ void ld_words(const uint32_t *p, uint32_t (&v)[E]) {
     v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
   } else {
     const uint2 t = *reinterpret_cast<const uint2 *>(p);
-    v[0] = t.x, v[1] = t.y;
-  }
-}
-template <int E>
-__device__ __forceinline__ void ldg_words(const uint32_t *p, uint32_t (&v)[E]) {
-  if constexpr (E == 4) {
-    const uint4 t = __ldg(reinterpret_cast<const uint4 *>(p));
-    v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
-  } else {
-    const uint2 t = __ldg(reinterpret_cast<const uint2 *>(p));
     v[0] = t.x, v[1] = t.y;
   }
 }
@@ -216,7 +206,7 @@ struct IpUnit {            // one unit, as the consumers need it
 // GEXT (hoisted rotations: the ModUp digits themselves are read through the
 // automorphism): only the key chunks stream through the stages; every digit's values
 // are gathered with plain loads one unit ahead (the shared digits stay in L2).
-template <bool GOWN, bool GEXT>
+template <bool GOWN, bool GEXT, bool DEP>
 __global__ void __launch_bounds__(kIpThreads + 32, 2) k_ip_bulk(const __grid_constant__ SegList sl, const PrimeC *pc,
                                                            int logn, unsigned int *status, int beta_max, int stages) {
   extern __shared__ __align__(128) uint8_t smem[];
@@ -237,8 +227,9 @@ __global__ void __launch_bounds__(kIpThreads + 32, 2) k_ip_bulk(const __grid_con
   // keys are read exactly once: evict them first, so that ModUp outputs (and the digits shared
   // by hoisted rotations) stay in L2
   const uint64_t key_policy = l2_evict_first_policy();
-  // the producer: describe unit u and stream its operands into stage st
-  auto issue = [&](int u, int st) {
+  // the producer: describe unit u and stream its operands into stage st; the first unit's keys,
+  // which no kernel of the program writes, are on their way before dep_wait
+  auto issue = [&](int u, int st, bool first) {  // (first: DEP only)
     int within;
     const Seg &sg = seg_at(sl, seg_find(sl, u / chunks, within));
     const KsArgs &ks = item_ks(sl, sg);
@@ -271,15 +262,24 @@ __global__ void __launch_bounds__(kIpThreads + 32, 2) k_ip_bulk(const __grid_con
     const uint32_t copies = GEXT ? 2u * (uint32_t)ks.beta : 3u * (uint32_t)ks.beta - (d.gjd >= 0 ? 1u : 0u);
     mbar_arrive_expect_tx(&bar[st], copies * kIpChunk * 4u);
     uint32_t *dst = buf + (size_t)st * stage_words;
+    auto digits = [&] {
+      for (int jd = 0; jd < ks.beta; jd++)
+        if (!GEXT && jd != d.gjd) {
+          const bool own = t < ks.level && t >= jd * ks.alpha && t < (jd + 1) * ks.alpha;
+          const uint32_t *e = own ? ks.own + (size_t)t * N : ks.ext + ((size_t)jd * ks.n_ext + t) * N;
+          bulk_g2s(dst + (size_t)(RPD * jd) * kIpChunk, e + c0, kIpChunk * 4u, &bar[st]);
+        }
+    };
+    if (!first) digits();
     for (int jd = 0; jd < ks.beta; jd++) {
-      if (!GEXT && jd != d.gjd) {
-        const bool own = t < ks.level && t >= jd * ks.alpha && t < (jd + 1) * ks.alpha;
-        const uint32_t *e = own ? ks.own + (size_t)t * N : ks.ext + ((size_t)jd * ks.n_ext + t) * N;
-        bulk_g2s(dst + (size_t)(RPD * jd) * kIpChunk, e + c0, kIpChunk * 4u, &bar[st]);
-      }
       const uint32_t *kp = ks.key + jd * kstride + (size_t)row * N + c0;
       bulk_g2s_hint(dst + (size_t)(RPD * jd + KR) * kIpChunk, kp, kIpChunk * 4u, &bar[st], key_policy);
       bulk_g2s_hint(dst + (size_t)(RPD * jd + KR + 1) * kIpChunk, kp + half, kIpChunk * 4u, &bar[st], key_policy);
+    }
+    if (first) {
+      dep_wait();
+      asm volatile("fence.proxy.async;" ::: "memory");  // bulk copies read what earlier kernels wrote
+      digits();
     }
   };
   // Warp specialisation: warps 0..7 reduce units, warp 8 (one lane) produces them.  The
@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(kIpThreads + 32, 2) k_ip_bulk(const __grid_con
       // the consumers released this stage's previous unit (bounded: if they gave up, so do we)
       if (k >= stages && !mbar_wait_bounded(&ebar[st], (uint32_t)(k / stages - 1) & 1u)) break;
       fence_proxy_async_smem();
-      issue(u, st);
+      issue(u, st, DEP && k == 0);
     }
     return;
   }
@@ -319,8 +319,9 @@ __global__ void __launch_bounds__(kIpThreads + 32, 2) k_ip_bulk(const __grid_con
   auto pass = [&](const IpUnit &d, uint32_t (&p0)[E], uint32_t (&p1)[E]) {
     const uint32_t j = d.j0 + tid * E;
     if (d.galois_add == 1u) {
-      ldg_words<E>(d.add0 + j, p0);
-      if (d.add1) ldg_words<E>(d.add0 + d.add1_off + j, p1);
+      // (HMult's tensor: written by this program's first kernel)
+      ld_in4<DEP>(d.add0 + j, p0);
+      if (d.add1) ld_in4<DEP>(d.add0 + d.add1_off + j, p1);
     } else {
 #pragma unroll
       for (int e = 0; e < E; e++) p0[e] = __ldg(d.add0 + galois_src(j + e, d.galois_add, logn));
@@ -337,6 +338,7 @@ __global__ void __launch_bounds__(kIpThreads + 32, 2) k_ip_bulk(const __grid_con
         for (int e = 0; e < E; e++) v[jd][e] = __ldg(d.esrc[jd] + galois_src(j + e, d.egal[jd], logn));
   };
   // every consumer thread waits on the barriers itself (bounded; a warp gives up as a whole)
+  if (DEP) dep_wait();
   uint32_t gnext[E] = {}, pnext0[E] = {}, pnext1[E] = {}, xnext[XD][E] = {};
   bool ok = true;
   if ((int)blockIdx.x < total) {

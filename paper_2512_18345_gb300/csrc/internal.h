@@ -74,6 +74,7 @@ struct DevTables {
   int ip_staged;           // hoisted inner product: digits' permuted blocks staged (ip_hoisted.cuh)
   int ip_staged_ctas;      // resident CTAs per SM of that kernel (1 or 2)
   int ip_staged_depth;     // its stages per warp (2..4; 0: 2)
+  int dep;                 // the next launch is a dependent one (set stage by stage by run_program_inline)
   int tc_k;                // K of the context's tensor-core BConv tables (48 or 64; 0: none)
 };
 
@@ -89,6 +90,24 @@ struct TraceScope {
   }
 };
 void note_launch();
+
+// Launch a kernel that begins with dep_wait (common.cuh); with t.dep it may start while the
+// kernel before it on the stream is still running.
+template <class... P, class... A>
+cudaError_t launch_dep(const DevTables &t, void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s,
+                       const A &...args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = t.dep ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
 // the block passes' lo-round twiddles in thread order, from the bit-reversed table (legacy stream)
 cudaError_t build_lo_table(const uint2 *tw, uint4 *lo, int logn, int nprimes);
 // the byte-digit table of the tensor-core base conversion (host side)

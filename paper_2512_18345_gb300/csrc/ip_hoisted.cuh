@@ -115,7 +115,7 @@ __device__ __forceinline__ void ih_limb(const SegList &sl, const PrimeC *pc, int
 // the limbs listed by extended-basis index (every rotation of a hoisted set beside the others
 // at the same limb), the digits in use at any time are a few limbs', which stay in L2 while
 // every rotation reads them, and a warp's limb (and its arguments) change once per run.
-template <int D>
+template <int D, bool DEP>
 __global__ void __launch_bounds__(kIhMaxWarps * 32, 1)
     k_ip_hoisted(const __grid_constant__ SegList sl, const PrimeC *pc, int logn, int beta_max) {
   extern __shared__ __align__(128) uint8_t smem[];
@@ -175,6 +175,7 @@ __global__ void __launch_bounds__(kIhMaxWarps * 32, 1)
     cp_async_commit();  // (an empty group past the end keeps the group count uniform)
   };
 
+  if (DEP) dep_wait();
 #pragma unroll
   for (int k = 0; k < D - 1; k++) stage(k);
   for (int k = 0; k < n; k++) {

@@ -76,9 +76,8 @@ static cudaError_t ntt_blk_go(const DevTables &t, const SegList &sl, cudaStream_
   const unsigned grid = (unsigned)(sl.total * ((1 << LOGN) / kTile));
   if (grid == 0) return cudaSuccess;
   TraceScope ts(t, ntt_name<LOGN, false, FWD, PRO, EPI, false>(), s);
-  k_ntt_blk<LOGN, FWD, PRO, EPI><<<grid, kNttThreads, 0, s>>>(sl, t.ntt);
   g_launches++;
-  return cudaGetLastError();
+  return launch_dep(t, t.dep ? k_ntt_blk<LOGN, FWD, PRO, EPI, true> : k_ntt_blk<LOGN, FWD, PRO, EPI, false>, grid, kNttThreads, 0, s, sl, t.ntt);
 }
 
 // Column pass with warp-private twiddles (ntt_col.cuh).
@@ -87,9 +86,8 @@ static cudaError_t ntt_col_go(const DevTables &t, const SegList &sl, cudaStream_
   const unsigned grid = (unsigned)(sl.total * ((1 << LOGN) / kTile));
   if (grid == 0) return cudaSuccess;
   TraceScope ts(t, ntt_name<LOGN, true, FWD, PRO, EPI, false>(), s);
-  k_ntt_col<LOGN, FWD, PRO, EPI><<<grid, kNttThreads, 0, s>>>(sl, t.ntt);
   g_launches++;
-  return cudaGetLastError();
+  return launch_dep(t, t.dep ? k_ntt_col<LOGN, FWD, PRO, EPI, true> : k_ntt_col<LOGN, FWD, PRO, EPI, false>, grid, kNttThreads, 0, s, sl, t.ntt);
 }
 
 cudaError_t build_lo_table(const uint2 *tw, uint4 *lo, int logn, int nprimes) {
@@ -299,18 +297,44 @@ cudaError_t launch_bconv(const DevTables &t, const BconvArgs &a, int max_in, int
   const dim3 grid((unsigned)((1u << t.logn) / (4 * kBconvThreads)), (unsigned)((max_out + kBconvOutChunk - 1) / kBconvOutChunk),
                   (unsigned)a.ngroups);
   TraceScope ts(t, "bconv", s);
+  g_launches++;
   switch (max_in) {
 #define BC(n) \
-  case n: k_bconv<n><<<grid, kBconvThreads, 0, s>>>(a, t.pc, t.logn); break;
+  case n: return launch_dep(t, t.dep ? k_bconv<n, true> : k_bconv<n, false>, grid, kBconvThreads, 0, s, a, t.pc, t.logn);
     BC(1) BC(2) BC(3) BC(4) BC(5) BC(6) BC(7) BC(8)
 #undef BC
     default:
-      if (max_in <= 12) k_bconv<12><<<grid, kBconvThreads, 0, s>>>(a, t.pc, t.logn);
-      else if (max_in <= 16) k_bconv<16><<<grid, kBconvThreads, 0, s>>>(a, t.pc, t.logn);
-      else return cudaErrorInvalidValue;
+      if (max_in <= 12) return launch_dep(t, t.dep ? k_bconv<12, true> : k_bconv<12, false>, grid, kBconvThreads, 0, s, a, t.pc, t.logn);
+      if (max_in <= 16) return launch_dep(t, t.dep ? k_bconv<16, true> : k_bconv<16, false>, grid, kBconvThreads, 0, s, a, t.pc, t.logn);
+      return cudaErrorInvalidValue;
   }
-  g_launches++;
-  return cudaGetLastError();
+}
+
+template <int D>
+static cudaError_t ih_go(const DevTables &t, unsigned grid, unsigned block, int smem, cudaStream_t s, const SegList &sl,
+                         int beta_max) {
+  static PerDeviceOnce configured;
+  const cudaError_t e = configured.run([] {
+    constexpr int kMax = 227 * 1024;
+    const cudaError_t e0 = cudaFuncSetAttribute(k_ip_hoisted<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
+    return e0 != cudaSuccess ? e0
+                             : cudaFuncSetAttribute(k_ip_hoisted<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
+  });
+  if (e != cudaSuccess) return e;
+  return launch_dep(t, t.dep ? k_ip_hoisted<D, true> : k_ip_hoisted<D, false>, grid, block, smem, s, sl, t.pc, t.logn,
+                    beta_max);
+}
+
+template <bool GOWN, bool GEXT, bool DEP>
+static cudaError_t ip_bulk_go(const DevTables &t, unsigned grid, int smem, cudaStream_t s, const SegList &sl, int beta_max,
+                              int stages) {
+  static PerDeviceOnce configured;
+  const cudaError_t e = configured.run([] {
+    return cudaFuncSetAttribute(k_ip_bulk<GOWN, GEXT, DEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024);
+  });
+  if (e != cudaSuccess) return e;
+  return launch_dep(t, k_ip_bulk<GOWN, GEXT, DEP>, grid, kIpThreads + 32, smem, s, sl, t.pc, t.logn, t.status, beta_max,
+                    stages);
 }
 
 cudaError_t launch_ip(const DevTables &t, const SegList &sl, bool gather_own, bool gather_ext, bool add_c1,
@@ -328,25 +352,18 @@ cudaError_t launch_ip(const DevTables &t, const SegList &sl, bool gather_own, bo
     int D = t.ip_staged_depth >= 2 && t.ip_staged_depth <= 4 ? t.ip_staged_depth : 2;
     while (D > 2 && budget / (D * ws) < 1) D--;
     const int warps = std::max(1, std::min(kIhMaxWarps / ctas, budget / (D * ws)));
-    static PerDeviceOnce configured[3];
-    const cudaError_t e = configured[D - 2].run([D] {
-      constexpr int kMax = 227 * 1024;
-      return D == 2   ? cudaFuncSetAttribute(k_ip_hoisted<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax)
-             : D == 3 ? cudaFuncSetAttribute(k_ip_hoisted<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax)
-                      : cudaFuncSetAttribute(k_ip_hoisted<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
-    });
-    if (e != cudaSuccess) return e;
     int sms = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int wunits = sl.total * ((1 << t.logn) / kIhUnit);
     const unsigned grid = (unsigned)std::min((wunits + warps - 1) / warps, ctas * sms);
     const int smem = warps * D * ws;
-    if (D == 2) k_ip_hoisted<2><<<grid, warps * 32, smem, s>>>(sl, t.pc, t.logn, beta_max);
-    else if (D == 3) k_ip_hoisted<3><<<grid, warps * 32, smem, s>>>(sl, t.pc, t.logn, beta_max);
-    else k_ip_hoisted<4><<<grid, warps * 32, smem, s>>>(sl, t.pc, t.logn, beta_max);
+    cudaError_t le;
+    if (D == 2) le = ih_go<2>(t, grid, warps * 32, smem, s, sl, beta_max);
+    else if (D == 3) le = ih_go<3>(t, grid, warps * 32, smem, s, sl, beta_max);
+    else le = ih_go<4>(t, grid, warps * 32, smem, s, sl, beta_max);
     g_launches++;
-    return cudaGetLastError();
+    return le;
   }
   if (beta_max >= 1 && beta_max <= 4 && (1 << t.logn) % kIpChunk == 0) {
     // streaming kernel, one or two CTAs per SM.  Two stages per CTA where each stage holds
@@ -359,31 +376,19 @@ cudaError_t launch_ip(const DevTables &t, const SegList &sl, bool gather_own, bo
     const int per_stage = stage_bytes + 24 + (int)sizeof(IpUnit);  // data, three mbarriers, descriptor
     const int stages = std::min(ge ? 4 : 2, (113 * 1024 - 256) / per_stage);
     const int smem = stages * per_stage;
-    static PerDeviceOnce configured[4];
-    const int variant = (go ? 1 : 0) + (ge ? 2 : 0);
-    const cudaError_t e = configured[variant].run([variant] {
-      constexpr int kMax = 113 * 1024;
-      switch (variant) {
-        case 0: return cudaFuncSetAttribute(k_ip_bulk<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
-        case 1: return cudaFuncSetAttribute(k_ip_bulk<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
-        case 2: return cudaFuncSetAttribute(k_ip_bulk<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
-        default: return cudaFuncSetAttribute(k_ip_bulk<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
-      }
-    });
-    if (e != cudaSuccess) return e;
     int sms = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int units = sl.total * ((1 << t.logn) / kIpChunk);
     const unsigned grid = (unsigned)std::min(units, std::max(1, std::min(2, t.ip_ctas_per_sm)) * sms);
-    switch (variant) {
-      case 0: k_ip_bulk<false, false><<<grid, kIpThreads + 32, smem, s>>>(sl, t.pc, t.logn, t.status, beta_max, stages); break;
-      case 1: k_ip_bulk<true, false><<<grid, kIpThreads + 32, smem, s>>>(sl, t.pc, t.logn, t.status, beta_max, stages); break;
-      case 2: k_ip_bulk<false, true><<<grid, kIpThreads + 32, smem, s>>>(sl, t.pc, t.logn, t.status, beta_max, stages); break;
-      default: k_ip_bulk<true, true><<<grid, kIpThreads + 32, smem, s>>>(sl, t.pc, t.logn, t.status, beta_max, stages); break;
-    }
     g_launches++;
-    return cudaGetLastError();
+    if (go && ge) return ip_bulk_go<true, true, false>(t, grid, smem, s, sl, beta_max, stages);
+    if (ge) return ip_bulk_go<false, true, false>(t, grid, smem, s, sl, beta_max, stages);
+    if (go)
+      return t.dep ? ip_bulk_go<true, false, true>(t, grid, smem, s, sl, beta_max, stages)
+                   : ip_bulk_go<true, false, false>(t, grid, smem, s, sl, beta_max, stages);
+    return t.dep ? ip_bulk_go<false, false, true>(t, grid, smem, s, sl, beta_max, stages)
+                 : ip_bulk_go<false, false, false>(t, grid, smem, s, sl, beta_max, stages);
   }
   const unsigned per_limb = (unsigned)((1u << t.logn) / (4 * kEwThreads));
   const unsigned grid = (unsigned)sl.total * per_limb;

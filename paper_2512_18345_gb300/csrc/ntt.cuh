@@ -103,8 +103,9 @@ __device__ __forceinline__ void ld4(const uint32_t *p, uint32_t *v) {
   const uint4 w = *reinterpret_cast<const uint4 *>(p);
   v[0] = w.x, v[1] = w.y, v[2] = w.z, v[3] = w.w;
 }
-__device__ __forceinline__ void ldg4(const uint32_t *p, uint32_t *v) {
-  const uint4 w = __ldg(reinterpret_cast<const uint4 *>(p));
+template <bool DEP>
+__device__ __forceinline__ void ld_in4(const uint32_t *p, uint32_t *v) {
+  const uint4 w = ld_in4<DEP>(p);
   v[0] = w.x, v[1] = w.y, v[2] = w.z, v[3] = w.w;
 }
 __device__ __forceinline__ void st4(uint32_t *p, const uint32_t *v) {

@@ -130,7 +130,7 @@ __device__ __forceinline__ void nb_round_hi(uint32_t (&x)[16], const uint2 *hw, 
 // Forward: PRO_PLAIN with EPI_PLAIN, EPI_COMBINE or EPI_RESCALE; inverse: PRO_PLAIN or
 // PRO_GATHER with EPI_LAZY.  Residency: 48 registers (16 values, 30 of twiddles), five CTAs
 // (four and six, and loading the lo twiddles after the hi round: within 1 % or slower).
-template <int LOGN, bool FWD, int PRO, int EPI>
+template <int LOGN, bool FWD, int PRO, int EPI, bool DEP>
 __global__ void __launch_bounds__(kNttThreads, 5) k_ntt_blk(const __grid_constant__ SegList sl, const NttTables tb) {
   constexpr int TILES = (1 << LOGN) / kTile, S0 = LOGN - 8;
   __shared__ __align__(16) uint32_t sm[16 * 272];
@@ -141,9 +141,10 @@ __global__ void __launch_bounds__(kNttThreads, 5) k_ntt_blk(const __grid_constan
   const uint32_t q = tb.pc[lb.prime].q;
   const int blk = tile * 16 + c;
   uint2 *hw = hws + c * 16;
+  uint2 h1 = make_uint2(0, 0);
   if (tau) {  // this block's hi-round twiddles psi^brv(2^(S0 + m) + (blk << m) + j) at 2^m + j
     const int m = 31 - __clz(tau);
-    hw[tau] = __ldg((FWD ? tb.tw_fwd : tb.tw_inv) + ((size_t)lb.prime << LOGN) + (((1 << S0) + blk) << m) + tau - (1 << m));
+    h1 = __ldg((FWD ? tb.tw_fwd : tb.tw_inv) + ((size_t)lb.prime << LOGN) + (((1 << S0) + blk) << m) + tau - (1 << m));
   }
   uint2 tl[16];
   load_lo_twiddles<LOGN>(FWD ? tb.lo_fwd : tb.lo_inv, lb.prime, tile, tid, tl);
@@ -151,10 +152,12 @@ __global__ void __launch_bounds__(kNttThreads, 5) k_ntt_blk(const __grid_constan
   // this thread's i-th 16-byte chunk in memory order: element 64 i + 4 tau of the block
   auto lin = [&](int i) { return sm + nb_blk_addr(c, 64 * i + 4 * tau); };
   uint32_t x[16];
+  if (DEP) dep_wait();
   if (FWD) {
     const uint32_t *src = lb.src + blk * 256 + tau;
 #pragma unroll
-    for (int e = 0; e < 16; e++) x[e] = __ldg(src + e * 16);
+    for (int e = 0; e < 16; e++) x[e] = ld_in<DEP>(src + e * 16);
+    hw[tau] = h1;  // (stored after the loads are on their way, so that their latencies overlap)
     __syncwarp();  // the hi-round twiddles
     nb_round_hi<true>(x, hw, q);
 #pragma unroll
@@ -172,7 +175,7 @@ __global__ void __launch_bounds__(kNttThreads, 5) k_ntt_blk(const __grid_constan
     for (int i = 0; i < 4; i++) {
       const int j = blk * 256 + 64 * i + 4 * tau;
       uint32_t o[4], a[4];
-      if (EPI == EPI_COMBINE || EPI == EPI_RESCALE) ldg4(lb.src2 + j, a);
+      if (EPI == EPI_COMBINE || EPI == EPI_RESCALE) ld_in4<DEP>(lb.src2 + j, a);
       ld4(lin(i), o);
 #pragma unroll
       for (int e = 0; e < 4; e++) {
@@ -196,9 +199,10 @@ __global__ void __launch_bounds__(kNttThreads, 5) k_ntt_blk(const __grid_constan
     }
     uint32_t w[16];
 #pragma unroll
-    for (int i = 0; i < 4; i++) ldg4(src + 64 * i + 4 * tau, w + 4 * i);
+    for (int i = 0; i < 4; i++) ld_in4<DEP>(src + 64 * i + 4 * tau, w + 4 * i);
 #pragma unroll
     for (int i = 0; i < 4; i++) st4(lin(i), w + 4 * i);
+    hw[tau] = h1;
     __syncwarp();
     if (PRO == PRO_GATHER) {
       const uint32_t base = (__brev((uint32_t)tau) >> 28) * lb.galois + kadd;

@@ -21,7 +21,7 @@ template <bool FWD>
 constexpr int ntt_col_ctas() { return FWD ? 6 : 7; }
 
 // Forward: PRO_PLAIN or PRO_REDUCE with EPI_LAZY; inverse: PRO_PLAIN with EPI_SCALE.
-template <int LOGN, bool FWD, int PRO, int EPI>
+template <int LOGN, bool FWD, int PRO, int EPI, bool DEP>
 __global__ void __launch_bounds__(kNttThreads, ntt_col_ctas<FWD>())
     k_ntt_col(const __grid_constant__ SegList sl, const NttTables tb) {
   using G = NttGeom<LOGN, true>;
@@ -38,18 +38,23 @@ __global__ void __launch_bounds__(kNttThreads, ntt_col_ctas<FWD>())
   const uint32_t q = P.q;
   const uint2 *tw = (FWD ? tb.tw_fwd : tb.tw_inv) + ((size_t)lb.prime << LOGN);
   uint2 *hw = tws[tid >> 5];
-  if (lane < 16) hw[lane] = __ldg(tw + lane);  // hi round: entry 2^m + j is index 2^m + j
-  if (R == 8 && (lane & 15)) {                 // lo round: entry 2^m + j is index (16 + tau) 2^m + j
+  uint2 h1 = make_uint2(0, 0), h2 = make_uint2(0, 0);
+  if (lane < 16) h1 = __ldg(tw + lane);  // hi round: entry 2^m + j is index 2^m + j
+  if (R == 8 && (lane & 15)) {           // lo round: entry 2^m + j is index (16 + tau) 2^m + j
     const int h = lane & 15, m = 31 - __clz(h);
-    hw[16 + (lane >> 4) * kLo + h] = __ldg(tw + ((16 + tau) << m) + h - (1 << m));
+    h2 = __ldg(tw + ((16 + tau) << m) + h - (1 << m));
   }
   const uint2 *lw = hw + 16 + (tau & 1) * kLo;
+  if (DEP) dep_wait();
   uint32_t x[16];
 #pragma unroll
-  for (int e = 0; e < 16; e++) {
-    const uint32_t w = __ldg(lb.src + G::gidx(tile, c, kmap<R>(FWD, e, tau)));
-    x[e] = PRO == PRO_REDUCE ? reduce_u64(w, P) : w;  // a value of another prime, reduced exactly mod q
-  }
+  for (int e = 0; e < 16; e++) x[e] = ld_in<DEP>(lb.src + G::gidx(tile, c, kmap<R>(FWD, e, tau)));
+  // (stored after the loads are on their way, so that their latencies overlap)
+  if (lane < 16) hw[lane] = h1;
+  if (R == 8) hw[16 + (lane >> 4) * kLo + (lane & 15)] = h2;
+  if (PRO == PRO_REDUCE)
+#pragma unroll
+    for (int e = 0; e < 16; e++) x[e] = reduce_u64(x[e], P);  // a value of another prime, reduced exactly mod q
   __syncwarp();
   if (R == 4) {
     nb_round_hi<FWD>(x, hw, q);

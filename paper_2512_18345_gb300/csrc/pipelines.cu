@@ -64,7 +64,7 @@ static bool overlaps(const void *a, size_t abytes, const void *b, size_t bbytes)
 // run a program of at most kMaxInlineItems items with by-value launch arguments
 static int run_items(fhe_ctx *c, const std::vector<Item> &items, cudaStream_t s) {
   Program P;
-  int rc = build_program(c, items, c->fused != 0, P);
+  int rc = build_program(c, items, c->fused != 0, false, P);
   if (rc != FHE_OK) return rc;
   return run_program_inline(c, P, s);
 }
@@ -87,7 +87,7 @@ int run_items_chunked(fhe_ctx *c, const std::vector<Item> &items, int first_slot
       if (own_slot) it.slot = first_slot + nslot;
       chunk.push_back(it);
       Program Q;
-      const int rc = build_program(c, chunk, c->fused != 0, Q);
+      const int rc = build_program(c, chunk, c->fused != 0, false, Q);
       if (rc != FHE_OK) return rc;
       if (!program_fits_inline(Q)) {
         chunk.pop_back();

@@ -64,7 +64,7 @@ static void push_transform(fhe_ctx *c, Program &P, const Stage &first, const Sta
   P.stages.push_back(second);
 }
 
-int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, Program &P) {
+int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool fork, Program &P) {
   const size_t N = c->N;
   const int L = c->L, K = c->K, A = c->alpha;
   P.ks.clear();
@@ -291,10 +291,13 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, Progra
   ipp.gather_own = ipq.gather_own;
   ipp.gather_ext = ipq.gather_ext;
   ipp.add_c1 = ipq.add_c1;
-  // complementary pipelining (Section IV-B): the q-limb inner product on an auxiliary
-  // branch beside ModDown's special-limb chain; otherwise one launch over all limbs
+  // complementary pipelining (Section IV-B; `fork`, plans only): the q-limb inner product on an
+  // auxiliary branch beside ModDown's special-limb chain; otherwise one launch over all limbs.
+  // Single calls keep one stream: their stages are dependent launches, whose chain a fork and
+  // a join would break (one rotation at N = 2^16, L = 24: 120.5 us forked, 111.3 us on one
+  // stream; without dependent launches 137.8 and 135.8 us).
   const bool has_md = !m2.segs.empty();
-  const bool split = fused && c->comp_pipe && has_md && !ipq.segs.empty();
+  const bool split = fused && fork && has_md && !ipq.segs.empty();
   if (!ipq.segs.empty()) {
     if (split) {
       P.stages.push_back(marker(Stage::FORK));
@@ -366,6 +369,23 @@ static cudaError_t launch_stage(fhe_ctx *c, const Stage &st, const SegList &sl, 
   return cudaErrorInvalidValue;
 }
 
+// Largest launch (coefficients) taken as a dependent one: with several waves of CTAs the ramp
+// that a dependent launch hides is small beside the later waves' serialised prologues (256 limbs at
+// N = 2^16; with no limit the dense transform took 1281 us instead of 1250, with 128 limbs 1257 us
+// and one rotation at level 48 202.5 us instead of 198.9).
+static constexpr size_t kDepMaxWords = (size_t)256 << 16;
+
+// whether a stage's kernel begins with dep_wait (and so may be launched as a dependent one)
+static bool stage_waits(const fhe_ctx *c, const Stage &st) {
+  const DevTables &t = c->tabs;
+  switch (st.kind) {
+    case Stage::NTT: return !(st.column ? t.ntt_stream : t.ntt_stream || t.ntt_otf);
+    case Stage::BCONV: return c->bconv_mode != FHE_BCONV_TC || !t.bconv_tc_pipe;
+    case Stage::IP: return !st.gather_ext || (t.ip_staged && !st.add_c1);
+    default: return false;
+  }
+}
+
 bool program_fits_inline(const Program &P) {
   if ((int)P.ks.size() > kMaxInlineItems) return false;
   for (const Stage &st : P.stages) {
@@ -381,6 +401,13 @@ int run_program_inline(fhe_ctx *c, const Program &P, cudaStream_t s) {
   if (!program_fits_inline(P)) return fhe_fail(FHE_EINVAL, "internal: program does not fit inline launch arguments");
   SegList sl, sl2;
   BconvArgs ba;
+  // Dependent launches: a stage kernel that begins with dep_wait (the transform passes, the base
+  // conversions and the inner products in their default forms) may start its prologue under the
+  // stage before it, when that stage's kernel is the last thing on the stream.  Not while the
+  // caller captures, where forks and joins would mix with programmatic edges, nor under tracing.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool dep_ok = !c->tabs.tracer && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+  bool after_kernel = false;
   for (const Stage &st : P.stages) {
     memset(&sl, 0, sizeof sl);
     memset(&sl2, 0, sizeof sl2);
@@ -406,9 +433,17 @@ int run_program_inline(fhe_ctx *c, const Program &P, cudaStream_t s) {
       }
       sl.lm_groups = ok ? g : 0;
     }
-    for (const BconvGroup &g : st.groups) ba.g[ba.ngroups++] = g;
+    size_t limbs = sl.total;
+    for (const BconvGroup &g : st.groups) {
+      ba.g[ba.ngroups++] = g;
+      limbs += g.n_out;
+    }
     ba.lazy = 1;  // every conversion of a program feeds a forward NTT
+    const bool kernel = st.kind != Stage::FORK && st.kind != Stage::JOIN_RECORD && st.kind != Stage::JOIN_WAIT;
+    c->tabs.dep = dep_ok && after_kernel && !st.aux && (limbs << c->logn) <= kDepMaxWords && stage_waits(c, st);
     cudaError_t e = launch_stage(c, st, sl, ba, s, 0, &sl2);
+    c->tabs.dep = 0;
+    after_kernel = kernel && !st.aux;
     if (e != cudaSuccess) return fhe_fail(FHE_ECUDA, "stage launch: %s", cudaGetErrorString(e));
   }
   return FHE_OK;

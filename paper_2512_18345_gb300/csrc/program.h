@@ -58,7 +58,8 @@ struct DevProgram {
 };
 
 int ensure_slots(fhe_ctx *c, int n);
-int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, Program &P);
+// fork: the inner product of the ciphertext limbs on an auxiliary branch (complementary pipelining)
+int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool fork, Program &P);
 bool program_fits_inline(const Program &P);
 int run_program_inline(fhe_ctx *c, const Program &P, cudaStream_t s);
 int upload_program(fhe_ctx *c, const Program &P, DevProgram &D);
