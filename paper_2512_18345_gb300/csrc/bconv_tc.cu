@@ -20,7 +20,7 @@
 // accumulation in tensor memory is exact in any order, and the accumulator's
 // bit pattern is 0x4B000000 + S_b (no conversion instruction needed).
 // The epilogue forms lo = S_0 + 2^8 S_1 and hi = S_2 + 2^8 S_3 (both < 2^30)
-// and reduces lo + 2^16 hi modulo p_o once: bit-identical to the CUDA-core path.
+// and reduces lo + 2^16 hi modulo p_o: bit-identical to the CUDA-core path.
 //
 // Digits of 9..12 limbs (the paper's alpha = 12) use K = 64: 48 data slots and 8
 // offset slots whose B pieces may be negative (each in [-2048, 2048], summing to
@@ -28,8 +28,7 @@
 // ends at 2^23 + S_b with S_b < 48 * 255^2 < 2^22; every partial sum lies between the
 // sum of the negative terms (> -2^22 * 1.0) and the sum of the positive ones
 // (< 1024 * 12240 + 2^22 < 2^24), so the fp32 accumulation stays exact in any order.
-// The epilogue's lo, hi < 2^30 + 2^22, so one conditional subtraction after adding
-// 2^16 hi mod p suffices for primes above 2^30 + 2^23.
+// The epilogue's lo, hi < 2^30 + 2^22 then (tc_out1's bounds hold for both widths).
 //
 // A 128-coefficient tile of one group is one M = 128 MMA of K / 16 steps;
 // persistent CTAs of 256 threads walk the tiles (see k_bconv_tc).  Operands sit
@@ -82,38 +81,52 @@ struct TcOut {  // per output prime of the current group, read by whole warps (o
 // One warp's share of a tile's epilogue: outputs [o_beg, o_end) of the accumulator at tbase
 // (columns 4 o + b hold 2^23 + S_b[o]) for coefficient n, four outputs (one 16-column load)
 // at a time with no predicated slots except in a last partial group.  lo = S_0 + 2^8 S_1 and
-// hi = S_2 + 2^8 S_3 (the 0x4B000000 of each accumulator cancels modulo 2^32), then
-// lo + (2^16 hi mod p) reduced once.  LAZY: the value is left in [0, 2p) (the conversions
-// inside the key-switching pipeline feed a forward NTT, which takes such inputs).
-template <bool LAZY>
-__device__ __forceinline__ void tc_out1(const uint32_t *r, const TcOut &t, uint32_t *gn, bool big_primes) {
+// hi = S_2 + 2^8 S_3 (the 0x4B000000 of each accumulator cancels modulo 2^32), both below
+// 2^30 + 2^22.  t = 2^16 hi - floor(hi w16s / 2^32) p: as hi / 2^32 < 0.251, the quotient is
+// short of the true one by less than 1.251, so t < 1.251 p and lo + t < 2^32 with no
+// reduction between; for primes above kBigPrime lo + t < 2 p, so LAZY outputs (the conversions
+// inside the key-switching pipeline feed a forward NTT, which takes [0, 2p)) are done there and
+// the others need one conditional subtraction.  BIG: every output prime of the group is above
+// kBigPrime, decided per group and outside the loop.  Bound: instruction issue (58 % busy, the
+// MMA itself is small).  The two conversions of 8 rotations at N = 2^16, L = 24, K = 8 take
+// 92.0 us; reducing t and choosing BIG inside the loop took 104.4.
+constexpr uint32_t kBigPrime = 1450000000u;  // > (2^30 + 2^22) / (2 - 1.251)
+template <bool LAZY, bool BIG>
+__device__ __forceinline__ void tc_out1(const uint32_t *r, const TcOut &t, uint32_t *gn) {
   const uint32_t lo = r[1] * 256u + r[0] - 0x4B000000u;
   const uint32_t hi = r[3] * 256u + r[2] - 0x4B000000u;
-  const uint32_t sum = lo + red2(shoup_lazy(hi, 65536u, t.w16s, t.q), t.q);  // < 2^30 + 2^22 + q
-  uint32_t v;
-  if (big_primes) v = LAZY ? sum : red2(sum, t.q);
-  else {
-    v = shoup_lazy(sum, 1u, t.div32, t.q);
-    if (!LAZY) v = red2(v, t.q);
-  }
-  gn[t.off] = v;
+  uint32_t v = lo + shoup_lazy(hi, 65536u, t.w16s, t.q);
+  if (!BIG) v = shoup_lazy(v, 1u, t.div32, t.q);
+  gn[t.off] = LAZY ? v : red2(v, t.q);
 }
-template <bool LAZY>
-__device__ __forceinline__ void tc_reduce_outputs(uint32_t tbase, int o_beg, int o_end, const TcOut *sO, uint32_t *gn,
-                                                  bool big_primes) {
-  for (int o0 = o_beg; o0 < o_end; o0 += 4) {
+template <bool LAZY, bool BIG>
+__device__ __forceinline__ void tc_reduce_outputs(uint32_t tbase, int o_beg, int o_end, const TcOut *sO, uint32_t *gn) {
+  int o0 = o_beg;
+  for (; o0 + 4 <= o_end; o0 += 4) {
+    uint32_t rr[16];
+    tmem_ld16(rr, tbase + (uint32_t)(4 * o0));
+    TcOut t[4];
+#pragma unroll
+    for (int i = 0; i < 4; i++) t[i] = sO[o0 + i];
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 4; i++) tc_out1<LAZY, BIG>(rr + 4 * i, t[i], gn);
+  }
+  if (o0 < o_end) {
     uint32_t rr[16];
     tmem_ld16(rr, tbase + (uint32_t)(4 * o0));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    if (o0 + 4 <= o_end) {
 #pragma unroll
-      for (int i = 0; i < 4; i++) tc_out1<LAZY>(rr + 4 * i, sO[o0 + i], gn, big_primes);
-    } else {
-#pragma unroll
-      for (int i = 0; i < 3; i++)
-        if (o0 + i < o_end) tc_out1<LAZY>(rr + 4 * i, sO[o0 + i], gn, big_primes);
-    }
+    for (int i = 0; i < 3; i++)
+      if (o0 + i < o_end) tc_out1<LAZY, BIG>(rr + 4 * i, sO[o0 + i], gn);
   }
+}
+__device__ __forceinline__ void tc_epilogue(bool lazy, bool big, uint32_t tbase, int o_beg, int o_end, const TcOut *sO,
+                                            uint32_t *gn) {
+  if (lazy && big) tc_reduce_outputs<true, true>(tbase, o_beg, o_end, sO, gn);
+  else if (lazy) tc_reduce_outputs<true, false>(tbase, o_beg, o_end, sO, gn);
+  else if (big) tc_reduce_outputs<false, true>(tbase, o_beg, o_end, sO, gn);
+  else tc_reduce_outputs<false, false>(tbase, o_beg, o_end, sO, gn);
 }
 
 // Persistent: a CTA walks tiles (group, 128-coefficient block) in group-major
@@ -133,7 +146,6 @@ __global__ void __launch_bounds__(kTcThreads, 4) k_bconv_tc(const __grid_constan
   constexpr uint32_t kSbo = (KT / 8) * 128u;         // 8-row group stride
   constexpr int kDataChunks = KT == kTcK ? 4 : 6;    // 8-slot K chunks holding inputs (two each)
   constexpr int kNch = kDataChunks / 2;              // data chunks built by each thread
-  constexpr uint32_t kBigPrime = KT == kTcK ? (1u << 30) : (1u << 30) + (1u << 23);
   uint8_t *sA = smem;
   uint8_t *sB = smem + kTcM * kRowBytes;
   TcOut *sO = reinterpret_cast<TcOut *>(sB + (size_t)npad_max * kRowBytes);
@@ -187,7 +199,7 @@ __global__ void __launch_bounds__(kTcThreads, 4) k_bconv_tc(const __grid_constan
   for (int h = 0; h < 2 * kNch; h++) y[h] = 0u;
   if (DEP) dep_wait();
   bool prefetched = false;  // y holds the current tile's inputs
-  bool big_primes = true;   // the current group's output primes all exceed 2^30
+  bool big_primes = true;   // the current group's output primes all exceed kBigPrime
   for (int tile = t0; tile < t1 && ok; tile++) {
     const int grp = tile >> ltg;
     const size_t n0 = (size_t)(tile & (tiles_per_group - 1)) * kTcM;
@@ -201,7 +213,7 @@ __global__ void __launch_bounds__(kTcThreads, 4) k_bconv_tc(const __grid_constan
       uint4 *dst = reinterpret_cast<uint4 *>(sB);
       const int n16 = npad * (int)kRowBytes / 16;
       for (int i = tid; i < n16; i += kTcThreads) dst[i] = __ldg(src + i);
-      bool big = true;  // every output prime above kBigPrime: one conditional subtraction suffices
+      bool big = true;
       for (int o = tid; o < n_out; o += kTcThreads) {
         const int2 m = gp->omap[o];
         const PrimeC p = pc[m.y];
@@ -271,8 +283,7 @@ __global__ void __launch_bounds__(kTcThreads, 4) k_bconv_tc(const __grid_constan
       const int H = ((n_out + 1) / 2 + 3) & ~3;
       const int o_end = (warp >> 2) ? n_out : min(H, n_out);
       uint32_t *gn = gp->out + n;  // this thread's coefficient of the group's output limb 0
-      if (a.lazy) tc_reduce_outputs<true>(tbase, (warp >> 2) ? H : 0, o_end, sO, gn, big_primes);
-      else tc_reduce_outputs<false>(tbase, (warp >> 2) ? H : 0, o_end, sO, gn, big_primes);
+      tc_epilogue(a.lazy, big_primes, tbase, (warp >> 2) ? H : 0, o_end, sO, gn);
     } else {
       if ((tid & 31) == 0) atomicOr(status, 1u);  // expired wait: report, give the MMA a second bounded chance
       mbar_wait_bounded(bar, phase ^ 1u);
@@ -305,7 +316,6 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_bconv_tc_pipe(const __grid_co
   constexpr uint32_t kSbo = (KT / 8) * 128u;
   constexpr int kDataChunks = KT == kTcK ? 4 : 6;
   constexpr int kNch = kDataChunks / 2;
-  constexpr uint32_t kBigPrime = KT == kTcK ? (1u << 30) : (1u << 30) + (1u << 23);
   constexpr uint32_t kAbytes = kTcM * kRowBytes;
   uint8_t *sA = smem;  // two buffers
   uint8_t *sB = smem + 2 * kAbytes;
@@ -381,8 +391,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_bconv_tc_pipe(const __grid_co
     const int H = ((n_out + 1) / 2 + 3) & ~3;
     const int o_end = (warp >> 2) ? n_out : min(H, n_out);
     uint32_t *gn = gp->out + n;
-    if (a.lazy) tc_reduce_outputs<true>(tbase, (warp >> 2) ? H : 0, o_end, sO, gn, big_primes);
-    else tc_reduce_outputs<false>(tbase, (warp >> 2) ? H : 0, o_end, sO, gn, big_primes);
+    tc_epilogue(a.lazy, big_primes, tbase, (warp >> 2) ? H : 0, o_end, sO, gn);
   };
   for (int tile = t0; tile < t1 && ok; tile++) {
     const int grp = tile >> ltg;
