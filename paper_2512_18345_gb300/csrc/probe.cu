@@ -111,7 +111,10 @@ __global__ void __launch_bounds__(kProbeThreads, kProbeCtasPerSm) k_probe_int(ui
 
 extern "C" int fhe_probe_int(int device, fhe_int_peaks *out) {
   if (!out) return fhe_fail(FHE_EINVAL, "fhe_probe_int: null output");
-  if (cudaSetDevice(device) != cudaSuccess) return fhe_fail(FHE_ECUDA, "fhe_probe_int: device %d", device);
+  if (cudaSetDevice(device) != cudaSuccess) {
+    cudaGetLastError();  // (not left pending for the thread's next launch)
+    return fhe_fail(FHE_ECUDA, "fhe_probe_int: device %d", device);
+  }
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   const int grid = sms * kProbeCtasPerSm;
@@ -178,7 +181,10 @@ extern "C" int fhe_probe_bandwidth(int device, size_t bytes, int reps, double *r
                                    double *copy_gbs) {
   if (bytes < (1u << 20) || reps < 1 || !read_gbs || !write_gbs || !copy_gbs)
     return fhe_fail(FHE_EINVAL, "fhe_probe_bandwidth: bytes >= 1 MiB, reps >= 1, non-null outputs");
-  if (cudaSetDevice(device) != cudaSuccess) return fhe_fail(FHE_ECUDA, "fhe_probe_bandwidth: device %d", device);
+  if (cudaSetDevice(device) != cudaSuccess) {
+    cudaGetLastError();  // (not left pending for the thread's next launch)
+    return fhe_fail(FHE_ECUDA, "fhe_probe_bandwidth: device %d", device);
+  }
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
   uint4 *a = nullptr, *b = nullptr;

@@ -27,8 +27,8 @@ def test_transform_of_many_limbs(fhe_lib, n, run):
 
 
 def test_context_after_a_refused_call(fhe_lib):
-    """A probe of a device that is not there leaves a pending CUDA error on the thread; a context
-    is created after it and computes all the same."""
+    """A probe of a device that is not there fails alone: a context is created after it and
+    computes, its first launches included."""
     from paper_2512_18345_gb300 import binding
     P = inputs.workload_params("hmult_relin_rescale_N4096_L4")
     with pytest.raises(binding.FheError):
@@ -38,3 +38,5 @@ def test_context_after_a_refused_call(fhe_lib):
     t = binding.to_device(a)
     ctx.ntt(t, [0, 1])
     assert np.array_equal(binding.to_numpy(t), oracle.ntt(a, P.primes[:2]))
+    assert np.array_equal(binding.to_numpy(ctx.add(t, t, 2, npoly=1))[0], (2 * oracle.ntt(a, P.primes[:2]).astype(np.uint64) %
+                                                                         np.array(P.primes[:2], np.uint64)[:, None]))
