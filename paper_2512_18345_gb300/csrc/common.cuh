@@ -82,6 +82,12 @@ __device__ __forceinline__ uint32_t mul_mod(uint32_t a, uint32_t b, const PrimeC
   return reduce_u64((uint64_t)a * b, P);
 }
 
+// a = hi 2^34 + lo  ->  hi r34 + lo with r34 = 2^34 mod q: the same residue, below 2^61 + 2^34
+// for any 64-bit a (hi < 2^30, r34 < 2^31), so three more products below 2^62 still fit
+__device__ __forceinline__ uint64_t fold34(uint64_t a, uint32_t r34) {
+  return (uint64_t)(uint32_t)(a >> 34) * r34 + (a & ((1ull << 34) - 1));
+}
+
 // ---------------------------------------------------------------- automorphism
 // NTT-form Galois map sigma_k: slot i (value at psi^(2 brv(i)+1)) of the
 // output is slot j of the input with 2 brv(j) + 1 = (2 brv(i) + 1) k mod 2N,
@@ -106,9 +112,11 @@ struct Seg {
   const uint2 *scale;  // per-limb Shoup constant pairs (inverse-NTT output scale), or null
   int t0;            // extended-basis index of the first limb (inner product)
   int key_row0;      // key row of the first limb
-  int c;             // which half (0: b / c0, 1: a / c1) a combine uses
+  int c;             // small ring's inner product: 1 where the limb's inverse transform follows
   int item;          // index of this segment's key-switching arguments
   uint32_t galois;   // Galois element applied when src is gathered (1: none)
+  int n_in;          // PRO_BCONV: src is n_in limbs, T the first limb's row of the conversion table
+  const uint32_t *T;
 };
 
 // Key-switching arguments of one item (one key switch) for the inner product,
@@ -141,9 +149,11 @@ struct alignas(16) Limb {
   uint32_t *dst;
   const uint32_t *src2;
   const uint2 *scale;  // the limb's own constant (output scale, or P^-1 for a combine), or null
+  const uint32_t *T;   // PRO_BCONV: its row of the conversion table, over n_in input limbs at src
   int prime;
   uint32_t galois;     // sigma applied when reading src (PRO_GATHER, EW_GATHER)
   int n;               // limbs in the segment (the HMult tensor's polynomial stride)
+  int n_in;
 };
 
 // A launch's work list: segments and per-item arguments, either inline (by
@@ -198,10 +208,10 @@ template <bool COMBINE>
 __device__ __forceinline__ Limb limb_at(const SegList &L, int v, const uint2 *dflt, int logn) {
   if (L.limbs) {
     const uint4 *p = reinterpret_cast<const uint4 *>(L.limbs + v);
-    union { uint4 w[3]; Limb d; } u;
-    u.w[0] = __ldg(p);
-    u.w[1] = __ldg(p + 1);
-    u.w[2] = __ldg(p + 2);
+    static_assert(sizeof(Limb) == 64, "a limb descriptor is four 16-byte loads");
+    union { uint4 w[4]; Limb d; } u;
+#pragma unroll
+    for (int i = 0; i < 4; i++) u.w[i] = __ldg(p + i);
     return u.d;
   }
   int within;
@@ -215,6 +225,8 @@ __device__ __forceinline__ Limb limb_at(const SegList &L, int v, const uint2 *df
   d.scale = COMBINE ? L.ks[s.item].pinv + d.prime : s.scale ? s.scale + within : dflt ? dflt + d.prime : nullptr;
   d.galois = s.galois;
   d.n = s.n;
+  d.T = s.T + (size_t)within * s.n_in;
+  d.n_in = s.n_in;
   return d;
 }
 

@@ -129,6 +129,11 @@ cudaError_t launch_ntt_single(const DevTables &t, bool fwd, int pro, int epi, co
                               const SegList &second, cudaStream_t s);
 // how many 16-CTA clusters of the single-pass NTT the current device holds at once (0: none)
 int ntt_single_pass_clusters();
+// the small ring's whole-limb transform and inner product (ntt_small.cuh); a transform reads
+// its source and prologue from sl and writes its destination and epilogue in one launch
+bool ntt_small_ok(const DevTables &t);
+cudaError_t launch_small_ntt(const DevTables &t, bool fwd, int pro, int epi, const SegList &sl, cudaStream_t s);
+cudaError_t launch_small_ip(const DevTables &t, const SegList &sl, cudaStream_t s);
 cudaError_t launch_bconv(const DevTables &t, const BconvArgs &a, int max_in, int max_out, cudaStream_t s);
 // kt: the K of the groups' tables (48: max_in <= 8; 64: max_in <= 12)
 cudaError_t launch_bconv_tc(const DevTables &t, const BconvArgs &a, int max_in, int max_out, cudaStream_t s, int kt);

@@ -10,6 +10,7 @@
 #include "ntt.cuh"
 #include "ntt_blk.cuh"
 #include "ntt_col.cuh"
+#include "ntt_small.cuh"
 #include "ntt_bulk.cuh"
 #include "ip_intt.cuh"
 #include "ip_hoisted.cuh"
@@ -281,8 +282,49 @@ static bool same_limbs(const SegList &a, const SegList &b) {
   return true;
 }
 
+// N = 2^12 with the default twiddles: whole-limb transforms, one launch each
+bool ntt_small_ok(const DevTables &t) { return t.logn == kSmallLogN && !t.ntt_otf; }
+
+cudaError_t launch_small_ntt(const DevTables &t, bool fwd, int pro, int epi, const SegList &sl, cudaStream_t s) {
+  if (sl.total == 0) return cudaSuccess;
+  TraceScope ts(t, fwd ? (pro == PRO_BCONV ? (epi == EPI_COMBINE ? "small_bconv_ntt+combine" : "small_bconv_ntt") : "small_ntt")
+                       : "small_intt", s);
+  g_launches++;
+#define SMALL_FWD(P, E)              \
+  if (fwd && pro == P && epi == E)   \
+    return launch_dep(t, t.dep ? k_small_ntt<P, E, true> : k_small_ntt<P, E, false>, sl.total, kNttThreads, 0, s, sl, t.ntt);
+  SMALL_FWD(PRO_PLAIN, EPI_PLAIN)
+  SMALL_FWD(PRO_REDUCE, EPI_RESCALE)
+  SMALL_FWD(PRO_BCONV, EPI_PLAIN)
+  SMALL_FWD(PRO_BCONV, EPI_COMBINE)
+#undef SMALL_FWD
+  if (fwd || epi != EPI_SCALE) return cudaErrorInvalidValue;
+  if (pro == PRO_PLAIN)
+    return launch_dep(t, t.dep ? k_small_intt<PRO_PLAIN, true> : k_small_intt<PRO_PLAIN, false>, sl.total, kNttThreads, 0, s,
+                      sl, t.ntt);
+  if (pro == PRO_GATHER)
+    return launch_dep(t, t.dep ? k_small_intt<PRO_GATHER, true> : k_small_intt<PRO_GATHER, false>, sl.total, kNttThreads, 0,
+                      s, sl, t.ntt);
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_small_ip(const DevTables &t, const SegList &sl, cudaStream_t s) {
+  if (sl.total == 0) return cudaSuccess;
+  TraceScope ts(t, "small_ip", s);
+  g_launches++;
+  return launch_dep(t, t.dep ? k_small_ip<true> : k_small_ip<false>, 2 * sl.total, kNttThreads, 0, s, sl, t.ntt);
+}
+
 cudaError_t launch_ntt(const DevTables &t, bool fwd, int pro, int epi, const SegList &first, const SegList &second,
                        cudaStream_t s) {
+  if (ntt_small_ok(t) && same_limbs(first, second)) {
+    SegList one = second;  // the first pass's source, the second's destination and constants
+    for (int i = 0; i < one.nseg; i++) {
+      one.seg[i].src = first.seg[i].src;
+      one.seg[i].src_stride = first.seg[i].src_stride;
+    }
+    return launch_small_ntt(t, fwd, pro, epi, one, s);
+  }
   if ((t.ntt_single || t.ntt_persist) && ntt_single_pass_ok(t, pro, epi, fwd) && same_limbs(first, second))
     return launch_ntt_single(t, fwd, pro, epi, first, second, s);
   cudaError_t e;

@@ -69,12 +69,6 @@ constexpr int kDiagStageBytes = kDiagRows * kDiagChunk * 4 + 16;  // rows, two m
 constexpr int kDiagStages = 8;
 static_assert(kDiagStages * kDiagStageBytes <= 227 * 1024, "diagonal kernel: stages exceed shared memory");
 
-// a = hi 2^34 + lo  ->  hi r34 + lo with r34 = 2^34 mod q: the same residue, below 2^61 + 2^34
-// for any 64-bit a (hi < 2^30, r34 < 2^31), so three more products below 2^62 still fit
-__device__ __forceinline__ uint64_t fold34(uint64_t a, uint32_t r34) {
-  return (uint64_t)(uint32_t)(a >> 34) * r34 + (a & ((1ull << 34) - 1));
-}
-
 __global__ void __launch_bounds__(kDiagThreads + 32, 1) k_diag_bulk(const __grid_constant__ DiagArgs a, const PrimeC *pc,
                                                                    int logn, unsigned int *status) {
   constexpr int stages = kDiagStages;

@@ -45,6 +45,7 @@ enum : int {
   PRO_PLAIN = 0,   // src[j]
   PRO_GATHER = 1,  // src[sigma(j)], sigma = the limb's galois (NTT form input)
   PRO_REDUCE = 2,  // src[j] reduced from another prime (rescale: src_prime)
+  PRO_BCONV = 3,   // base conversion of n_in limbs at src (small ring)
 };
 // Epilogue modes (how the last pass writes an element)
 enum : int {

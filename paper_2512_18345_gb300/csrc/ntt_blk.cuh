@@ -127,12 +127,106 @@ __device__ __forceinline__ void nb_round_hi(uint32_t (&x)[16], const uint2 *hw, 
   }
 }
 
+// ---- the pass in pieces (thread (c, tau) of a 16-block tile; sm: the tile's 16 x 272 words)
+
+// this thread's entry tau of block blk's hi-round twiddles, psi^brv(2^(S0 + m) + (blk << m) + j)
+// at 2^m + j (entry 0 unused)
+template <int LOGN, bool FWD>
+__device__ __forceinline__ uint2 blk_hi_twiddle(const NttTables &tb, int prime, int blk, int tau) {
+  if (!tau) return make_uint2(0, 0);
+  const int m = 31 - __clz(tau);
+  return __ldg((FWD ? tb.tw_fwd : tb.tw_inv) + ((size_t)prime << LOGN) + (((1 << (LOGN - 8)) + blk) << m) + tau - (1 << m));
+}
+// a thread's i-th 16-byte chunk in memory order: element 64 i + 4 tau of block c
+__device__ __forceinline__ uint32_t *blk_lin(uint32_t *sm, int c, int tau, int i) {
+  return sm + nb_blk_addr(c, 64 * i + 4 * tau);
+}
+// forward: x in hi layout (element 16 e + tau) -> lazy results in sm
+__device__ __forceinline__ void blk_forward(uint32_t (&x)[16], uint32_t *sm, int c, int tau, const uint2 *hw,
+                                            const uint2 (&tl)[16], uint32_t q) {
+  nb_round_hi<true>(x, hw, q);
+#pragma unroll
+  for (int e = 0; e < 16; e++) sm[nb_blk_addr(c, (e << 4) | tau)] = x[e];
+  __syncwarp();
+#pragma unroll
+  for (int m = 0; m < 4; m++) ld4(sm + nb_blk_addr(c, (tau << 4) | (4 * m)), x + 4 * m);
+  nb_round<true>(x, [&](int m, int j) { return tl[(1 << m) - 1 + j]; }, q);
+#pragma unroll
+  for (int m = 0; m < 4; m++) st4(sm + nb_blk_addr(c, (tau << 4) | (4 * m)), x + 4 * m);
+  __syncwarp();
+}
+// write the results in sm to the limb in memory order
+template <int EPI, bool DEP>
+__device__ __forceinline__ void blk_store(const Limb &lb, int blk, uint32_t *sm, int c, int tau, uint2 scale, uint32_t q) {
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    const int j = blk * 256 + 64 * i + 4 * tau;
+    uint32_t o[4], a[4];
+    if (EPI == EPI_COMBINE || EPI == EPI_RESCALE) ld_in4<DEP>(lb.src2 + j, a);
+    ld4(blk_lin(sm, c, tau, i), o);
+#pragma unroll
+    for (int e = 0; e < 4; e++) {
+      o[e] = red2(o[e], q);
+      // COMBINE: a = inner product u (with P times the pass-through term folded in)
+      if (EPI == EPI_COMBINE || EPI == EPI_RESCALE) o[e] = shoup(a[e] + q - o[e], scale.x, scale.y, q);
+    }
+    st4(lb.dst + j, o);
+  }
+}
+// the inverse's input: block blk (PRO_GATHER: read through sigma_galois) into lo layout
+// (element 16 tau + e); `staged` runs once the loads are on their way
+template <int LOGN, int PRO, bool DEP, class F>
+__device__ __forceinline__ void blk_load(uint32_t (&x)[16], const uint32_t *src, uint32_t galois, int blk, uint32_t *sm,
+                                         int c, int tau, F staged) {
+  constexpr int S0 = LOGN - 8;
+  uint32_t kadd = 0;
+  if (PRO == PRO_GATHER) {
+    // index blk 256 + k has brv = brv8(k) 2^S0 + brv(blk); times g plus g >> 1, its low S0
+    // bits give the source block and the rest brv8 of the source element: brv8(k) g + kadd
+    const uint32_t r = (__brev((uint32_t)blk) >> (32 - S0)) * galois + (galois >> 1);
+    kadd = r >> S0;
+    src += (__brev(r << (32 - S0)) << 8);
+  } else {
+    src += blk * 256;
+  }
+  uint32_t w[16];
+#pragma unroll
+  for (int i = 0; i < 4; i++) ld_in4<DEP>(src + 64 * i + 4 * tau, w + 4 * i);
+#pragma unroll
+  for (int i = 0; i < 4; i++) st4(blk_lin(sm, c, tau, i), w + 4 * i);
+  staged();
+  __syncwarp();
+  if (PRO == PRO_GATHER) {
+    const uint32_t base = (__brev((uint32_t)tau) >> 28) * galois + kadd;
+#pragma unroll
+    for (int e = 0; e < 16; e++) {
+      const uint32_t be = ((e & 1) << 3) | ((e & 2) << 1) | ((e & 4) >> 1) | ((e & 8) >> 3);  // brv4(e)
+      x[e] = sm[nb_blk_addr(c, (int)(__brev(base + be * 16u * galois) >> 24))];
+    }
+    __syncwarp();  // every lane's reads come before the rows are rewritten
+  } else {
+#pragma unroll
+    for (int m = 0; m < 4; m++) ld4(sm + nb_blk_addr(c, (tau << 4) | (4 * m)), x + 4 * m);
+  }
+}
+// inverse: x in lo layout -> x in hi layout
+__device__ __forceinline__ void blk_inverse(uint32_t (&x)[16], uint32_t *sm, int c, int tau, const uint2 *hw,
+                                            const uint2 (&tl)[16], uint32_t q) {
+  nb_round<false>(x, [&](int m, int j) { return tl[(1 << m) - 1 + j]; }, q);
+#pragma unroll
+  for (int m = 0; m < 4; m++) st4(sm + nb_blk_addr(c, (tau << 4) | (4 * m)), x + 4 * m);
+  __syncwarp();
+#pragma unroll
+  for (int e = 0; e < 16; e++) x[e] = sm[nb_blk_addr(c, (e << 4) | tau)];
+  nb_round_hi<false>(x, hw, q);
+}
+
 // Forward: PRO_PLAIN with EPI_PLAIN, EPI_COMBINE or EPI_RESCALE; inverse: PRO_PLAIN or
 // PRO_GATHER with EPI_LAZY.  Residency: 48 registers (16 values, 30 of twiddles), five CTAs
 // (four and six, and loading the lo twiddles after the hi round: within 1 % or slower).
 template <int LOGN, bool FWD, int PRO, int EPI, bool DEP>
-__global__ void __launch_bounds__(kNttThreads, 5) k_ntt_blk(const __grid_constant__ SegList sl, const NttTables tb) {
-  constexpr int TILES = (1 << LOGN) / kTile, S0 = LOGN - 8;
+__global__ void __launch_bounds__(kNttThreads, DEP && FWD ? 4 : 5) k_ntt_blk(const __grid_constant__ SegList sl, const NttTables tb) {
+  constexpr int TILES = (1 << LOGN) / kTile;
   __shared__ __align__(16) uint32_t sm[16 * 272];
   __shared__ __align__(16) uint2 hws[16 * 16];
   const int tid = threadIdx.x, c = tid >> 4, tau = tid & 15;
@@ -141,16 +235,9 @@ __global__ void __launch_bounds__(kNttThreads, 5) k_ntt_blk(const __grid_constan
   const uint32_t q = tb.pc[lb.prime].q;
   const int blk = tile * 16 + c;
   uint2 *hw = hws + c * 16;
-  uint2 h1 = make_uint2(0, 0);
-  if (tau) {  // this block's hi-round twiddles psi^brv(2^(S0 + m) + (blk << m) + j) at 2^m + j
-    const int m = 31 - __clz(tau);
-    h1 = __ldg((FWD ? tb.tw_fwd : tb.tw_inv) + ((size_t)lb.prime << LOGN) + (((1 << S0) + blk) << m) + tau - (1 << m));
-  }
+  const uint2 h1 = blk_hi_twiddle<LOGN, FWD>(tb, lb.prime, blk, tau);
   uint2 tl[16];
   load_lo_twiddles<LOGN>(FWD ? tb.lo_fwd : tb.lo_inv, lb.prime, tile, tid, tl);
-  auto lw = [&](int m, int j) { return tl[(1 << m) - 1 + j]; };
-  // this thread's i-th 16-byte chunk in memory order: element 64 i + 4 tau of the block
-  auto lin = [&](int i) { return sm + nb_blk_addr(c, 64 * i + 4 * tau); };
   uint32_t x[16];
   if (DEP) dep_wait();
   if (FWD) {
@@ -159,70 +246,13 @@ __global__ void __launch_bounds__(kNttThreads, 5) k_ntt_blk(const __grid_constan
     for (int e = 0; e < 16; e++) x[e] = ld_in<DEP>(src + e * 16);
     hw[tau] = h1;  // (stored after the loads are on their way, so that their latencies overlap)
     __syncwarp();  // the hi-round twiddles
-    nb_round_hi<true>(x, hw, q);
-#pragma unroll
-    for (int e = 0; e < 16; e++) sm[nb_blk_addr(c, (e << 4) | tau)] = x[e];
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < 4; m++) ld4(sm + nb_blk_addr(c, (tau << 4) | (4 * m)), x + 4 * m);
-    nb_round<true>(x, lw, q);
-#pragma unroll
-    for (int m = 0; m < 4; m++) st4(sm + nb_blk_addr(c, (tau << 4) | (4 * m)), x + 4 * m);
+    blk_forward(x, sm, c, tau, hw, tl, q);
     uint2 scale = make_uint2(0, 0);
     if (EPI == EPI_COMBINE || EPI == EPI_RESCALE) scale = __ldg(lb.scale);
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-      const int j = blk * 256 + 64 * i + 4 * tau;
-      uint32_t o[4], a[4];
-      if (EPI == EPI_COMBINE || EPI == EPI_RESCALE) ld_in4<DEP>(lb.src2 + j, a);
-      ld4(lin(i), o);
-#pragma unroll
-      for (int e = 0; e < 4; e++) {
-        o[e] = red2(o[e], q);
-        // COMBINE: a = inner product u (with P times the pass-through term folded in)
-        if (EPI == EPI_COMBINE || EPI == EPI_RESCALE) o[e] = shoup(a[e] + q - o[e], scale.x, scale.y, q);
-      }
-      st4(lb.dst + j, o);
-    }
+    blk_store<EPI, DEP>(lb, blk, sm, c, tau, scale, q);
   } else {
-    const uint32_t *src = lb.src;
-    uint32_t kadd = 0;
-    if (PRO == PRO_GATHER) {
-      // index blk 256 + k has brv = brv8(k) 2^S0 + brv(blk); times g plus g >> 1, its low S0
-      // bits give the source block and the rest brv8 of the source element: brv8(k) g + kadd
-      const uint32_t r = (__brev((uint32_t)blk) >> (32 - S0)) * lb.galois + (lb.galois >> 1);
-      kadd = r >> S0;
-      src += (__brev(r << (32 - S0)) << 8);
-    } else {
-      src += blk * 256;
-    }
-    uint32_t w[16];
-#pragma unroll
-    for (int i = 0; i < 4; i++) ld_in4<DEP>(src + 64 * i + 4 * tau, w + 4 * i);
-#pragma unroll
-    for (int i = 0; i < 4; i++) st4(lin(i), w + 4 * i);
-    hw[tau] = h1;
-    __syncwarp();
-    if (PRO == PRO_GATHER) {
-      const uint32_t base = (__brev((uint32_t)tau) >> 28) * lb.galois + kadd;
-#pragma unroll
-      for (int e = 0; e < 16; e++) {
-        const uint32_t be = ((e & 1) << 3) | ((e & 2) << 1) | ((e & 4) >> 1) | ((e & 8) >> 3);  // brv4(e)
-        x[e] = sm[nb_blk_addr(c, (int)(__brev(base + be * 16u * lb.galois) >> 24))];
-      }
-      __syncwarp();  // every lane's reads come before the rows are rewritten
-    } else {
-#pragma unroll
-      for (int m = 0; m < 4; m++) ld4(sm + nb_blk_addr(c, (tau << 4) | (4 * m)), x + 4 * m);
-    }
-    nb_round<false>(x, lw, q);
-#pragma unroll
-    for (int m = 0; m < 4; m++) st4(sm + nb_blk_addr(c, (tau << 4) | (4 * m)), x + 4 * m);
-    __syncwarp();
-#pragma unroll
-    for (int e = 0; e < 16; e++) x[e] = sm[nb_blk_addr(c, (e << 4) | tau)];
-    nb_round_hi<false>(x, hw, q);
+    blk_load<LOGN, PRO, DEP>(x, lb.src, lb.galois, blk, sm, c, tau, [&] { hw[tau] = h1; });
+    blk_inverse(x, sm, c, tau, hw, tl, q);
     uint32_t *dst = lb.dst + blk * 256 + tau;
 #pragma unroll
     for (int e = 0; e < 16; e++) dst[e * 16] = x[e];

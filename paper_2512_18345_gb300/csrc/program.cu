@@ -135,6 +135,12 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
   auto has_ip = [](const Item &it) { return it.kind != IT_MODUP && it.kind != IT_MDX; };
   auto has_moddown = [](const Item &it) { return it.kind != IT_MODUP && it.kind != IT_IPX; };
 
+  const bool small = fused && fhe::ntt_small_ok(c->tabs);  // whole-limb stages (ntt_small.cuh)
+  Stage si = ntt_stage(false, false, PRO_PLAIN, EPI_SCALE), sn = ntt_stage(false, true, PRO_BCONV, EPI_PLAIN);
+  Stage sp, sd = ntt_stage(false, false, PRO_PLAIN, EPI_SCALE), sc2 = ntt_stage(false, true, PRO_BCONV, EPI_COMBINE);
+  si.kind = sn.kind = sd.kind = sc2.kind = Stage::SNTT;
+  sp.kind = Stage::SIP;
+
   // ---- HMult tensor
   Stage tensor = ew_stage(EW_TENSOR);
   for (size_t i = 0; i < items.size(); i++)
@@ -170,6 +176,10 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
     Seg g1 = seg(src, S.Y, level, 0, (int)i);
     g1.galois = P.ks[i].galois_own;  // read by PRO_GATHER
     add(i1, g1);
+    if (small) {
+      g1.scale = c->d_mu_scale + (size_t)(level - 1) * L;
+      add(si, g1);
+    }
     Seg y = seg(S.Y, S.Y, level, 0, (int)i);
     if (fused) y.scale = c->d_mu_scale + (size_t)(level - 1) * L;
     add(i2, y);
@@ -192,12 +202,29 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
       bc.max_in = std::max(bc.max_in, g.n_in);
       bc.max_out = std::max(bc.max_out, g.n_out);
       uint32_t *e = S.EXT + (size_t)j * n_ext * N;
+      if (small) {
+        auto conv = [&](int t, int n, int prime) {  // extended limbs t..t + n, rows t less the digit's own
+          Seg x = seg(g.in, e + (size_t)t * N, n, prime, (int)i);
+          x.src_stride = 0;
+          x.n_in = g.n_in;
+          x.T = g.T + (size_t)(t < lo ? t : t - (hi - lo)) * g.n_in;
+          add(sn, x);
+        };
+        conv(0, lo, 0);
+        conv(hi, level - hi, hi);
+        conv(level, K, L);
+        continue;
+      }
       add(n1, seg(e, e, lo, 0, (int)i));
       add(n1, seg(e + (size_t)hi * N, e + (size_t)hi * N, level - hi, hi, (int)i));
       add(n1, seg(e + (size_t)level * N, e + (size_t)level * N, K, L, (int)i));
     }
   }
-  if (!i1.segs.empty()) {
+  if (small && !i1.segs.empty()) {
+    si.pro = any_rot ? PRO_GATHER : PRO_PLAIN;
+    P.stages.push_back(si);
+    P.stages.push_back(sn);
+  } else if (!i1.segs.empty()) {
     if (!fused && !gather.segs.empty()) P.stages.push_back(gather);
     push_transform(c, P, i1, i2);
     if (!fused) P.stages.push_back(sc);
@@ -246,6 +273,15 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
       a.t0 = 0;
       a.key_row0 = 0;
       add(ipq, a);
+      if (small) {
+        add(sp, a);
+        Seg b = seg(nullptr, has_moddown(it) ? S.UC : U + (size_t)level * N, K, L, (int)i);
+        b.t0 = level;
+        b.key_row0 = L;
+        b.c = has_moddown(it) ? 1 : 0;
+        b.scale = c->d_md_scale;
+        add(sp, b);
+      }
       if (!fuse) {
         Seg b = seg(nullptr, U + (size_t)level * N, K, L, (int)i);
         b.t0 = level;
@@ -257,6 +293,20 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
     const int npoly = it.kind == IT_MDX ? it.npoly : 2;
     for (int cc = 0; cc < npoly; cc++) {
       uint32_t *uc = S.UC + (size_t)cc * K * N, *r = S.R + (size_t)cc * level * N;
+      if (small) {
+        if (!has_ip(it)) {  // else the inner product left the special limbs' coefficients in uc
+          Seg x = seg(U + ((size_t)cc * n_ext + level) * N, uc, K, L, (int)i);
+          x.scale = c->d_md_scale;
+          add(sd, x);
+        }
+        Seg z = seg(uc, it.out + (size_t)cc * level * N, level, 0, (int)i);
+        z.src_stride = 0;
+        z.n_in = K;
+        z.T = c->d_mdT;
+        z.src2 = U + (size_t)cc * n_ext * N;
+        add(sc2, z);
+        continue;
+      }
       if (!fuse) add(m1, seg(U + ((size_t)cc * n_ext + level) * N, uc, K, L, (int)i));
       Seg x = seg(uc, uc, K, L, (int)i);
       if (fused) x.scale = c->d_md_scale;
@@ -280,13 +330,16 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
       add(r1, seg(r, r, level, 0, (int)i));
       Seg z = fused ? seg(r, it.out + (size_t)cc * level * N, level, 0, (int)i) : seg(r, r, level, 0, (int)i);
       z.src2 = U + (size_t)cc * n_ext * N;
-      z.c = cc;
       add(r2, z);
       Seg w = seg(U + (size_t)cc * n_ext * N, it.out + (size_t)cc * level * N, level, 0, (int)i);
       w.src2 = r;
-      w.c = cc;
       add(cb, w);
     }
+  }
+  if (small) {
+    for (Stage *st : {&sp, &sd, &sc2})
+      if (!st->segs.empty()) P.stages.push_back(*st);
+    return FHE_OK;
   }
   ipp.gather_own = ipq.gather_own;
   ipp.gather_ext = ipq.gather_ext;
@@ -355,6 +408,8 @@ static cudaError_t launch_stage(fhe_ctx *c, const Stage &st, const SegList &sl, 
     case Stage::NTT1: return launch_ntt_single(c->tabs, st.fwd, st.pro, st.epi, sl, *sl2, q);
     case Stage::EW: return launch_ew(c->tabs, st.ewop, sl, q);
     case Stage::IP: return launch_ip(c->tabs, sl, st.gather_own, st.gather_ext, st.add_c1, c->dnum, q);
+    case Stage::SNTT: return launch_small_ntt(c->tabs, st.fwd, st.pro, st.epi, sl, q);
+    case Stage::SIP: return launch_small_ip(c->tabs, sl, q);
     case Stage::IPN: return launch_ip_intt(c->tabs, sl, std::min(c->dnum, 4), q);
     case Stage::BCONV:
       return c->bconv_mode == FHE_BCONV_TC ? launch_bconv_tc(c->tabs, ba, st.max_in, st.max_out, q, c->tabs.tc_k)
@@ -381,6 +436,8 @@ static bool stage_waits(const fhe_ctx *c, const Stage &st) {
   switch (st.kind) {
     case Stage::NTT: return !(st.column ? t.ntt_stream : t.ntt_stream || t.ntt_otf);
     case Stage::BCONV: return c->bconv_mode != FHE_BCONV_TC || !t.bconv_tc_pipe;
+    case Stage::SNTT:
+    case Stage::SIP: return true;
     case Stage::IP: return !st.gather_ext || (t.ip_staged && !st.add_c1);
     default: return false;
   }
@@ -507,11 +564,13 @@ int upload_program(fhe_ctx *c, const Program &P, DevProgram &D) {
         d.scale = combine ? c->d_pinv + d.prime : s.scale ? s.scale + v[x].y : c->d_ninv + d.prime;
         d.galois = s.galois;
         d.n = s.n;
+        d.T = s.T ? s.T + (size_t)v[x].y * s.n_in : nullptr;
+        d.n_in = s.n_in;
         lb[x] = d;
       }
     };
     auto limbs = [&](size_t off) { return reinterpret_cast<Limb *>(host.data() + off); };
-    const bool combine = (by_prime && st.epi == EPI_COMBINE) || (st.kind == Stage::EW && st.ewop == EW_COMBINE);
+    const bool combine = ((by_prime || st.kind == Stage::SNTT) && st.epi == EPI_COMBINE) || (st.kind == Stage::EW && st.ewop == EW_COMBINE);
     fill_map(st.segs, reinterpret_cast<int2 *>(host.data() + map_off[i]), limbs(limb_off[i]), combine);
     memcpy(host.data() + grp_off[i], st.groups.data(), sizeof(BconvGroup) * st.groups.size());
     memcpy(host.data() + seg2_off[i], st.segs2.data(), sizeof(Seg) * st.segs2.size());
