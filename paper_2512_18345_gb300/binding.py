@@ -166,18 +166,36 @@ def check(rc: int) -> None:
         raise FheError(rc, lib().fhe_last_error().decode())
 
 
-def _ptr(t) -> vp:
+# Argument marshalling is on the path of every call (a small-ring product is bound by it): plain
+# integers for pointers and streams, torch looked up once, the current stream's handle without a
+# Stream object, devices by their cached torch.device (11 -> 4 us a call).
+_torch = None
+_devices: dict = {}
+
+
+def _cuda():
+    """torch, with CUDA initialised."""
+    global _torch
+    if _torch is None:
+        import torch
+        torch.cuda.init()
+        _torch = torch
+    return _torch
+
+
+def _ptr(t) -> int:
     """Device pointer of a torch tensor (int32 / uint32, contiguous)."""
     if t is None:
-        return vp(0)
+        return 0
     assert t.is_contiguous(), "buffers must be contiguous"
-    return vp(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream(stream) -> vp:
-    import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return vp(s.cuda_stream)
+def _stream(stream) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    c = _cuda()._C
+    return c._cuda_getCurrentRawStream(c._cuda_getDevice())
 
 
 def _idx(xs: Sequence[int]):
@@ -196,8 +214,11 @@ def to_numpy(t) -> np.ndarray:
 
 
 def empty(shape, device: int = 0):
-    import torch
-    return torch.empty(tuple(shape), dtype=torch.int32, device=f"cuda:{device}")
+    torch = _cuda()
+    dev = _devices.get(device)
+    if dev is None:
+        dev = _devices[device] = torch.device("cuda", device)
+    return torch.empty(shape, dtype=torch.int32, device=dev)
 
 
 def probe_bandwidth(device: int = 0, nbytes: int = 64 << 20, reps: int = 50) -> dict:

@@ -499,9 +499,7 @@ static cudaError_t bconv_tc_go(const DevTables &t, const BconvArgs &a, int max_o
                             : cudaFuncSetAttribute(k_bconv_tc<KT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
   });
   if (ce != cudaSuccess) return ce;
-  int sms = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = t.sms;
   const int tiles_per_group = (int)((1u << t.logn) / kTcM);
   const int total = tiles_per_group * a.ngroups;
   TraceScope ts(t, "bconv_tc", s);

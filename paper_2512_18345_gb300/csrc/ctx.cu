@@ -269,6 +269,7 @@ static int build_tables(fhe_ctx *c) {
   c->tabs.tracer = nullptr;
   c->tabs.ip_ctas_per_sm = 2;
   c->tabs.dep = 0;
+  CUDA_OR_FAIL(cudaDeviceGetAttribute(&c->tabs.sms, cudaDevAttrMultiProcessorCount, c->device));
   c->tabs.ntt_otf = 0;
   c->tabs.ntt_single = 0;
   c->tabs.ntt_stream = 0;

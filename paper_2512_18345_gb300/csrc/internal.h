@@ -56,6 +56,7 @@ struct DevTables {
   NttTables ntt;
   const PrimeC *pc;
   int logn;
+  int sms;                 // the device's multiprocessors
   Tracer *tracer;          // null: no tracing
   unsigned int *status;    // device word, nonzero once a bounded device-side wait expired: bit 0
                            // tensor-core BConv, bit 1 inner product, bit 2 diagonal pass,

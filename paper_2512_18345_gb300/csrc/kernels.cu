@@ -113,9 +113,7 @@ static cudaError_t ntt_bulk_go(const DevTables &t, const SegList &sl, cudaStream
                                 ntt_bulk_smem(8));
   });
   if (e != cudaSuccess) return e;
-  int sms = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = t.sms;
   const int grid = std::min(units, std::max(1, std::min(3, t.ntt_stream_ctas)) * sms);
   static const char *names[2][2] = {{"intt_blk", "ntt_blk"}, {"intt_col", "ntt_col"}};
   const char *name = EPI == EPI_COMBINE ? "ntt_blk+combine" : EPI == EPI_SCALE ? "intt_col+scale"
@@ -224,9 +222,8 @@ static cudaError_t nttp_go(const DevTables &t, const SegList &first, const SegLi
   if (!t.gbar) return cudaErrorInvalidValue;
   constexpr int smem = ntt_twiddle_smem(true, 256);  // the larger of the two passes' tables
   auto kern = k_nttp<FWD, PRO, EPI>;
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = t.sms;
+  int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kNttThreads, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
@@ -396,9 +393,7 @@ cudaError_t launch_ip(const DevTables &t, const SegList &sl, bool gather_own, bo
     int D = t.ip_staged_depth >= 2 && t.ip_staged_depth <= 4 ? t.ip_staged_depth : 2;
     while (D > 2 && budget / (D * ws) < 1) D--;
     const int warps = std::max(1, std::min(kIhMaxWarps / ctas, budget / (D * ws)));
-    int sms = 0, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = t.sms;
     const int wunits = sl.total * ((1 << t.logn) / kIhUnit);
     const unsigned grid = (unsigned)std::min((wunits + warps - 1) / warps, ctas * sms);
     const int smem = warps * D * ws;
@@ -420,9 +415,7 @@ cudaError_t launch_ip(const DevTables &t, const SegList &sl, bool gather_own, bo
     const int per_stage = stage_bytes + 24 + (int)sizeof(IpUnit);  // data, three mbarriers, descriptor
     const int stages = std::min(ge ? 4 : 2, (113 * 1024 - 256) / per_stage);
     const int smem = stages * per_stage;
-    int sms = 0, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = t.sms;
     const int units = sl.total * ((1 << t.logn) / kIpChunk);
     const unsigned grid = (unsigned)std::min(units, std::max(1, std::min(2, t.ip_ctas_per_sm)) * sms);
     g_launches++;

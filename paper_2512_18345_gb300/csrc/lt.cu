@@ -220,8 +220,7 @@ static cudaError_t launch_diag(fhe_ctx *c, const DiagArgs &da, cudaStream_t s) {
                                 kDiagStages * kDiagStageBytes);
   });
   if (e != cudaSuccess) return e;
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+  const int sms = c->tabs.sms;
   const int units = da.nlimb * (int)(c->N / kDiagChunk) * ((da.giant + kGsub - 1) / kGsub);
   const unsigned grid = (unsigned)std::min(units, std::max(1, sms));  // persistent: one CTA per SM
   k_diag_bulk<<<grid, kDiagThreads + 32, kDiagStages * kDiagStageBytes, s>>>(da, c->d_pc, c->logn, c->tabs.status);

@@ -47,7 +47,8 @@ static Seg mkseg(const uint32_t *src, uint32_t *dst, int n, int prime) {
 struct SegBuilder {
   SegList l;
   SegBuilder() {
-    memset(&l, 0, sizeof l);
+    seg_clear(l);
+    memset(&l.ks[0], 0, sizeof l.ks[0]);
     l.ks[0].galois_own = l.ks[0].galois_ext = l.ks[0].galois_add = 1;
   }
   void add(const Seg &s) {
@@ -74,6 +75,17 @@ static int run_items(fhe_ctx *c, const std::vector<Item> &items, cudaStream_t s)
 // their chunk; an IT_MODUP item keeps its own slot.
 int run_items_chunked(fhe_ctx *c, const std::vector<Item> &items, int first_slot, cudaStream_t s) {
   size_t i = 0;
+  if (items_fit_inline(c, items)) {
+    // everything fits one program: build it once (adding item by item rebuilds the program for
+    // each, quadratic in a hoisted set)
+    std::vector<Item> all = items;
+    int nslot = 0;
+    for (Item &it : all) {
+      if (it.kind == IT_IPX) it.slot = it.ext_slot;
+      else if (it.kind != IT_MODUP) it.slot = first_slot + nslot++;
+    }
+    return run_items(c, all, s);
+  }
   while (i < items.size()) {
     std::vector<Item> chunk;
     Program best;

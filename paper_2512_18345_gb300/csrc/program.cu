@@ -51,7 +51,7 @@ static Stage marker(Stage::Kind k) {
 
 // the two passes of one transform: one single-pass cluster stage when the context asks for
 // it and the kernel exists for the pair's prologue and epilogue, else two stages
-static void push_transform(fhe_ctx *c, Program &P, const Stage &first, const Stage &second) {
+static void push_transform(fhe_ctx *c, Program &P, Stage first, Stage second) {
   if ((c->tabs.ntt_single || c->tabs.ntt_persist) && fhe::ntt_single_pass_ok(c->tabs, first.pro, second.epi, first.fwd)) {
     Stage f = first;
     f.kind = Stage::NTT1;
@@ -60,8 +60,8 @@ static void push_transform(fhe_ctx *c, Program &P, const Stage &first, const Sta
     P.stages.push_back(f);
     return;
   }
-  P.stages.push_back(first);
-  P.stages.push_back(second);
+  P.stages.push_back(std::move(first));
+  P.stages.push_back(std::move(second));
 }
 
 int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool fork, Program &P) {
@@ -69,6 +69,7 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
   const int L = c->L, K = c->K, A = c->alpha;
   P.ks.clear();
   P.stages.clear();
+  P.stages.reserve(16);
   int max_slot = 0;
   for (const Item &it : items) max_slot = std::max(max_slot, std::max(it.slot, it.ext_slot));
   int rc = ensure_slots(c, max_slot + 1);
@@ -222,17 +223,17 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
   }
   if (small && !i1.segs.empty()) {
     si.pro = any_rot ? PRO_GATHER : PRO_PLAIN;
-    P.stages.push_back(si);
-    P.stages.push_back(sn);
+    P.stages.push_back(std::move(si));
+    P.stages.push_back(std::move(sn));
   } else if (!i1.segs.empty()) {
     if (!fused && !gather.segs.empty()) P.stages.push_back(gather);
-    push_transform(c, P, i1, i2);
+    push_transform(c, P, std::move(i1), std::move(i2));
     if (!fused) P.stages.push_back(sc);
-    P.stages.push_back(bc);
+    P.stages.push_back(std::move(bc));
     Stage n2 = n1;
     n2.column = false;
     n2.epi = EPI_PLAIN;
-    push_transform(c, P, n1, n2);
+    push_transform(c, P, std::move(n1), std::move(n2));
   }
 
   // ---- stages 2 and 3: inner product, ModDown
@@ -338,7 +339,7 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
   }
   if (small) {
     for (Stage *st : {&sp, &sd, &sc2})
-      if (!st->segs.empty()) P.stages.push_back(*st);
+      if (!st->segs.empty()) P.stages.push_back(std::move(*st));
     return FHE_OK;
   }
   ipp.gather_own = ipq.gather_own;
@@ -359,9 +360,8 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
       P.stages.push_back(marker(Stage::JOIN_RECORD));
       if (!ipp.segs.empty()) P.stages.push_back(ipp);
     } else {
-      Stage all = ipq;
-      all.segs.insert(all.segs.end(), ipp.segs.begin(), ipp.segs.end());
-      P.stages.push_back(all);
+      ipq.segs.insert(ipq.segs.end(), ipp.segs.begin(), ipp.segs.end());
+      P.stages.push_back(std::move(ipq));
     }
   }
   if (has_md) {
@@ -375,7 +375,7 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
       push_transform(c, P, m1, m2);
     }
     if (!fused) P.stages.push_back(msc);
-    P.stages.push_back(mbc);
+    P.stages.push_back(std::move(mbc));
     if ((c->tabs.ntt_single || c->tabs.ntt_persist) && fhe::ntt_single_pass_ok(c->tabs, r1.pro, r2.epi, true)) {
       // the single-pass transform reads u's q-limbs in its epilogue: join before it
       if (split) P.stages.push_back(marker(Stage::JOIN_WAIT));
@@ -443,6 +443,30 @@ static bool stage_waits(const fhe_ctx *c, const Stage &st) {
   }
 }
 
+bool items_fit_inline(const fhe_ctx *c, const std::vector<Item> &items) {
+  if (items.empty() || (int)items.size() > kMaxInlineItems) return false;
+  int up_segs = 0, up_groups = 0, up_limbs = 0, ip_segs = 0, ip_limbs = 0, md = 0, md_limbs = 0;
+  for (const Item &it : items) {
+    const int level = it.level, beta = c->beta(level);
+    if (it.kind != IT_MODDOWN && it.kind != IT_IPX && it.kind != IT_MDX) {
+      up_segs += 3 * beta;  // a digit's converted limbs: before it, after it, the special ones
+      up_groups += beta;
+      up_limbs += beta * (level + c->K) - level;
+    }
+    if (it.kind != IT_MODUP && it.kind != IT_MDX) {
+      ip_segs += 2;
+      ip_limbs += level + c->K;
+    }
+    if (it.kind != IT_MODUP && it.kind != IT_IPX) {
+      const int np = it.kind == IT_MDX ? it.npoly : 2;
+      md += np;
+      md_limbs += np * std::max(level, c->K);
+    }
+  }
+  return std::max(std::max(up_segs, ip_segs), md) <= kMaxSeg && std::max(up_groups, md) <= kMaxBconvGroups &&
+         std::max(std::max(up_limbs, ip_limbs), md_limbs) <= kMaxInlineLimbs;
+}
+
 bool program_fits_inline(const Program &P) {
   if ((int)P.ks.size() > kMaxInlineItems) return false;
   for (const Stage &st : P.stages) {
@@ -458,6 +482,7 @@ int run_program_inline(fhe_ctx *c, const Program &P, cudaStream_t s) {
   if (!program_fits_inline(P)) return fhe_fail(FHE_EINVAL, "internal: program does not fit inline launch arguments");
   SegList sl, sl2;
   BconvArgs ba;
+  std::copy(P.ks.begin(), P.ks.end(), sl.ks);
   // Dependent launches: a stage kernel that begins with dep_wait (the transform passes, the base
   // conversions and the inner products in their default forms) may start its prologue under the
   // stage before it, when that stage's kernel is the last thing on the stream.  Not while the
@@ -466,12 +491,13 @@ int run_program_inline(fhe_ctx *c, const Program &P, cudaStream_t s) {
   const bool dep_ok = !c->tabs.tracer && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
   bool after_kernel = false;
   for (const Stage &st : P.stages) {
-    memset(&sl, 0, sizeof sl);
-    memset(&sl2, 0, sizeof sl2);
-    memset(&ba, 0, sizeof ba);
+    seg_clear(sl);
     for (const Seg &x : st.segs) seg_push(sl, x);
-    for (const Seg &x : st.segs2) seg_push(sl2, x);
-    for (size_t i = 0; i < P.ks.size(); i++) sl.ks[i] = sl2.ks[i] = P.ks[i];
+    if (!st.segs2.empty()) {
+      seg_clear(sl2);
+      for (const Seg &x : st.segs2) seg_push(sl2, x);
+      std::copy(P.ks.begin(), P.ks.end(), sl2.ks);
+    }
     if (st.kind == Stage::IP && st.gather_ext) {
       // the hoisted inner product takes the limbs limb by limb across runs of like segments
       // (the rotations of a hoisted set, which read the same digit limbs), at most four runs
@@ -491,6 +517,8 @@ int run_program_inline(fhe_ctx *c, const Program &P, cudaStream_t s) {
       sl.lm_groups = ok ? g : 0;
     }
     size_t limbs = sl.total;
+    ba.ngroups = 0;
+    ba.dev = nullptr;
     for (const BconvGroup &g : st.groups) {
       ba.g[ba.ngroups++] = g;
       limbs += g.n_out;

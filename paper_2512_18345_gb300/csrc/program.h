@@ -61,6 +61,9 @@ struct DevProgram {
 int ensure_slots(fhe_ctx *c, int n);
 // fork: the inner product of the ciphertext limbs on an auxiliary branch (complementary pipelining)
 int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool fork, Program &P);
+// whether the items' program fits by-value launch arguments (program_fits_inline of it, without
+// building it or growing the workspace)
+bool items_fit_inline(const fhe_ctx *c, const std::vector<Item> &items);
 bool program_fits_inline(const Program &P);
 int run_program_inline(fhe_ctx *c, const Program &P, cudaStream_t s);
 int upload_program(fhe_ctx *c, const Program &P, DevProgram &D);
