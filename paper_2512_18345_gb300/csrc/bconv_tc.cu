@@ -517,7 +517,7 @@ static cudaError_t bconv_tc_go(const DevTables &t, const BconvArgs &a, int max_o
     k_bconv_tc_pipe<KT><<<grid2, kTcThreads, smem2, s>>>(a, t.pc, t.logn, t.status, npad, tiles_per_group);
   } else {
     const int grid = std::min(total, std::max(1, sms * per_sm));
-    const cudaError_t le = launch_dep(t, t.dep ? k_bconv_tc<KT, true> : k_bconv_tc<KT, false>, grid, kTcThreads, smem, s, a, t.pc, t.logn, t.status, npad,
+    const cudaError_t le = launch_dep(t.dep, t.dep ? k_bconv_tc<KT, true> : k_bconv_tc<KT, false>, grid, kTcThreads, smem, s, a, t.pc, t.logn, t.status, npad,
                                       tiles_per_group);
     if (le != cudaSuccess) return le;
   }

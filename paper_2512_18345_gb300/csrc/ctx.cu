@@ -96,6 +96,11 @@ int fhe_ctx::beta(int level) const { return ceil_div(level, alpha); }
 int fhe_ctx::ext_prime(int level, int t) const { return t < level ? t : L + (t - level); }
 
 void fhe_ctx::order_stream(cudaStream_t s) {
+  // no dependent launches under tracing, nor while the caller captures, where forks and joins
+  // would mix with programmatic edges
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  after_kernel = false;
+  dep_ok = !capturing && !tabs.tracer && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
   if (capturing) return;
   if (have_last && s != last_stream) {
     cudaEventRecord(order_ev, last_stream);
@@ -269,6 +274,7 @@ static int build_tables(fhe_ctx *c) {
   c->tabs.tracer = nullptr;
   c->tabs.ip_ctas_per_sm = 2;
   c->tabs.dep = 0;
+  c->tabs.chain = 0;
   CUDA_OR_FAIL(cudaDeviceGetAttribute(&c->tabs.sms, cudaDevAttrMultiProcessorCount, c->device));
   c->tabs.ntt_otf = 0;
   c->tabs.ntt_single = 0;

@@ -96,6 +96,17 @@ struct fhe_ctx {
   std::vector<Lane> lanes;
   int batch_lanes = 2;
 
+  // Dependent launches within one call (common.cuh): order_stream, with which every call begins,
+  // says whether the stream allows them; a kernel may be one when the last thing the call put on
+  // the stream is a kernel and the launch is small.
+  bool dep_ok = false, after_kernel = false;
+  bool dep_next(size_t limbs) const { return dep_ok && after_kernel && (limbs << logn) <= kDepMaxWords; }
+  // Largest launch (coefficients) taken as a dependent one: with several waves of CTAs the ramp
+  // that a dependent launch hides is small beside the later waves' serialised prologues (256 limbs at
+  // N = 2^16; with no limit the dense transform took 1281 us instead of 1250, with 128 limbs 1257 us
+  // and one rotation at level 48 202.5 us instead of 198.9).
+  static constexpr size_t kDepMaxWords = (size_t)256 << 16;
+
   int beta(int level) const;
   int ext_prime(int level, int t) const;
   void order_stream(cudaStream_t s);

@@ -75,7 +75,8 @@ struct DevTables {
   int ip_staged;           // hoisted inner product: digits' permuted blocks staged (ip_hoisted.cuh)
   int ip_staged_ctas;      // resident CTAs per SM of that kernel (1 or 2)
   int ip_staged_depth;     // its stages per warp (2..4; 0: 2)
-  int dep;                 // the next launch is a dependent one (set stage by stage by run_program_inline)
+  int dep;                 // the next launch may be a dependent one (fhe_ctx::dep_next)
+  int chain;               // so may the further launches of a launch_ntt call
   int tc_k;                // K of the context's tensor-core BConv tables (48 or 64; 0: none)
 };
 
@@ -92,10 +93,10 @@ struct TraceScope {
 };
 void note_launch();
 
-// Launch a kernel that begins with dep_wait (common.cuh); with t.dep it may start while the
-// kernel before it on the stream is still running.
+// Launch a kernel; with `dep` (only for a kernel that begins with dep_wait, common.cuh) it may
+// start while the kernel before it on the stream is still running.
 template <class... P, class... A>
-cudaError_t launch_dep(const DevTables &t, void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s,
+cudaError_t launch_dep(bool dep, void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s,
                        const A &...args) {
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -106,7 +107,7 @@ cudaError_t launch_dep(const DevTables &t, void (*kern)(P...), dim3 grid, unsign
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = &attr;
-  cfg.numAttrs = t.dep ? 1 : 0;
+  cfg.numAttrs = dep ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 // the block passes' lo-round twiddles in thread order, from the bit-reversed table (legacy stream)

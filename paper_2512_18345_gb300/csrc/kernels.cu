@@ -78,7 +78,7 @@ static cudaError_t ntt_blk_go(const DevTables &t, const SegList &sl, cudaStream_
   if (grid == 0) return cudaSuccess;
   TraceScope ts(t, ntt_name<LOGN, false, FWD, PRO, EPI, false>(), s);
   g_launches++;
-  return launch_dep(t, t.dep ? k_ntt_blk<LOGN, FWD, PRO, EPI, true> : k_ntt_blk<LOGN, FWD, PRO, EPI, false>, grid, kNttThreads, 0, s, sl, t.ntt);
+  return launch_dep(t.dep, t.dep ? k_ntt_blk<LOGN, FWD, PRO, EPI, true> : k_ntt_blk<LOGN, FWD, PRO, EPI, false>, grid, kNttThreads, 0, s, sl, t.ntt);
 }
 
 // Column pass with warp-private twiddles (ntt_col.cuh).
@@ -88,7 +88,7 @@ static cudaError_t ntt_col_go(const DevTables &t, const SegList &sl, cudaStream_
   if (grid == 0) return cudaSuccess;
   TraceScope ts(t, ntt_name<LOGN, true, FWD, PRO, EPI, false>(), s);
   g_launches++;
-  return launch_dep(t, t.dep ? k_ntt_col<LOGN, FWD, PRO, EPI, true> : k_ntt_col<LOGN, FWD, PRO, EPI, false>, grid, kNttThreads, 0, s, sl, t.ntt);
+  return launch_dep(t.dep, t.dep ? k_ntt_col<LOGN, FWD, PRO, EPI, true> : k_ntt_col<LOGN, FWD, PRO, EPI, false>, grid, kNttThreads, 0, s, sl, t.ntt);
 }
 
 cudaError_t build_lo_table(const uint2 *tw, uint4 *lo, int logn, int nprimes) {
@@ -289,7 +289,7 @@ cudaError_t launch_small_ntt(const DevTables &t, bool fwd, int pro, int epi, con
   g_launches++;
 #define SMALL_FWD(P, E)              \
   if (fwd && pro == P && epi == E)   \
-    return launch_dep(t, t.dep ? k_small_ntt<P, E, true> : k_small_ntt<P, E, false>, sl.total, kNttThreads, 0, s, sl, t.ntt);
+    return launch_dep(t.dep, t.dep ? k_small_ntt<P, E, true> : k_small_ntt<P, E, false>, sl.total, kNttThreads, 0, s, sl, t.ntt);
   SMALL_FWD(PRO_PLAIN, EPI_PLAIN)
   SMALL_FWD(PRO_REDUCE, EPI_RESCALE)
   SMALL_FWD(PRO_BCONV, EPI_PLAIN)
@@ -297,10 +297,10 @@ cudaError_t launch_small_ntt(const DevTables &t, bool fwd, int pro, int epi, con
 #undef SMALL_FWD
   if (fwd || epi != EPI_SCALE) return cudaErrorInvalidValue;
   if (pro == PRO_PLAIN)
-    return launch_dep(t, t.dep ? k_small_intt<PRO_PLAIN, true> : k_small_intt<PRO_PLAIN, false>, sl.total, kNttThreads, 0, s,
+    return launch_dep(t.dep, t.dep ? k_small_intt<PRO_PLAIN, true> : k_small_intt<PRO_PLAIN, false>, sl.total, kNttThreads, 0, s,
                       sl, t.ntt);
   if (pro == PRO_GATHER)
-    return launch_dep(t, t.dep ? k_small_intt<PRO_GATHER, true> : k_small_intt<PRO_GATHER, false>, sl.total, kNttThreads, 0,
+    return launch_dep(t.dep, t.dep ? k_small_intt<PRO_GATHER, true> : k_small_intt<PRO_GATHER, false>, sl.total, kNttThreads, 0,
                       s, sl, t.ntt);
   return cudaErrorInvalidValue;
 }
@@ -309,7 +309,7 @@ cudaError_t launch_small_ip(const DevTables &t, const SegList &sl, cudaStream_t 
   if (sl.total == 0) return cudaSuccess;
   TraceScope ts(t, "small_ip", s);
   g_launches++;
-  return launch_dep(t, t.dep ? k_small_ip<true> : k_small_ip<false>, 2 * sl.total, kNttThreads, 0, s, sl, t.ntt);
+  return launch_dep(t.dep, t.dep ? k_small_ip<true> : k_small_ip<false>, 2 * sl.total, kNttThreads, 0, s, sl, t.ntt);
 }
 
 cudaError_t launch_ntt(const DevTables &t, bool fwd, int pro, int epi, const SegList &first, const SegList &second,
@@ -324,13 +324,15 @@ cudaError_t launch_ntt(const DevTables &t, bool fwd, int pro, int epi, const Seg
   }
   if ((t.ntt_single || t.ntt_persist) && ntt_single_pass_ok(t, pro, epi, fwd) && same_limbs(first, second))
     return launch_ntt_single(t, fwd, pro, epi, first, second, s);
+  DevTables t2 = t;
+  t2.dep = t.chain;
   cudaError_t e;
   if (fwd) {
     if ((e = launch_ntt_pass(t, true, true, pro, EPI_LAZY, first, s)) != cudaSuccess) return e;
-    return launch_ntt_pass(t, false, true, PRO_PLAIN, epi, second, s);
+    return launch_ntt_pass(t2, false, true, PRO_PLAIN, epi, second, s);
   }
   if ((e = launch_ntt_pass(t, false, false, pro, EPI_LAZY, first, s)) != cudaSuccess) return e;
-  return launch_ntt_pass(t, true, false, PRO_PLAIN, epi, second, s);
+  return launch_ntt_pass(t2, true, false, PRO_PLAIN, epi, second, s);
 }
 
 cudaError_t launch_bconv(const DevTables &t, const BconvArgs &a, int max_in, int max_out, cudaStream_t s) {
@@ -341,12 +343,12 @@ cudaError_t launch_bconv(const DevTables &t, const BconvArgs &a, int max_in, int
   g_launches++;
   switch (max_in) {
 #define BC(n) \
-  case n: return launch_dep(t, t.dep ? k_bconv<n, true> : k_bconv<n, false>, grid, kBconvThreads, 0, s, a, t.pc, t.logn);
+  case n: return launch_dep(t.dep, t.dep ? k_bconv<n, true> : k_bconv<n, false>, grid, kBconvThreads, 0, s, a, t.pc, t.logn);
     BC(1) BC(2) BC(3) BC(4) BC(5) BC(6) BC(7) BC(8)
 #undef BC
     default:
-      if (max_in <= 12) return launch_dep(t, t.dep ? k_bconv<12, true> : k_bconv<12, false>, grid, kBconvThreads, 0, s, a, t.pc, t.logn);
-      if (max_in <= 16) return launch_dep(t, t.dep ? k_bconv<16, true> : k_bconv<16, false>, grid, kBconvThreads, 0, s, a, t.pc, t.logn);
+      if (max_in <= 12) return launch_dep(t.dep, t.dep ? k_bconv<12, true> : k_bconv<12, false>, grid, kBconvThreads, 0, s, a, t.pc, t.logn);
+      if (max_in <= 16) return launch_dep(t.dep, t.dep ? k_bconv<16, true> : k_bconv<16, false>, grid, kBconvThreads, 0, s, a, t.pc, t.logn);
       return cudaErrorInvalidValue;
   }
 }
@@ -362,7 +364,7 @@ static cudaError_t ih_go(const DevTables &t, unsigned grid, unsigned block, int 
                              : cudaFuncSetAttribute(k_ip_hoisted<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
   });
   if (e != cudaSuccess) return e;
-  return launch_dep(t, t.dep ? k_ip_hoisted<D, true> : k_ip_hoisted<D, false>, grid, block, smem, s, sl, t.pc, t.logn,
+  return launch_dep(t.dep, t.dep ? k_ip_hoisted<D, true> : k_ip_hoisted<D, false>, grid, block, smem, s, sl, t.pc, t.logn,
                     beta_max);
 }
 
@@ -374,7 +376,7 @@ static cudaError_t ip_bulk_go(const DevTables &t, unsigned grid, int smem, cudaS
     return cudaFuncSetAttribute(k_ip_bulk<GOWN, GEXT, DEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024);
   });
   if (e != cudaSuccess) return e;
-  return launch_dep(t, k_ip_bulk<GOWN, GEXT, DEP>, grid, kIpThreads + 32, smem, s, sl, t.pc, t.logn, t.status, beta_max,
+  return launch_dep(DEP, k_ip_bulk<GOWN, GEXT, DEP>, grid, kIpThreads + 32, smem, s, sl, t.pc, t.logn, t.status, beta_max,
                     stages);
 }
 

@@ -69,6 +69,7 @@ constexpr int kDiagStageBytes = kDiagRows * kDiagChunk * 4 + 16;  // rows, two m
 constexpr int kDiagStages = 8;
 static_assert(kDiagStages * kDiagStageBytes <= 227 * 1024, "diagonal kernel: stages exceed shared memory");
 
+template <bool DEP>
 __global__ void __launch_bounds__(kDiagThreads + 32, 1) k_diag_bulk(const __grid_constant__ DiagArgs a, const PrimeC *pc,
                                                                    int logn, unsigned int *status) {
   constexpr int stages = kDiagStages;
@@ -104,6 +105,10 @@ __global__ void __launch_bounds__(kDiagThreads + 32, 1) k_diag_bulk(const __grid
   if (tid >= kDiagThreads) {  // the producer
     if (tid != kDiagThreads) return;
     const uint64_t once = l2_evict_first_policy();  // diagonals are read exactly once
+    if (DEP) {
+      dep_wait();
+      asm volatile("fence.proxy.async;" ::: "memory");  // bulk copies read what earlier kernels wrote
+    }
     int k = 0;
     for (int u = blockIdx.x; u < total; u += gridDim.x) {
       const int grp = u % groups, ch = (u / groups) % chunks, i = u / (groups * chunks);
@@ -134,6 +139,7 @@ __global__ void __launch_bounds__(kDiagThreads + 32, 1) k_diag_bulk(const __grid
     return;
   }
 
+  if (DEP) dep_wait();
   const int lane = tid & 31;
   bool ok = true;
   int k = 0;
@@ -216,16 +222,20 @@ __global__ void __launch_bounds__(kDiagThreads + 32, 1) k_diag_bulk(const __grid
 static cudaError_t launch_diag(fhe_ctx *c, const DiagArgs &da, cudaStream_t s) {
   static PerDeviceOnce configured;
   const cudaError_t e = configured.run([] {
-    return cudaFuncSetAttribute(k_diag_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                kDiagStages * kDiagStageBytes);
+    constexpr int kMax = kDiagStages * kDiagStageBytes;
+    const cudaError_t e0 = cudaFuncSetAttribute(k_diag_bulk<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
+    return e0 != cudaSuccess ? e0
+                             : cudaFuncSetAttribute(k_diag_bulk<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
   });
   if (e != cudaSuccess) return e;
   const int sms = c->tabs.sms;
   const int units = da.nlimb * (int)(c->N / kDiagChunk) * ((da.giant + kGsub - 1) / kGsub);
   const unsigned grid = (unsigned)std::min(units, std::max(1, sms));  // persistent: one CTA per SM
-  k_diag_bulk<<<grid, kDiagThreads + 32, kDiagStages * kDiagStageBytes, s>>>(da, c->d_pc, c->logn, c->tabs.status);
+  const bool dep = c->dep_next((size_t)2 * da.giant * da.nlimb);
   note_launch();
-  return cudaGetLastError();
+  c->after_kernel = true;
+  return launch_dep(dep, dep ? k_diag_bulk<true> : k_diag_bulk<false>, grid, kDiagThreads + 32,
+                    kDiagStages * kDiagStageBytes, s, da, c->d_pc, c->logn, c->tabs.status);
 }
 
 // The identity baby step of a double-hoisted transform, in the extended basis:
@@ -263,6 +273,7 @@ struct GsumArgs {
 // Four consecutive coefficients per thread: 16-byte loads and stores for every operand but
 // the sigma-gathered c0 halves.
 constexpr int kGsumEpt = 4;
+template <bool DEP>
 __global__ void __launch_bounds__(256) k_gsum(const __grid_constant__ GsumArgs a, const PrimeC *pc, int logn) {
   const size_t N = (size_t)1 << logn;
   const int per_limb = (int)(N / (256 * kGsumEpt));
@@ -272,12 +283,13 @@ __global__ void __launch_bounds__(256) k_gsum(const __grid_constant__ GsumArgs a
   const size_t poly = (size_t)a.nlimb * N, off = (size_t)i * N;
   uint32_t a0[kGsumEpt] = {}, a1[kGsumEpt] = {};
   auto add4 = [&](uint32_t (&acc)[kGsumEpt], const uint32_t *p) {
-    const uint4 w = __ldg(reinterpret_cast<const uint4 *>(p));
+    const uint4 w = ld_in4<DEP>(p);
     acc[0] = add_mod(acc[0], w.x, q);
     acc[1] = add_mod(acc[1], w.y, q);
     acc[2] = add_mod(acc[2], w.z, q);
     acc[3] = add_mod(acc[3], w.w, q);
   };
+  if (DEP) dep_wait();
   for (int g = 0; g < a.count; g++) {
     const uint32_t *in = a.inner[g] + off;
     if (!a.v[g]) {
@@ -285,7 +297,7 @@ __global__ void __launch_bounds__(256) k_gsum(const __grid_constant__ GsumArgs a
       add4(a1, in + poly + n);
     } else {
 #pragma unroll
-      for (int e = 0; e < kGsumEpt; e++) a0[e] = add_mod(a0[e], __ldg(in + galois_src(n + e, a.galois[g], logn)), q);
+      for (int e = 0; e < kGsumEpt; e++) a0[e] = add_mod(a0[e], ld_in<DEP>(in + galois_src(n + e, a.galois[g], logn)), q);
       add4(a0, a.v[g] + off + n);
       add4(a1, a.v[g] + poly + off + n);
     }
@@ -301,6 +313,7 @@ struct SumArgs {
   uint32_t *out;
   int count, level;
 };
+template <bool DEP>
 __global__ void __launch_bounds__(256) k_sum(const __grid_constant__ SumArgs a, const PrimeC *pc, int logn) {
   const size_t N = (size_t)1 << logn;
   const int per_limb = (int)(N / 1024);
@@ -308,11 +321,12 @@ __global__ void __launch_bounds__(256) k_sum(const __grid_constant__ SumArgs a, 
   const size_t n = (size_t)(blockIdx.x % per_limb) * 1024 + threadIdx.x * 4;
   const uint32_t q = pc[i].q;
   const size_t poly = (size_t)a.level * N;
+  if (DEP) dep_wait();
 #pragma unroll
   for (int c = 0; c < 2; c++) {
     uint32_t acc[4] = {0, 0, 0, 0};
     for (int g = 0; g < a.count; g++) {
-      const uint4 w = __ldg(reinterpret_cast<const uint4 *>(a.in[g] + c * poly + (size_t)i * N + n));
+      const uint4 w = ld_in4<DEP>(a.in[g] + c * poly + (size_t)i * N + n);
       acc[0] = add_mod(acc[0], w.x, q);
       acc[1] = add_mod(acc[1], w.y, q);
       acc[2] = add_mod(acc[2], w.z, q);
@@ -406,6 +420,7 @@ extern "C" int fhe_linear_transform(fhe_ctx *c, const uint32_t *ct, int level, c
       if (cudaMemcpyAsync(grot + g * ct_words, inner + g * ct_words, 4 * ct_words, cudaMemcpyDeviceToDevice, s) !=
           cudaSuccess)
         return fhe_fail(FHE_ECUDA, "fhe_linear_transform: copy");
+      c->after_kernel = false;
       continue;
     }
     Item it;
@@ -429,9 +444,12 @@ extern "C" int fhe_linear_transform(fhe_ctx *c, const uint32_t *ct, int level, c
   sa.level = level;
   {
     TraceScope ts(c->tabs, "lt_sum", s);
-    k_sum<<<(unsigned)(level * (N / 1024)), 256, 0, s>>>(sa, c->d_pc, c->logn);
+    const bool dep = c->dep_next((size_t)2 * level);
     note_launch();
-    if (cudaGetLastError() != cudaSuccess) return fhe_fail(FHE_ECUDA, "fhe_linear_transform: sum kernel");
+    c->after_kernel = true;
+    if (launch_dep(dep, dep ? k_sum<true> : k_sum<false>, (unsigned)(level * (N / 1024)), 256, 0, s, sa, c->d_pc, c->logn) !=
+        cudaSuccess)
+      return fhe_fail(FHE_ECUDA, "fhe_linear_transform: sum kernel");
   }
   return FHE_OK;
 }
@@ -499,6 +517,7 @@ extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level
       k_lift<<<grid_x / 4, 256, 0, s>>>(ct, bab + b * xct, c->d_pmod, c->d_pc, level, n_ext, c->logn);
       note_launch();
       if (cudaGetLastError() != cudaSuccess) return fhe_fail(FHE_ECUDA, "%s: lift kernel", fn);
+      c->after_kernel = true;
       continue;
     }
     Item it;
@@ -596,9 +615,11 @@ extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level
   ga.L = c->L;
   {
     TraceScope ts(c->tabs, "lt_gsum", s);
-    k_gsum<<<grid_x / kGsumEpt, 256, 0, s>>>(ga, c->d_pc, c->logn);
+    const bool dep = c->dep_next((size_t)2 * n_ext);
     note_launch();
-    if (cudaGetLastError() != cudaSuccess) return fhe_fail(FHE_ECUDA, "%s: giant-step sum kernel", fn);
+    c->after_kernel = true;
+    if (launch_dep(dep, dep ? k_gsum<true> : k_gsum<false>, grid_x / kGsumEpt, 256, 0, s, ga, c->d_pc, c->logn) != cudaSuccess)
+      return fhe_fail(FHE_ECUDA, "%s: giant-step sum kernel", fn);
   }
   Item fin;
   fin.kind = IT_MDX;

@@ -222,7 +222,10 @@ extern "C" int fhe_rescale(fhe_ctx *c, const uint32_t *ct, int level, uint32_t *
     f1.add(mkseg(ct + cc * poly + (size_t)(level - 1) * N, V + cc * N, 1, level - 1));
     f2.add(mkseg(V + cc * N, V + cc * N, 1, level - 1));
   }
-  LAUNCH_OR_FAIL(launch_ntt(c->tabs, false, PRO_PLAIN, EPI_SCALE, f1.l, f2.l, s));
+  DevTables t = c->tabs;  // the further launches depend on the ones before them
+  t.chain = c->dep_ok;
+  LAUNCH_OR_FAIL(launch_ntt(t, false, PRO_PLAIN, EPI_SCALE, f1.l, f2.l, s));
+  t.dep = c->dep_ok;
   for (int cc = 0; cc < 2; cc++) {
     uint32_t *o = out + (size_t)cc * (level - 1) * N;
     Seg a = mkseg(V + cc * N, o, level - 1, 0);
@@ -234,7 +237,7 @@ extern "C" int fhe_rescale(fhe_ctx *c, const uint32_t *ct, int level, uint32_t *
     b.scale = c->d_rs_qinv + (size_t)(level - 1) * c->L;
     g2.add(b);
   }
-  LAUNCH_OR_FAIL(launch_ntt(c->tabs, true, PRO_REDUCE, EPI_RESCALE, g1.l, g2.l, s));
+  LAUNCH_OR_FAIL(launch_ntt(t, true, PRO_REDUCE, EPI_RESCALE, g1.l, g2.l, s));
   return FHE_OK;
 }
 
@@ -373,16 +376,15 @@ extern "C" int fhe_modup(fhe_ctx *c, const uint32_t *d, int level, uint32_t *ext
   it.kind = IT_MODUP;
   it.level = level;
   it.in = d;
+  it.out = ext;
   it.slot = 0;
   CHECK(run_items(c, {it}, s));
-  if (cudaMemcpyAsync(ext, c->slots[0].EXT, 4 * N * (size_t)beta * n_ext, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-    return fhe_fail(FHE_ECUDA, "fhe_modup: copy");
+  SegBuilder own;  // the digits' own limbs
   for (int j = 0; j < beta; j++) {
     const int lo = j * c->alpha, hi = std::min((j + 1) * c->alpha, level);
-    if (cudaMemcpyAsync(ext + ((size_t)j * n_ext + lo) * N, d + (size_t)lo * N, 4 * N * (hi - lo),
-                        cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-      return fhe_fail(FHE_ECUDA, "fhe_modup: copy");
+    own.add(mkseg(d + (size_t)lo * N, ext + ((size_t)j * n_ext + lo) * N, hi - lo, lo));
   }
+  LAUNCH_OR_FAIL(launch_ew(c->tabs, EW_COPY, own.l, s));
   return FHE_OK;
 }
 
@@ -392,42 +394,17 @@ extern "C" int fhe_moddown(fhe_ctx *c, const uint32_t *u, int level, uint32_t *o
   CHECK(check_ptr(u, "fhe_moddown", "u"));
   CHECK(check_ptr(out, "fhe_moddown", "out"));
   const size_t N = c->N;
-  const int K = c->K, L = c->L;
-  if (overlaps(u, 4 * N * (level + K), out, 4 * N * level)) return fhe_fail(FHE_EALIAS, "fhe_moddown: out overlaps u");
+  if (overlaps(u, 4 * N * (level + c->K), out, 4 * N * level)) return fhe_fail(FHE_EALIAS, "fhe_moddown: out overlaps u");
   cudaSetDevice(c->device);
   cudaStream_t s = (cudaStream_t)stream;
   c->order_stream(s);
-  uint32_t *UC = c->slots[0].UC, *R = c->slots[0].R;
-  SegBuilder first, second, nr, cb;
-  first.add(mkseg(u + (size_t)level * N, UC, K, L));
-  Seg b = mkseg(UC, UC, K, L);
-  b.scale = c->d_md_scale;
-  second.add(b);
-  LAUNCH_OR_FAIL(launch_ntt(c->tabs, false, PRO_PLAIN, EPI_SCALE, first.l, second.l, s));
-  BconvArgs ba;
-  memset(&ba, 0, sizeof ba);
-  BconvGroup &g = ba.g[ba.ngroups++];
-  g.in = UC;
-  g.out = R;
-  g.T = c->d_mdT;
-  g.omap = c->d_mdmap;
-  g.n_in = K;
-  g.n_out = level;
-  g.Btc = c->d_md_Btc;
-  g.npad = tc_npad(level);
-  if (c->bconv_mode == FHE_BCONV_TC)
-    LAUNCH_OR_FAIL(launch_bconv_tc(c->tabs, ba, K, level, s, c->tabs.tc_k));
-  else
-    LAUNCH_OR_FAIL(launch_bconv(c->tabs, ba, K, level, s));
-  nr.add(mkseg(R, R, level, 0));
-  LAUNCH_OR_FAIL(launch_ntt(c->tabs, true, PRO_PLAIN, EPI_PLAIN, nr.l, nr.l, s));
-  Seg x = mkseg(u, out, level, 0);
-  x.src2 = R;
-  cb.add(x);
-  cb.l.ks[0].pinv = c->d_pinv;
-  cb.l.ks[0].level = level;
-  LAUNCH_OR_FAIL(launch_ew(c->tabs, EW_COMBINE, cb.l, s));
-  return FHE_OK;
+  Item it;
+  it.kind = IT_MDX;
+  it.level = level;
+  it.in = u;
+  it.out = out;
+  it.npoly = 1;
+  return run_items(c, {it}, s);
 }
 
 // The tables of one fhe_bconv combination (input primes, output primes, kernel): the
@@ -554,6 +531,7 @@ extern "C" int fhe_bconv(fhe_ctx *c, const uint32_t *in, const int *in_idx, int 
       sb.add(x);
     }
     if (launch_ew(c->tabs, EW_SCALE, sb.l, s) != cudaSuccess) return fhe_fail(FHE_ECUDA, "fhe_bconv: scale");
+    c->after_kernel = true;
   }
   BconvArgs ba;
   memset(&ba, 0, sizeof ba);
@@ -566,7 +544,9 @@ extern "C" int fhe_bconv(fhe_ctx *c, const uint32_t *in, const int *in_idx, int 
   g.n_out = n_out;
   g.Btc = prep.Btc;
   g.npad = tc_npad(n_out);
-  const cudaError_t e = tc ? launch_bconv_tc(c->tabs, ba, n_in, n_out, s, kt) : launch_bconv(c->tabs, ba, n_in, n_out, s);
+  DevTables t = c->tabs;
+  t.dep = c->dep_next(n_out);
+  const cudaError_t e = tc ? launch_bconv_tc(t, ba, n_in, n_out, s, kt) : launch_bconv(t, ba, n_in, n_out, s);
   if (e != cudaSuccess) return fhe_fail(FHE_ECUDA, "fhe_bconv: %s", cudaGetErrorString(e));
   return FHE_OK;
 }

@@ -110,6 +110,7 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
         break;
       case IT_MODUP:  // `in` is the polynomial itself
         dpoly[i] = it.in;
+        if (it.out) k.ext = it.out;
         break;
       case IT_MODDOWN:
         k.ext = c->slots[it.ext_slot].EXT;
@@ -168,6 +169,7 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
     const fhe_ctx::Slot &S = c->slots[it.slot];
     const int level = it.level, n_ext = level + K, beta = c->beta(level);
     const uint32_t *src = dpoly[i];
+    uint32_t *EXT = it.kind == IT_MODUP && it.out ? it.out : S.EXT;
     if (!fused && it.kind == IT_ROTATE && it.galois != 1u) {
       Seg gs = seg(src, S.TMP, level, 0, (int)i);
       gs.galois = it.galois;
@@ -192,7 +194,7 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
       BconvGroup g;
       memset(&g, 0, sizeof g);
       g.in = S.Y + (size_t)lo * N;
-      g.out = S.EXT + (size_t)j * n_ext * N;
+      g.out = EXT + (size_t)j * n_ext * N;
       g.T = c->modup_T[(size_t)(level - 1) * c->dnum + j];
       g.omap = c->modup_map[(size_t)(level - 1) * c->dnum + j];
       g.n_in = hi - lo;
@@ -202,7 +204,7 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
       bc.groups.push_back(g);
       bc.max_in = std::max(bc.max_in, g.n_in);
       bc.max_out = std::max(bc.max_out, g.n_out);
-      uint32_t *e = S.EXT + (size_t)j * n_ext * N;
+      uint32_t *e = EXT + (size_t)j * n_ext * N;
       if (small) {
         auto conv = [&](int t, int n, int prime) {  // extended limbs t..t + n, rows t less the digit's own
           Seg x = seg(g.in, e + (size_t)t * N, n, prime, (int)i);
@@ -424,25 +426,6 @@ static cudaError_t launch_stage(fhe_ctx *c, const Stage &st, const SegList &sl, 
   return cudaErrorInvalidValue;
 }
 
-// Largest launch (coefficients) taken as a dependent one: with several waves of CTAs the ramp
-// that a dependent launch hides is small beside the later waves' serialised prologues (256 limbs at
-// N = 2^16; with no limit the dense transform took 1281 us instead of 1250, with 128 limbs 1257 us
-// and one rotation at level 48 202.5 us instead of 198.9).
-static constexpr size_t kDepMaxWords = (size_t)256 << 16;
-
-// whether a stage's kernel begins with dep_wait (and so may be launched as a dependent one)
-static bool stage_waits(const fhe_ctx *c, const Stage &st) {
-  const DevTables &t = c->tabs;
-  switch (st.kind) {
-    case Stage::NTT: return !(st.column ? t.ntt_stream : t.ntt_stream || t.ntt_otf);
-    case Stage::BCONV: return c->bconv_mode != FHE_BCONV_TC || !t.bconv_tc_pipe;
-    case Stage::SNTT:
-    case Stage::SIP: return true;
-    case Stage::IP: return !st.gather_ext || (t.ip_staged && !st.add_c1);
-    default: return false;
-  }
-}
-
 bool items_fit_inline(const fhe_ctx *c, const std::vector<Item> &items) {
   if (items.empty() || (int)items.size() > kMaxInlineItems) return false;
   int up_segs = 0, up_groups = 0, up_limbs = 0, ip_segs = 0, ip_limbs = 0, md = 0, md_limbs = 0;
@@ -483,13 +466,6 @@ int run_program_inline(fhe_ctx *c, const Program &P, cudaStream_t s) {
   SegList sl, sl2;
   BconvArgs ba;
   std::copy(P.ks.begin(), P.ks.end(), sl.ks);
-  // Dependent launches: a stage kernel that begins with dep_wait (the transform passes, the base
-  // conversions and the inner products in their default forms) may start its prologue under the
-  // stage before it, when that stage's kernel is the last thing on the stream.  Not while the
-  // caller captures, where forks and joins would mix with programmatic edges, nor under tracing.
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  const bool dep_ok = !c->tabs.tracer && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
-  bool after_kernel = false;
   for (const Stage &st : P.stages) {
     seg_clear(sl);
     for (const Seg &x : st.segs) seg_push(sl, x);
@@ -524,11 +500,11 @@ int run_program_inline(fhe_ctx *c, const Program &P, cudaStream_t s) {
       limbs += g.n_out;
     }
     ba.lazy = 1;  // every conversion of a program feeds a forward NTT
-    const bool kernel = st.kind != Stage::FORK && st.kind != Stage::JOIN_RECORD && st.kind != Stage::JOIN_WAIT;
-    c->tabs.dep = dep_ok && after_kernel && !st.aux && (limbs << c->logn) <= kDepMaxWords && stage_waits(c, st);
+    // (a program run here has one stream: no forks, no auxiliary stages)
+    c->tabs.dep = c->dep_next(limbs);
     cudaError_t e = launch_stage(c, st, sl, ba, s, 0, &sl2);
     c->tabs.dep = 0;
-    after_kernel = kernel && !st.aux;
+    c->after_kernel = true;
     if (e != cudaSuccess) return fhe_fail(FHE_ECUDA, "stage launch: %s", cudaGetErrorString(e));
   }
   return FHE_OK;

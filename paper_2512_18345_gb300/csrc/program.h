@@ -21,7 +21,7 @@ struct Item {
   const uint32_t *in = nullptr;    // KS / MODUP: d [level][N]; ROTATE / MODDOWN: ct [2][level][N]; RELIN: a;
                                    // IPX: the polynomial that was ModUp'ed [level][N]; MDX: [npoly][level+K][N]
   const uint32_t *in2 = nullptr;   // RELIN: b; IPX: pass-through c0 [level][N] or null
-  uint32_t *out = nullptr;         // [2][level][N] (not for MODUP)
+  uint32_t *out = nullptr;         // [2][level][N]; MODUP: [beta][level+K][N], or null (the slot's)
   const uint32_t *key = nullptr;   // switching key (not for MODUP)
   int slot = 0;                    // workspace slot of this item
   int ext_slot = 0;                // MODDOWN / IPX: slot whose EXT holds the shared ModUp output

@@ -35,6 +35,7 @@ def calls(ctx, level, a, b):
     out = [ctx.rotate(a, level, 5), ctx.keyswitch(a[0].contiguous(), level), ctx.hmult(a, b, level)]
     out += ctx.rotate_hoisted(a, level, [1, 0, 2])
     out += [ctx.modup(a[1].contiguous(), level)]
+    out += [ctx.moddown(out[-1][0].contiguous(), level), ctx.bconv(a[0, :1].contiguous(), [0], list(range(1, ctx.L + ctx.K)))]
     return out + ([ctx.rescale(out[2], level)] if level > 1 else [])
 
 
