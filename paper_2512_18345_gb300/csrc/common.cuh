@@ -127,6 +127,8 @@ struct KsArgs {
   const uint32_t *key;   // [dnum][2][L+K][N]
   const uint32_t *addp;  // [2][level][N] pass-through polynomial (c = 0, 1) of the output, or null; the
                          // inner product adds P * addp to u's q-limbs, so ModDown's (u - r) P^-1 carries it
+  const uint32_t *mul_a, *mul_b;  // HMult's factors [2][level][N] when the tensor product is formed on the fly
+                         // (own limbs a1 b1, pass-through (a0 b0, a0 b1 + a1 b0)), else null
   const uint2 *pinv;     // [L] Shoup pairs of P^-1 mod q_i
   const uint2 *pmod;     // [L] Shoup pairs of P mod q_i
   int level, n_ext, beta, alpha, L, K;

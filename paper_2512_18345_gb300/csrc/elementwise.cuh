@@ -15,7 +15,6 @@ constexpr int kEwThreads = 256;
 enum : int {
   EW_GATHER = 0,   // dst = src[sigma(j)]               (galois = seg.galois)
   EW_SCALE = 1,    // dst = src * scale[l]
-  EW_IP = 2,       // (k_ip) both halves of the key inner product
   EW_COMBINE = 3,  // dst = (src - src2) P^-1  (src = u, src2 = NTT(r))
   EW_ADD = 4,      // dst = src + src2
   EW_MUL = 5,      // dst = src * src2
@@ -82,80 +81,21 @@ __global__ void __launch_bounds__(kEwThreads) k_ew(const __grid_constant__ SegLi
   *reinterpret_cast<uint4 *>(dst + j0) = make_uint4(o[0], o[1], o[2], o[3]);
 }
 
-// Stage 2: the key inner product for a run of extended limbs, both halves at
-// once (each ModUp value is read once):
+// Stage 2: the key inner product for a run of extended limbs, both halves at once (each ModUp
+// value is read once):
 //   u_c[t][n] = sum_{j < beta} E_j[t][n] key[j][c][row(t)][n] mod prime(t),
 // E_j[t] = own[t] (read through sigma_{galois_own}) when t is one of digit j's
 // q-limbs, else ext[j][t] (read through sigma_{galois_ext}).  seg.dst points
 // at u_0[t0]; u_1 sits n_ext limbs further.  beta <= 4, so the four 62-bit
 // products of a sum fit one 64-bit accumulator.
-template <bool GOWN, bool GEXT>
-__global__ void __launch_bounds__(kEwThreads) k_ip(const __grid_constant__ SegList sl, const PrimeC *pc, int logn) {
-  const size_t N = (size_t)1 << logn;
-  const int blocks_per_limb = (int)(N / (4 * kEwThreads));
-  const int v = blockIdx.x / blocks_per_limb;
-  const uint32_t j0 = (uint32_t)((blockIdx.x % blocks_per_limb) * 4 * kEwThreads + threadIdx.x * 4);
-  int within;
-  const Seg &sg = seg_at(sl, seg_find(sl, v, within));
-  const KsArgs &ks = item_ks(sl, sg);
-  const int t = sg.t0 + within, row = sg.key_row0 + within;
-  const PrimeC P = pc[sg.prime + within];
-  const size_t kstride = (size_t)2 * (ks.L + ks.K) * N;
-  // issue every digit's loads before any arithmetic (memory-level parallelism)
-  uint4 ev[4], kv0[4], kv1[4];
-#pragma unroll
-  for (int jd = 0; jd < 4; jd++) {
-    if (jd < ks.beta) {
-      const bool own = t < ks.level && t >= jd * ks.alpha && t < (jd + 1) * ks.alpha;
-      const uint32_t *p = own ? ks.own + (size_t)t * N : ks.ext + ((size_t)jd * ks.n_ext + t) * N;
-      if ((own && GOWN) || (!own && GEXT)) {
-        const uint32_t g = own ? ks.galois_own : ks.galois_ext;
-        ev[jd] = make_uint4(__ldg(p + galois_src(j0, g, logn)), __ldg(p + galois_src(j0 + 1, g, logn)),
-                            __ldg(p + galois_src(j0 + 2, g, logn)), __ldg(p + galois_src(j0 + 3, g, logn)));
-      } else {
-        ev[jd] = __ldg(reinterpret_cast<const uint4 *>(p + j0));
-      }
-      const uint32_t *kp = ks.key + jd * kstride + (size_t)row * N + j0;
-      kv0[jd] = __ldg(reinterpret_cast<const uint4 *>(kp));
-      kv1[jd] = __ldg(reinterpret_cast<const uint4 *>(kp + (size_t)(ks.L + ks.K) * N));
-    } else {
-      ev[jd] = kv0[jd] = kv1[jd] = make_uint4(0, 0, 0, 0);
-    }
-  }
-  uint64_t a0[4] = {0, 0, 0, 0}, a1[4] = {0, 0, 0, 0};
-#pragma unroll
-  for (int jd = 0; jd < 4; jd++) {
-    const uint32_t e4[4] = {ev[jd].x, ev[jd].y, ev[jd].z, ev[jd].w};
-    const uint32_t k0[4] = {kv0[jd].x, kv0[jd].y, kv0[jd].z, kv0[jd].w};
-    const uint32_t k1[4] = {kv1[jd].x, kv1[jd].y, kv1[jd].z, kv1[jd].w};
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-      a0[i] += (uint64_t)e4[i] * k0[i];
-      a1[i] += (uint64_t)e4[i] * k1[i];
-    }
-  }
-  uint32_t r0[4], r1[4];
-#pragma unroll
-  for (int i = 0; i < 4; i++) {
-    r0[i] = reduce_u64(a0[i], P);
-    r1[i] = reduce_u64(a1[i], P);
-  }
-  if (ks.addp && t < ks.level) {  // pass-through term: u_c += P * addp_c (c = 0; c = 1 for HMult)
-    const uint2 pm = ks.pmod[t];
-    const uint32_t *ap = ks.addp + (size_t)t * N;
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-      const uint32_t ja = ks.galois_add == 1u ? j0 + i : galois_src(j0 + i, ks.galois_add, logn);
-      r0[i] = add_mod(r0[i], shoup(__ldg(ap + ja), pm.x, pm.y, P.q), P.q);
-      if (ks.add_c1) r1[i] = add_mod(r1[i], shoup(__ldg(ap + (size_t)ks.level * N + ja), pm.x, pm.y, P.q), P.q);
-    }
-  }
-  uint32_t *d0 = sg.dst + (size_t)within * N + j0, *d1 = d0 + (size_t)ks.n_ext * N;
-  *reinterpret_cast<uint4 *>(d0) = make_uint4(r0[0], r0[1], r0[2], r0[3]);
-  *reinterpret_cast<uint4 *>(d1) = make_uint4(r1[0], r1[1], r1[2], r1[3]);
-}
-
-// Stage 2 as a persistent streaming kernel (the ext limbs are read in order).
+//
+// HMult (MUL: some item multiplies on the fly): the tensor product is never stored.  Its d2 =
+// a1 b1 is formed in the inverse transform's loads and again here for the own digit, d0 = a0 b0
+// and d1 = a0 b1 + a1 b0 here for the pass-through term, from the factors' four rows loaded one
+// unit ahead: 6 l limb rows in all instead of the tensor kernel's 7 l and 4 l reads of its
+// output.
+//
+// A persistent streaming kernel (the ext limbs are read in order).
 // A unit is kIpChunk coefficients of one extended limb.  A producer warp (one
 // lane) streams each unit's operands -- per digit the ModUp value (ext, or the
 // own limb when it is not read through an automorphism) and both key halves,
@@ -201,12 +141,13 @@ struct IpUnit {            // one unit, as the consumers need it
   uint2 pm;                // P mod the unit's prime (Shoup pair)
   uint32_t d1_off, galois, j0, galois_add, add1_off;
   int beta, gjd, add1;
+  int mul;                 // HMult on the fly: add0 = a0, gsrc = b0 (a1, b1 add1_off further)
 };
 
 // GEXT (hoisted rotations: the ModUp digits themselves are read through the
 // automorphism): only the key chunks stream through the stages; every digit's values
 // are gathered with plain loads one unit ahead (the shared digits stay in L2).
-template <bool GOWN, bool GEXT, bool DEP>
+template <bool GOWN, bool GEXT, bool MUL, bool DEP>
 __global__ void __launch_bounds__(kIpThreads + 32, 2) k_ip_bulk(const __grid_constant__ SegList sl, const PrimeC *pc,
                                                            int logn, unsigned int *status, int beta_max, int stages) {
   extern __shared__ __align__(128) uint8_t smem[];
@@ -240,8 +181,9 @@ __global__ void __launch_bounds__(kIpThreads + 32, 2) k_ip_bulk(const __grid_con
     d.d1_off = (uint32_t)((size_t)ks.n_ext * N);
     d.P = pc[sg.prime + within];
     d.beta = ks.beta;
-    d.gjd = (GOWN && !GEXT && t < ks.level) ? t / ks.alpha : -1;
-    d.gsrc = d.gjd >= 0 ? ks.own + (size_t)t * N : nullptr;
+    d.mul = MUL && ks.mul_a && t < ks.level;
+    d.gjd = ((GOWN || d.mul) && !GEXT && t < ks.level) ? t / ks.alpha : -1;
+    d.gsrc = d.mul ? ks.mul_b + (size_t)t * N : d.gjd >= 0 ? ks.own + (size_t)t * N : nullptr;
     if (GEXT)
       for (int jd = 0; jd < 4; jd++) {
         const bool own = t < ks.level && t >= jd * ks.alpha && t < (jd + 1) * ks.alpha;
@@ -250,9 +192,9 @@ __global__ void __launch_bounds__(kIpThreads + 32, 2) k_ip_bulk(const __grid_con
       }
     d.galois = ks.galois_own;
     d.j0 = (uint32_t)c0;
-    const bool add = ks.addp && t < ks.level;
-    d.add0 = add ? ks.addp + (size_t)t * N : nullptr;
-    d.add1 = add && ks.add_c1;
+    const bool add = d.mul || (ks.addp && t < ks.level);
+    d.add0 = d.mul ? ks.mul_a + (size_t)t * N : add ? ks.addp + (size_t)t * N : nullptr;
+    d.add1 = d.mul || (add && ks.add_c1);
     d.add1_off = (uint32_t)((size_t)ks.level * N);
     d.galois_add = ks.galois_add;
     d.pm = add ? ks.pmod[t] : make_uint2(0, 0);
@@ -315,9 +257,19 @@ __global__ void __launch_bounds__(kIpThreads + 32, 2) k_ip_bulk(const __grid_con
 #pragma unroll
     for (int e = 0; e < E; e++) v[e] = __ldg(d.gsrc + galois_src(j + e, d.galois, logn));
   };
-  // pass-through values of a unit (read through sigma_{galois_add}), also one unit ahead
-  auto pass = [&](const IpUnit &d, uint32_t (&p0)[E], uint32_t (&p1)[E]) {
+  // pass-through values of a unit (read through sigma_{galois_add}), also one unit ahead; for an
+  // HMult the factors: p0, p1 = a0, a1 and m0, m1 = b0, b1
+  constexpr int M = MUL ? E : 1;
+  auto pass = [&](const IpUnit &d, uint32_t (&p0)[E], uint32_t (&p1)[E], uint32_t (&m0)[M], uint32_t (&m1)[M]) {
     const uint32_t j = d.j0 + tid * E;
+    if constexpr (MUL)
+      if (d.mul) {
+        ld_in4<false>(d.add0 + j, p0);
+        ld_in4<false>(d.add0 + d.add1_off + j, p1);
+        ld_in4<false>(d.gsrc + j, m0);
+        ld_in4<false>(d.gsrc + d.add1_off + j, m1);
+        return;
+      }
     if (d.galois_add == 1u) {
       // (HMult's tensor: written by this program's first kernel)
       ld_in4<DEP>(d.add0 + j, p0);
@@ -339,22 +291,24 @@ __global__ void __launch_bounds__(kIpThreads + 32, 2) k_ip_bulk(const __grid_con
   };
   // every consumer thread waits on the barriers itself (bounded; a warp gives up as a whole)
   if (DEP) dep_wait();
-  uint32_t gnext[E] = {}, pnext0[E] = {}, pnext1[E] = {}, xnext[XD][E] = {};
+  uint32_t gnext[E] = {}, pnext0[E] = {}, pnext1[E] = {}, xnext[XD][E] = {}, mnext0[M] = {}, mnext1[M] = {};
   bool ok = true;
   if ((int)blockIdx.x < total) {
     ok = __all_sync(0xffffffffu, mbar_wait_bounded(&dbar[0], 0u));
     if (ok) {
-      if (GOWN && desc[0].gjd >= 0) gather(desc[0], gnext);
+      if (GOWN && desc[0].gjd >= 0 && !(MUL && desc[0].mul)) gather(desc[0], gnext);
       if (GEXT) gather_all(desc[0], xnext);
-      if (desc[0].add0) pass(desc[0], pnext0, pnext1);
+      if (desc[0].add0) pass(desc[0], pnext0, pnext1, mnext0, mnext1);
     }
   }
   int k = 0;
   for (int u = blockIdx.x; ok && u < total; u += gridDim.x, k++) {
     const int st = k % stages;
-    uint32_t gv[E], pv0[E], pv1[E], xv[XD][E];
+    uint32_t gv[E], pv0[E], pv1[E], xv[XD][E], mv0[M], mv1[M];
 #pragma unroll
     for (int e = 0; e < E; e++) gv[e] = gnext[e], pv0[e] = pnext0[e], pv1[e] = pnext1[e];
+#pragma unroll
+    for (int e = 0; e < M; e++) mv0[e] = mnext0[e], mv1[e] = mnext1[e];
 #pragma unroll
     for (int jd = 0; jd < XD; jd++)
 #pragma unroll
@@ -367,10 +321,20 @@ __global__ void __launch_bounds__(kIpThreads + 32, 2) k_ip_bulk(const __grid_con
     const IpUnit d = desc[st];
     if (has_next) {  // the next unit's descriptor (its readiness was waited for above)
       const IpUnit dn = desc[(k + 1) % stages];
-      if (GOWN && dn.gjd >= 0) gather(dn, gnext);
+      if (GOWN && dn.gjd >= 0 && !(MUL && dn.mul)) gather(dn, gnext);
       if (GEXT) gather_all(dn, xnext);
-      if (dn.add0) pass(dn, pnext0, pnext1);
+      if (dn.add0) pass(dn, pnext0, pnext1, mnext0, mnext1);
     }
+    if constexpr (MUL)
+      if (d.mul) {  // (d2, and (d0, d1) in the pass-through's place)
+#pragma unroll
+        for (int e = 0; e < E; e++) {
+          gv[e] = mul_mod(pv1[e], mv1[e], d.P);
+          const uint64_t d1 = (uint64_t)pv0[e] * mv1[e] + (uint64_t)pv1[e] * mv0[e];  // < 2^63
+          pv0[e] = mul_mod(pv0[e], mv0[e], d.P);
+          pv1[e] = reduce_u64(d1, d.P);
+        }
+      }
     const uint32_t *src = buf + (size_t)st * stage_words + tid * E;
     uint64_t a0[E] = {}, a1[E] = {};
 #pragma unroll

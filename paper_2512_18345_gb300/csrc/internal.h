@@ -135,14 +135,15 @@ int ntt_single_pass_clusters();
 // its source and prologue from sl and writes its destination and epilogue in one launch
 bool ntt_small_ok(const DevTables &t);
 cudaError_t launch_small_ntt(const DevTables &t, bool fwd, int pro, int epi, const SegList &sl, cudaStream_t s);
-cudaError_t launch_small_ip(const DevTables &t, const SegList &sl, cudaStream_t s);
+cudaError_t launch_small_ip(const DevTables &t, const SegList &sl, bool mul, cudaStream_t s);
 cudaError_t launch_bconv(const DevTables &t, const BconvArgs &a, int max_in, int max_out, cudaStream_t s);
 // kt: the K of the groups' tables (48: max_in <= 8; 64: max_in <= 12)
 cudaError_t launch_bconv_tc(const DevTables &t, const BconvArgs &a, int max_in, int max_out, cudaStream_t s, int kt);
 cudaError_t launch_ew(const DevTables &t, int op, const SegList &sl, cudaStream_t s);
 // key inner product (both halves) for the ext limbs of sl; seg.dst = u_0[t0]
 // beta_max: the largest digit count among the segments' items (sizes the stages)
-cudaError_t launch_ip(const DevTables &t, const SegList &sl, bool gather_own, bool gather_ext, bool add_c1, int beta_max,
+// mul: some item forms its tensor product on the fly (KsArgs::mul_a)
+cudaError_t launch_ip(const DevTables &t, const SegList &sl, bool gather_own, bool gather_ext, bool add_c1, bool mul, int beta_max,
                       cudaStream_t s);
 // the special limbs' inner product fused with ModDown's first inverse-NTT pass (ip_intt.cuh);
 // sl: one segment per item over its K special limbs, dst = the item's UC [2][K][N]

@@ -42,7 +42,7 @@ void note_launch() { g_launches++; }
 
 template <int LOGN, bool COLUMN, bool FWD, int PRO, int EPI, bool OTF>
 static const char *ntt_name() {
-  static const char *pro[] = {"", "+gather", "+reduce"};
+  static const char *pro[] = {"", "+gather", "+reduce", "+bconv", "+mul"};
   static const char *epi[] = {"", "", "+scale", "+combine", "+rescale"};
   static const std::string name = [] {  // initialised once, thread-safe
     char buf[64];
@@ -154,6 +154,7 @@ static cudaError_t ntt_dispatch(const DevTables &t, bool column, bool fwd, int p
   NTT_CASE(false, false, PRO_GATHER, EPI_LAZY)
   NTT_CASE(true, false, PRO_PLAIN, EPI_SCALE)
 #undef NTT_CASE
+  if (!column && !fwd && pro == PRO_MUL && epi == EPI_LAZY) return ntt_blk_go<LOGN, false, PRO_MUL, EPI_LAZY>(t, sl, s);
   return cudaErrorInvalidValue;
 }
 
@@ -302,14 +303,19 @@ cudaError_t launch_small_ntt(const DevTables &t, bool fwd, int pro, int epi, con
   if (pro == PRO_GATHER)
     return launch_dep(t.dep, t.dep ? k_small_intt<PRO_GATHER, true> : k_small_intt<PRO_GATHER, false>, sl.total, kNttThreads, 0,
                       s, sl, t.ntt);
+  if (pro == PRO_MUL)
+    return launch_dep(t.dep, t.dep ? k_small_intt<PRO_MUL, true> : k_small_intt<PRO_MUL, false>, sl.total, kNttThreads, 0, s,
+                      sl, t.ntt);
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_small_ip(const DevTables &t, const SegList &sl, cudaStream_t s) {
+cudaError_t launch_small_ip(const DevTables &t, const SegList &sl, bool mul, cudaStream_t s) {
   if (sl.total == 0) return cudaSuccess;
   TraceScope ts(t, "small_ip", s);
   g_launches++;
-  return launch_dep(t.dep, t.dep ? k_small_ip<true> : k_small_ip<false>, 2 * sl.total, kNttThreads, 0, s, sl, t.ntt);
+  return launch_dep(t.dep, mul ? (t.dep ? k_small_ip<true, true> : k_small_ip<true, false>)
+                               : (t.dep ? k_small_ip<false, true> : k_small_ip<false, false>),
+                    2 * sl.total, kNttThreads, 0, s, sl, t.ntt);
 }
 
 cudaError_t launch_ntt(const DevTables &t, bool fwd, int pro, int epi, const SegList &first, const SegList &second,
@@ -368,19 +374,19 @@ static cudaError_t ih_go(const DevTables &t, unsigned grid, unsigned block, int 
                     beta_max);
 }
 
-template <bool GOWN, bool GEXT, bool DEP>
+template <bool GOWN, bool GEXT, bool MUL, bool DEP>
 static cudaError_t ip_bulk_go(const DevTables &t, unsigned grid, int smem, cudaStream_t s, const SegList &sl, int beta_max,
                               int stages) {
   static PerDeviceOnce configured;
   const cudaError_t e = configured.run([] {
-    return cudaFuncSetAttribute(k_ip_bulk<GOWN, GEXT, DEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024);
+    return cudaFuncSetAttribute(k_ip_bulk<GOWN, GEXT, MUL, DEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024);
   });
   if (e != cudaSuccess) return e;
-  return launch_dep(DEP, k_ip_bulk<GOWN, GEXT, DEP>, grid, kIpThreads + 32, smem, s, sl, t.pc, t.logn, t.status, beta_max,
+  return launch_dep(DEP, k_ip_bulk<GOWN, GEXT, MUL, DEP>, grid, kIpThreads + 32, smem, s, sl, t.pc, t.logn, t.status, beta_max,
                     stages);
 }
 
-cudaError_t launch_ip(const DevTables &t, const SegList &sl, bool gather_own, bool gather_ext, bool add_c1,
+cudaError_t launch_ip(const DevTables &t, const SegList &sl, bool gather_own, bool gather_ext, bool add_c1, bool mul,
                       int beta_max, cudaStream_t s) {
   if (sl.total == 0) return cudaSuccess;
   TraceScope ts(t, "inner_product", s);
@@ -421,29 +427,23 @@ cudaError_t launch_ip(const DevTables &t, const SegList &sl, bool gather_own, bo
     const int units = sl.total * ((1 << t.logn) / kIpChunk);
     const unsigned grid = (unsigned)std::min(units, std::max(1, std::min(2, t.ip_ctas_per_sm)) * sms);
     g_launches++;
-    if (go && ge) return ip_bulk_go<true, true, false>(t, grid, smem, s, sl, beta_max, stages);
-    if (ge) return ip_bulk_go<false, true, false>(t, grid, smem, s, sl, beta_max, stages);
-    if (go)
-      return t.dep ? ip_bulk_go<true, false, true>(t, grid, smem, s, sl, beta_max, stages)
-                   : ip_bulk_go<true, false, false>(t, grid, smem, s, sl, beta_max, stages);
-    return t.dep ? ip_bulk_go<false, false, true>(t, grid, smem, s, sl, beta_max, stages)
-                 : ip_bulk_go<false, false, false>(t, grid, smem, s, sl, beta_max, stages);
+    // (single HMults take MUL with DEP; a plan mixes them with rotations)
+#define IP_GO(GO, GE, MU, DE) ip_bulk_go<GO, GE, MU, DE>(t, grid, smem, s, sl, beta_max, stages)
+    if (ge) return go ? IP_GO(true, true, false, false) : IP_GO(false, true, false, false);
+    if (mul && go) return IP_GO(true, false, true, false);
+    if (mul) return t.dep ? IP_GO(false, false, true, true) : IP_GO(false, false, true, false);
+    if (go) return t.dep ? IP_GO(true, false, false, true) : IP_GO(true, false, false, false);
+    return t.dep ? IP_GO(false, false, false, true) : IP_GO(false, false, false, false);
+#undef IP_GO
   }
-  const unsigned per_limb = (unsigned)((1u << t.logn) / (4 * kEwThreads));
-  const unsigned grid = (unsigned)sl.total * per_limb;
-  if (go && ge) k_ip<true, true><<<grid, kEwThreads, 0, s>>>(sl, t.pc, t.logn);
-  else if (go) k_ip<true, false><<<grid, kEwThreads, 0, s>>>(sl, t.pc, t.logn);
-  else if (ge) k_ip<false, true><<<grid, kEwThreads, 0, s>>>(sl, t.pc, t.logn);
-  else k_ip<false, false><<<grid, kEwThreads, 0, s>>>(sl, t.pc, t.logn);
-  g_launches++;
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;  // (contexts have at most four digits)
 }
 
 cudaError_t launch_ew(const DevTables &t, int op, const SegList &sl, cudaStream_t s) {
   const unsigned per_limb = (unsigned)((1u << t.logn) / (4 * kEwThreads));
   const unsigned grid = (unsigned)sl.total * per_limb;
   if (grid == 0) return cudaSuccess;
-  static const char *names[] = {"ew_gather", "ew_scale", "ew_ip", "ew_combine", "ew_add", "ew_mul", "ew_copy",
+  static const char *names[] = {"ew_gather", "ew_scale", "ew", "ew_combine", "ew_add", "ew_mul", "ew_copy",
                                 "tensor"};
   TraceScope ts(t, op >= 0 && op < 8 ? names[op] : "ew", s);
   switch (op) {

@@ -46,6 +46,7 @@ enum : int {
   PRO_GATHER = 1,  // src[sigma(j)], sigma = the limb's galois (NTT form input)
   PRO_REDUCE = 2,  // src[j] reduced from another prime (rescale: src_prime)
   PRO_BCONV = 3,   // base conversion of n_in limbs at src (small ring)
+  PRO_MUL = 4,     // src[j] src2[j] where the limb has a src2 (HMult's d2), else as PRO_GATHER
 };
 // Epilogue modes (how the last pass writes an element)
 enum : int {

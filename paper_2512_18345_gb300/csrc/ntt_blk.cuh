@@ -176,11 +176,14 @@ __device__ __forceinline__ void blk_store(const Limb &lb, int blk, uint32_t *sm,
 // the inverse's input: block blk (PRO_GATHER: read through sigma_galois) into lo layout
 // (element 16 tau + e); `staged` runs once the loads are on their way
 template <int LOGN, int PRO, bool DEP, class F>
-__device__ __forceinline__ void blk_load(uint32_t (&x)[16], const uint32_t *src, uint32_t galois, int blk, uint32_t *sm,
-                                         int c, int tau, F staged) {
+__device__ __forceinline__ void blk_load(uint32_t (&x)[16], const Limb &lb, const PrimeC &P, int blk, uint32_t *sm, int c,
+                                         int tau, F staged) {
   constexpr int S0 = LOGN - 8;
+  constexpr bool GATHER = PRO == PRO_GATHER || PRO == PRO_MUL;
+  const uint32_t *src = lb.src;
+  const uint32_t galois = lb.galois;
   uint32_t kadd = 0;
-  if (PRO == PRO_GATHER) {
+  if (GATHER) {
     // index blk 256 + k has brv = brv8(k) 2^S0 + brv(blk); times g plus g >> 1, its low S0
     // bits give the source block and the rest brv8 of the source element: brv8(k) g + kadd
     const uint32_t r = (__brev((uint32_t)blk) >> (32 - S0)) * galois + (galois >> 1);
@@ -192,11 +195,20 @@ __device__ __forceinline__ void blk_load(uint32_t (&x)[16], const uint32_t *src,
   uint32_t w[16];
 #pragma unroll
   for (int i = 0; i < 4; i++) ld_in4<DEP>(src + 64 * i + 4 * tau, w + 4 * i);
+  if (PRO == PRO_MUL && lb.src2) {  // (uniform per limb; such a limb has galois 1)
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      uint32_t w2[4];
+      ld_in4<DEP>(lb.src2 + blk * 256 + 64 * i + 4 * tau, w2);
+#pragma unroll
+      for (int e = 0; e < 4; e++) w[4 * i + e] = mul_mod(w[4 * i + e], w2[e], P);
+    }
+  }
 #pragma unroll
   for (int i = 0; i < 4; i++) st4(blk_lin(sm, c, tau, i), w + 4 * i);
   staged();
   __syncwarp();
-  if (PRO == PRO_GATHER) {
+  if (PRO == PRO_GATHER || (PRO == PRO_MUL && galois != 1u)) {
     const uint32_t base = (__brev((uint32_t)tau) >> 28) * galois + kadd;
 #pragma unroll
     for (int e = 0; e < 16; e++) {
@@ -221,18 +233,19 @@ __device__ __forceinline__ void blk_inverse(uint32_t (&x)[16], uint32_t *sm, int
   nb_round_hi<false>(x, hw, q);
 }
 
-// Forward: PRO_PLAIN with EPI_PLAIN, EPI_COMBINE or EPI_RESCALE; inverse: PRO_PLAIN or
-// PRO_GATHER with EPI_LAZY.  Residency: 48 registers (16 values, 30 of twiddles), five CTAs
+// Forward: PRO_PLAIN with EPI_PLAIN, EPI_COMBINE or EPI_RESCALE; inverse: PRO_PLAIN,
+// PRO_GATHER or PRO_MUL with EPI_LAZY.  Residency: 48 registers (16 values, 30 of twiddles), five CTAs
 // (four and six, and loading the lo twiddles after the hi round: within 1 % or slower).
 template <int LOGN, bool FWD, int PRO, int EPI, bool DEP>
-__global__ void __launch_bounds__(kNttThreads, DEP && FWD ? 4 : 5) k_ntt_blk(const __grid_constant__ SegList sl, const NttTables tb) {
+__global__ void __launch_bounds__(kNttThreads, (DEP && FWD) || PRO == PRO_MUL ? 4 : 5) k_ntt_blk(const __grid_constant__ SegList sl, const NttTables tb) {
   constexpr int TILES = (1 << LOGN) / kTile;
   __shared__ __align__(16) uint32_t sm[16 * 272];
   __shared__ __align__(16) uint2 hws[16 * 16];
   const int tid = threadIdx.x, c = tid >> 4, tau = tid & 15;
   const int v = blockIdx.x / TILES, tile = blockIdx.x % TILES;
   const Limb lb = limb_at<EPI == EPI_COMBINE>(sl, v, tb.ninv, LOGN);
-  const uint32_t q = tb.pc[lb.prime].q;
+  const PrimeC P = tb.pc[lb.prime];
+  const uint32_t q = P.q;
   const int blk = tile * 16 + c;
   uint2 *hw = hws + c * 16;
   const uint2 h1 = blk_hi_twiddle<LOGN, FWD>(tb, lb.prime, blk, tau);
@@ -251,7 +264,7 @@ __global__ void __launch_bounds__(kNttThreads, DEP && FWD ? 4 : 5) k_ntt_blk(con
     if (EPI == EPI_COMBINE || EPI == EPI_RESCALE) scale = __ldg(lb.scale);
     blk_store<EPI, DEP>(lb, blk, sm, c, tau, scale, q);
   } else {
-    blk_load<LOGN, PRO, DEP>(x, lb.src, lb.galois, blk, sm, c, tau, [&] { hw[tau] = h1; });
+    blk_load<LOGN, PRO, DEP>(x, lb, P, blk, sm, c, tau, [&] { hw[tau] = h1; });
     blk_inverse(x, sm, c, tau, hw, tl, q);
     uint32_t *dst = lb.dst + blk * 256 + tau;
 #pragma unroll

@@ -6,7 +6,7 @@
 //   k_small_ntt   forward, from coefficients, from another prime's limb (rescale), or from the
 //                 base conversion of up to 16 limbs formed in the prologue; ending plain, in the
 //                 ModDown combine or in the rescale;
-//   k_small_intt  inverse (with the rotation's gather) and output scale;
+//   k_small_intt  inverse (with the rotation's gather, or of HMult's d2 = a1 b1) and output scale;
 //   k_small_ip    the key inner product of one extended limb and half; a special limb of a key
 //                 switch goes on to its inverse transform in the same CTA.
 // A key switch is then four launches (inverse, convert + forward, inner product + inverse,
@@ -46,11 +46,12 @@ __device__ __forceinline__ void small_inverse(uint32_t (&x)[16], SmallShared &s,
 }
 
 template <int PRO, bool DEP>
-__global__ void __launch_bounds__(kNttThreads, 4) k_small_intt(const __grid_constant__ SegList sl, const NttTables tb) {
+__global__ void __launch_bounds__(kNttThreads, PRO == PRO_MUL ? 3 : 4) k_small_intt(const __grid_constant__ SegList sl, const NttTables tb) {
   __shared__ SmallShared s;
   const int tid = threadIdx.x, c = tid >> 4, tau = tid & 15;
   const Limb lb = limb_at<false>(sl, blockIdx.x, tb.ninv, kSmallLogN);
-  const uint32_t q = tb.pc[lb.prime].q;
+  const PrimeC P = tb.pc[lb.prime];
+  const uint32_t q = P.q;
   const uint2 h1 = blk_hi_twiddle<kSmallLogN, false>(tb, lb.prime, c, tau);
   const uint2 h0 = __ldg(tb.tw_inv + ((size_t)lb.prime << kSmallLogN) + tau);
   const uint2 scale = __ldg(lb.scale);
@@ -58,7 +59,7 @@ __global__ void __launch_bounds__(kNttThreads, 4) k_small_intt(const __grid_cons
   load_lo_twiddles<kSmallLogN>(tb.lo_inv, lb.prime, 0, tid, tl);
   if (DEP) dep_wait();
   uint32_t x[16];
-  blk_load<kSmallLogN, PRO, DEP>(x, lb.src, lb.galois, c, s.sm, c, tau, [&] {
+  blk_load<kSmallLogN, PRO, DEP>(x, lb, P, c, s.sm, c, tau, [&] {
     s.hws[tid] = h1;
     if ((tid & 31) < 16) s.h0[tid >> 5][tau] = h0;
   });
@@ -118,7 +119,7 @@ __global__ void __launch_bounds__(kNttThreads, PRO == PRO_BCONV ? 2 : 4)
 // at 16 coefficients per thread in memory order.  seg.c = 1: a special limb of a key switch,
 // whose inverse transform follows (seg.dst = UC, halves K limbs apart, seg.scale its output
 // scale); else u is written (halves n_ext limbs apart).
-template <bool DEP>
+template <bool MUL, bool DEP>
 __global__ void __launch_bounds__(kNttThreads, 2) k_small_ip(const __grid_constant__ SegList sl, const NttTables tb) {
   constexpr int N = 1 << kSmallLogN;
   __shared__ SmallShared s;
@@ -154,7 +155,15 @@ __global__ void __launch_bounds__(kNttThreads, 2) k_small_ip(const __grid_consta
 #pragma unroll
     for (int i = 0; i < 4; i++) {
       uint32_t ev[4];
-      load(ep, own ? ks.galois_own : ks.galois_ext, i, ev);
+      if (MUL && own && ks.mul_a) {  // HMult's d2 = a1 b1
+        uint32_t w[4];
+        ld_in4<DEP>(ks.mul_a + (size_t)(ks.level + t) * N + at(i), ev);
+        ld_in4<DEP>(ks.mul_b + (size_t)(ks.level + t) * N + at(i), w);
+#pragma unroll
+        for (int e = 0; e < 4; e++) ev[e] = mul_mod(ev[e], w[e], P);
+      } else {
+        load(ep, own ? ks.galois_own : ks.galois_ext, i, ev);
+      }
       const uint4 kv = __ldg(reinterpret_cast<const uint4 *>(kp + at(i)));
       acc[4 * i] += (uint64_t)ev[0] * kv.x;
       acc[4 * i + 1] += (uint64_t)ev[1] * kv.y;
@@ -174,6 +183,25 @@ __global__ void __launch_bounds__(kNttThreads, 2) k_small_ip(const __grid_consta
       load(ap, ks.galois_add, i, w);
 #pragma unroll
       for (int e = 0; e < 4; e++) x[4 * i + e] = add_mod(x[4 * i + e], shoup(w[e], pm.x, pm.y, q), q);
+    }
+  }
+  if (MUL && ks.mul_a && t < ks.level) {  // HMult's d0 = a0 b0, d1 = a0 b1 + a1 b0
+    const uint2 pm = ks.pmod[t];
+    const size_t p0 = (size_t)t * N, p1 = (size_t)(ks.level + t) * N;
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      uint32_t a0[4], b0[4], a1[4], b1[4];
+      ld_in4<DEP>(ks.mul_a + p0 + at(i), a0);
+      ld_in4<DEP>(ks.mul_b + (cc ? p1 : p0) + at(i), b0);  // a0 b0, or a0 b1 ...
+      if (cc) {
+        ld_in4<DEP>(ks.mul_a + p1 + at(i), a1);
+        ld_in4<DEP>(ks.mul_b + p0 + at(i), b1);  // ... + a1 b0
+      }
+#pragma unroll
+      for (int e = 0; e < 4; e++) {
+        const uint64_t d = (uint64_t)a0[e] * b0[e] + (cc ? (uint64_t)a1[e] * b1[e] : 0);  // < 2^63
+        x[4 * i + e] = add_mod(x[4 * i + e], shoup(reduce_u64(d, P), pm.x, pm.y, q), q);
+      }
     }
   }
   uint32_t *dst = sg.dst + ((size_t)cc * (invert ? ks.K : ks.n_ext) + within) * N;

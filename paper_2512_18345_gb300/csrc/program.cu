@@ -70,6 +70,11 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
   P.ks.clear();
   P.stages.clear();
   P.stages.reserve(16);
+  const bool small = fused && fhe::ntt_small_ok(c->tabs);  // whole-limb stages (ntt_small.cuh)
+  // HMult's tensor product formed on the fly by its readers (PRO_MUL, the inner product), where
+  // the first transform is a default block pass or a whole-limb one; else by a kernel of its own
+  const DevTables &tb = c->tabs;
+  const bool mul = fused && (small || (c->logn == 16 && !tb.ntt_otf && !tb.ntt_single && !tb.ntt_stream && !tb.ntt_persist));
   int max_slot = 0;
   for (const Item &it : items) max_slot = std::max(max_slot, std::max(it.slot, it.ext_slot));
   int rc = ensure_slots(c, max_slot + 1);
@@ -104,6 +109,12 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
         k.addp = it.in;
         break;
       case IT_RELIN:
+        if (mul) {
+          dpoly[i] = it.in + poly;  // a1; times b1 where it is read
+          k.mul_a = it.in;
+          k.mul_b = it.in2;
+          break;
+        }
         dpoly[i] = S.D + 2 * poly;
         k.addp = S.D;
         k.add_c1 = 1;
@@ -137,7 +148,6 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
   auto has_ip = [](const Item &it) { return it.kind != IT_MODUP && it.kind != IT_MDX; };
   auto has_moddown = [](const Item &it) { return it.kind != IT_MODUP && it.kind != IT_IPX; };
 
-  const bool small = fused && fhe::ntt_small_ok(c->tabs);  // whole-limb stages (ntt_small.cuh)
   Stage si = ntt_stage(false, false, PRO_PLAIN, EPI_SCALE), sn = ntt_stage(false, true, PRO_BCONV, EPI_PLAIN);
   Stage sp, sd = ntt_stage(false, false, PRO_PLAIN, EPI_SCALE), sc2 = ntt_stage(false, true, PRO_BCONV, EPI_COMBINE);
   si.kind = sn.kind = sd.kind = sc2.kind = Stage::SNTT;
@@ -146,7 +156,7 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
   // ---- HMult tensor
   Stage tensor = ew_stage(EW_TENSOR);
   for (size_t i = 0; i < items.size(); i++)
-    if (items[i].kind == IT_RELIN) {
+    if (items[i].kind == IT_RELIN && !mul) {
       Seg s = seg(items[i].in, c->slots[items[i].slot].D, items[i].level, 0, (int)i);
       s.src2 = items[i].in2;
       add(tensor, s);
@@ -154,10 +164,14 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
   if (!tensor.segs.empty()) P.stages.push_back(tensor);
 
   // ---- stage 1: ModUp
-  bool any_rot = false;
-  for (const Item &it : items) any_rot |= has_modup(it) && it.kind == IT_ROTATE && it.galois != 1u;
+  bool any_rot = false, any_mul = false;
+  for (const Item &it : items) {
+    any_rot |= has_modup(it) && it.kind == IT_ROTATE && it.galois != 1u;
+    any_mul |= mul && it.kind == IT_RELIN;
+  }
+  const int pro = any_mul ? PRO_MUL : fused && any_rot ? PRO_GATHER : PRO_PLAIN;
   Stage gather = ew_stage(EW_GATHER);
-  Stage i1 = ntt_stage(false, false, (fused && any_rot) ? PRO_GATHER : PRO_PLAIN, EPI_LAZY);
+  Stage i1 = ntt_stage(false, false, pro, EPI_LAZY);
   Stage i2 = ntt_stage(true, false, PRO_PLAIN, EPI_SCALE);
   Stage sc = ew_stage(EW_SCALE);
   Stage bc;
@@ -177,7 +191,8 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
       src = S.TMP;
     }
     Seg g1 = seg(src, S.Y, level, 0, (int)i);
-    g1.galois = P.ks[i].galois_own;  // read by PRO_GATHER
+    g1.galois = P.ks[i].galois_own;  // read by PRO_GATHER and PRO_MUL
+    if (mul && it.kind == IT_RELIN) g1.src2 = it.in2 + (size_t)level * N;
     add(i1, g1);
     if (small) {
       g1.scale = c->d_mu_scale + (size_t)(level - 1) * L;
@@ -224,7 +239,7 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
     }
   }
   if (small && !i1.segs.empty()) {
-    si.pro = any_rot ? PRO_GATHER : PRO_PLAIN;
+    si.pro = pro;
     P.stages.push_back(std::move(si));
     P.stages.push_back(std::move(sn));
   } else if (!i1.segs.empty()) {
@@ -272,11 +287,13 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
       ipq.gather_own |= k.galois_own != 1u;
       ipq.gather_ext |= k.galois_ext != 1u;
       ipq.add_c1 |= k.addp && k.add_c1;
+      ipq.mul |= k.mul_a != nullptr;
       Seg a = seg(nullptr, U, level, 0, (int)i);
       a.t0 = 0;
       a.key_row0 = 0;
       add(ipq, a);
       if (small) {
+        sp.mul |= k.mul_a != nullptr;
         add(sp, a);
         Seg b = seg(nullptr, has_moddown(it) ? S.UC : U + (size_t)level * N, K, L, (int)i);
         b.t0 = level;
@@ -347,6 +364,7 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
   ipp.gather_own = ipq.gather_own;
   ipp.gather_ext = ipq.gather_ext;
   ipp.add_c1 = ipq.add_c1;
+  ipp.mul = ipq.mul;
   // complementary pipelining (Section IV-B; `fork`, plans only): the q-limb inner product on an
   // auxiliary branch beside ModDown's special-limb chain; otherwise one launch over all limbs.
   // Single calls keep one stream: their stages are dependent launches, whose chain a fork and
@@ -409,9 +427,9 @@ static cudaError_t launch_stage(fhe_ctx *c, const Stage &st, const SegList &sl, 
     case Stage::NTT: return launch_ntt_pass(c->tabs, st.column, st.fwd, st.pro, st.epi, sl, q);
     case Stage::NTT1: return launch_ntt_single(c->tabs, st.fwd, st.pro, st.epi, sl, *sl2, q);
     case Stage::EW: return launch_ew(c->tabs, st.ewop, sl, q);
-    case Stage::IP: return launch_ip(c->tabs, sl, st.gather_own, st.gather_ext, st.add_c1, c->dnum, q);
+    case Stage::IP: return launch_ip(c->tabs, sl, st.gather_own, st.gather_ext, st.add_c1, st.mul, c->dnum, q);
     case Stage::SNTT: return launch_small_ntt(c->tabs, st.fwd, st.pro, st.epi, sl, q);
-    case Stage::SIP: return launch_small_ip(c->tabs, sl, q);
+    case Stage::SIP: return launch_small_ip(c->tabs, sl, st.mul, q);
     case Stage::IPN: return launch_ip_intt(c->tabs, sl, std::min(c->dnum, 4), q);
     case Stage::BCONV:
       return c->bconv_mode == FHE_BCONV_TC ? launch_bconv_tc(c->tabs, ba, st.max_in, st.max_out, q, c->tabs.tc_k)

@@ -39,6 +39,7 @@ struct Stage {
   bool aux = false;
   bool gather_own = false, gather_ext = false;
   bool add_c1 = false;  // IP: some item adds its pass-through polynomial to both halves
+  bool mul = false;     // IP: some item forms its tensor product on the fly
   int max_in = 0, max_out = 0;
   std::vector<fhe::Seg> segs;
   std::vector<fhe::Seg> segs2;

@@ -55,6 +55,12 @@ def test_back_to_back_calls(fhe_lib, name, level, tc):
         for i, g in enumerate(got):
             for k, (x, y) in enumerate(zip(g, want[i % 3])):
                 assert torch.equal(x, y), (rep, i, k)
+    # a product written over its own factor (the factors are read before the last kernel writes)
+    for k in (0, 1):
+        ab = [x.clone() for x in sets[1]]
+        assert torch.equal(ctx.hmult(ab[0], ab[1], level, out=ab[k]), want[1][2])
+    sq = sets[2][0].clone()
+    assert torch.equal(ctx.hmult(sq, sq, level, out=sq), ctx.hmult(sets[2][0], sets[2][0], level))
     # a caller's own capture of the same calls, replayed on other inputs
     a, b = (x.clone() for x in sets[0])
     torch.cuda.synchronize()
