@@ -74,11 +74,11 @@ static cudaError_t ntt_go(const DevTables &t, const SegList &sl, cudaStream_t s)
 // Block pass with each half-warp on its own (ntt_blk.cuh).
 template <int LOGN, bool FWD, int PRO, int EPI>
 static cudaError_t ntt_blk_go(const DevTables &t, const SegList &sl, cudaStream_t s) {
-  const unsigned grid = (unsigned)(sl.total * ((1 << LOGN) / kTile));
+  const unsigned grid = (unsigned)(sl.total * ((1 << LOGN) / (256 * kBlkBlocks)));
   if (grid == 0) return cudaSuccess;
   TraceScope ts(t, ntt_name<LOGN, false, FWD, PRO, EPI, false>(), s);
   g_launches++;
-  return launch_dep(t.dep, t.dep ? k_ntt_blk<LOGN, FWD, PRO, EPI, true> : k_ntt_blk<LOGN, FWD, PRO, EPI, false>, grid, kNttThreads, 0, s, sl, t.ntt);
+  return launch_dep(t.dep, t.dep ? k_ntt_blk<LOGN, FWD, PRO, EPI, true> : k_ntt_blk<LOGN, FWD, PRO, EPI, false>, grid, kBlkThreads, 0, s, sl, t.ntt);
 }
 
 // Column pass with warp-private twiddles (ntt_col.cuh).

@@ -234,23 +234,27 @@ __device__ __forceinline__ void blk_inverse(uint32_t (&x)[16], uint32_t *sm, int
 }
 
 // Forward: PRO_PLAIN with EPI_PLAIN, EPI_COMBINE or EPI_RESCALE; inverse: PRO_PLAIN,
-// PRO_GATHER or PRO_MUL with EPI_LAZY.  Residency: 48 registers (16 values, 30 of twiddles), five CTAs
-// (four and six, and loading the lo twiddles after the hi round: within 1 % or slower).
+// PRO_GATHER or PRO_MUL with EPI_LAZY.  Residency: 48 registers (16 values, 30 of twiddles), 40
+// warps per SM (32 and 48, and loading the lo twiddles after the hi round: within 1 % or slower).
+// Four blocks (two warps) per CTA: with no CTA barrier the size only sets how finely the launch
+// fills the SMs; against 256 and 128 threads the 64-item mixed plan takes 2444 us instead of 2465
+// and 2449, one rotation 99.4 instead of 100.4 and 99.7.
+constexpr int kBlkThreads = 64, kBlkBlocks = kBlkThreads / 16;
 template <int LOGN, bool FWD, int PRO, int EPI, bool DEP>
-__global__ void __launch_bounds__(kNttThreads, (DEP && FWD) || PRO == PRO_MUL ? 4 : 5) k_ntt_blk(const __grid_constant__ SegList sl, const NttTables tb) {
-  constexpr int TILES = (1 << LOGN) / kTile;
-  __shared__ __align__(16) uint32_t sm[16 * 272];
-  __shared__ __align__(16) uint2 hws[16 * 16];
+__global__ void __launch_bounds__(kBlkThreads, ((DEP && FWD) || PRO == PRO_MUL ? 4 : 5) * (256 / kBlkThreads)) k_ntt_blk(const __grid_constant__ SegList sl, const NttTables tb) {
+  constexpr int TILES = (1 << LOGN) / (256 * kBlkBlocks);
+  __shared__ __align__(16) uint32_t sm[kBlkBlocks * 272];
+  __shared__ __align__(16) uint2 hws[kBlkBlocks * 16];
   const int tid = threadIdx.x, c = tid >> 4, tau = tid & 15;
   const int v = blockIdx.x / TILES, tile = blockIdx.x % TILES;
   const Limb lb = limb_at<EPI == EPI_COMBINE>(sl, v, tb.ninv, LOGN);
   const PrimeC P = tb.pc[lb.prime];
   const uint32_t q = P.q;
-  const int blk = tile * 16 + c;
+  const int blk = tile * kBlkBlocks + c;
   uint2 *hw = hws + c * 16;
   const uint2 h1 = blk_hi_twiddle<LOGN, FWD>(tb, lb.prime, blk, tau);
   uint2 tl[16];
-  load_lo_twiddles<LOGN>(FWD ? tb.lo_fwd : tb.lo_inv, lb.prime, tile, tid, tl);
+  load_lo_twiddles<LOGN>(FWD ? tb.lo_fwd : tb.lo_inv, lb.prime, blk >> 4, (blk & 15) * 16 + tau, tl);
   uint32_t x[16];
   if (DEP) dep_wait();
   if (FWD) {
