@@ -129,6 +129,7 @@ struct KsArgs {
                          // inner product adds P * addp to u's q-limbs, so ModDown's (u - r) P^-1 carries it
   const uint32_t *mul_a, *mul_b;  // HMult's factors [2][level][N] when the tensor product is formed on the fly
                          // (own limbs a1 b1, pass-through (a0 b0, a0 b1 + a1 b0)), else null
+  const uint32_t *r, *u; // the item's converted special limbs and inner product (PRO_SUM, EPI_SUM)
   const uint2 *pinv;     // [L] Shoup pairs of P^-1 mod q_i
   const uint2 *pmod;     // [L] Shoup pairs of P mod q_i
   int level, n_ext, beta, alpha, L, K;
@@ -172,6 +173,7 @@ struct SegList {
   // and first extended-basis index, whose limbs are taken limb by limb across the segments
   int lm_groups;
   int lm_first[4], lm_count[4];
+  int sum_n;                 // PRO_SUM, EPI_SUM: items ks[0..sum_n) are summed
   Seg seg[kMaxSeg];
   KsArgs ks[kMaxInlineItems];
   uint16_t first[kMaxSeg];          // inline lists: the segment's first limb, and each limb's segment
@@ -182,7 +184,7 @@ static_assert(kMaxSeg <= 256, "segof holds a segment index in a byte");
 // an empty by-value list: the header alone (the arrays hold what their counts say; clearing the
 // 14 KB of them before each launch was a third of a small call's host time)
 inline void seg_clear(SegList &l) {
-  l.nseg = l.total = l.lm_groups = 0;
+  l.nseg = l.total = l.lm_groups = l.sum_n = 0;
   l.dev = nullptr;
   l.vmap = nullptr;
   l.limbs = nullptr;

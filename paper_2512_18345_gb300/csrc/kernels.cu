@@ -42,8 +42,8 @@ void note_launch() { g_launches++; }
 
 template <int LOGN, bool COLUMN, bool FWD, int PRO, int EPI, bool OTF>
 static const char *ntt_name() {
-  static const char *pro[] = {"", "+gather", "+reduce", "+bconv", "+mul"};
-  static const char *epi[] = {"", "", "+scale", "+combine", "+rescale"};
+  static const char *pro[] = {"", "+gather", "+reduce", "+bconv", "+mul", "+sum"};
+  static const char *epi[] = {"", "", "+scale", "+combine", "+rescale", "+sum"};
   static const std::string name = [] {  // initialised once, thread-safe
     char buf[64];
     snprintf(buf, sizeof buf, "%s_%s%s%s%s", FWD ? "ntt" : "intt", COLUMN ? "col" : "blk", pro[PRO], epi[EPI],
@@ -154,6 +154,10 @@ static cudaError_t ntt_dispatch(const DevTables &t, bool column, bool fwd, int p
   NTT_CASE(false, false, PRO_GATHER, EPI_LAZY)
   NTT_CASE(true, false, PRO_PLAIN, EPI_SCALE)
 #undef NTT_CASE
+  if constexpr (LOGN == 16) {
+    if (column && fwd && pro == PRO_SUM && epi == EPI_LAZY) return ntt_col_go<LOGN, true, PRO_SUM, EPI_LAZY>(t, sl, s);
+    if (!column && fwd && pro == PRO_PLAIN && epi == EPI_SUM) return ntt_blk_go<LOGN, true, PRO_PLAIN, EPI_SUM>(t, sl, s);
+  }
   if (!column && !fwd && pro == PRO_MUL && epi == EPI_LAZY) return ntt_blk_go<LOGN, false, PRO_MUL, EPI_LAZY>(t, sl, s);
   return cudaErrorInvalidValue;
 }

@@ -432,6 +432,33 @@ extern "C" int fhe_linear_transform(fhe_ctx *c, const uint32_t *ct, int level, c
     it.key = c->find_key(baby * g);
     its.push_back(it);
   }
+  if (merge_moddowns(c) && (int)its.size() == giant - 1 && giant > 1) {
+    // out = inner_0 + sum_g rot_{B g}(inner_g) with the rotations' ModDowns merged into one
+    // transform of the output's limbs (as many rotations per program as its launch arguments
+    // hold; a further program adds to out)
+    size_t i = 0;
+    const uint32_t *base = inner;
+    while (i < its.size()) {
+      std::vector<Item> chunk;
+      for (size_t j = i; j < its.size(); j++) {
+        Item it = its[j];
+        it.sum = true;
+        it.out = out;
+        it.in2 = base;
+        it.slot = (int)(j - i);
+        chunk.push_back(it);
+        if (chunk.size() > 1 && !items_fit_inline(c, chunk)) {
+          chunk.pop_back();
+          break;
+        }
+      }
+      rc = run_items_chunked(c, chunk, 0, s);  // (fits one program)
+      if (rc != FHE_OK) return rc;
+      i += chunk.size();
+      base = out;
+    }
+    return FHE_OK;
+  }
   rc = run_items_chunked(c, its, 0, s);
   if (rc != FHE_OK) return rc;
   // out = inner_0 + sum_g rot_{B g}(inner_g), in one pass

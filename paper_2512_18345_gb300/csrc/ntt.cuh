@@ -46,6 +46,7 @@ enum : int {
   PRO_GATHER = 1,  // src[sigma(j)], sigma = the limb's galois (NTT form input)
   PRO_REDUCE = 2,  // src[j] reduced from another prime (rescale: src_prime)
   PRO_BCONV = 3,   // base conversion of n_in limbs at src (small ring)
+  PRO_SUM = 5,     // sum over the list's items at src's place in each item's r (merged ModDowns)
   PRO_MUL = 4,     // src[j] src2[j] where the limb has a src2 (HMult's d2), else as PRO_GATHER
 };
 // Epilogue modes (how the last pass writes an element)
@@ -55,6 +56,7 @@ enum : int {
   EPI_SCALE = 2,    // write v * scale (inverse final: N^-1 * constant)
   EPI_COMBINE = 3,  // ModDown combine: (src2[j] - v) P^-1 (+ add), src2 = inner product u
   EPI_RESCALE = 4,  // (src2[j] - v) * scale
+  EPI_SUM = 5,      // T[j] + (sum over the items' u at src2's place - v) P^-1 (merged ModDowns)
 };
 
 template <int LOGN, bool COLUMN>

@@ -157,18 +157,35 @@ __device__ __forceinline__ void blk_forward(uint32_t (&x)[16], uint32_t *sm, int
 }
 // write the results in sm to the limb in memory order
 template <int EPI, bool DEP>
-__device__ __forceinline__ void blk_store(const Limb &lb, int blk, uint32_t *sm, int c, int tau, uint2 scale, uint32_t q) {
+__device__ __forceinline__ void blk_store(const SegList &sl, const Limb &lb, int blk, uint32_t *sm, int c, int tau,
+                                          uint2 scale, uint32_t q) {
 #pragma unroll
   for (int i = 0; i < 4; i++) {
     const int j = blk * 256 + 64 * i + 4 * tau;
     uint32_t o[4], a[4];
     if (EPI == EPI_COMBINE || EPI == EPI_RESCALE) ld_in4<DEP>(lb.src2 + j, a);
+    if (EPI == EPI_SUM) {
+      const size_t off = (size_t)(lb.src2 - sl.ks[0].u) + j;
+      a[0] = a[1] = a[2] = a[3] = 0;
+      for (int k = 0; k < sl.sum_n; k++) {
+        uint32_t w[4];
+        ld_in4<DEP>(sl.ks[k].u + off, w);
+#pragma unroll
+        for (int e = 0; e < 4; e++) a[e] = add_mod(a[e], w[e], q);
+      }
+    }
     ld4(blk_lin(sm, c, tau, i), o);
 #pragma unroll
     for (int e = 0; e < 4; e++) {
       o[e] = red2(o[e], q);
       // COMBINE: a = inner product u (with P times the pass-through term folded in)
-      if (EPI == EPI_COMBINE || EPI == EPI_RESCALE) o[e] = shoup(a[e] + q - o[e], scale.x, scale.y, q);
+      if (EPI == EPI_COMBINE || EPI == EPI_RESCALE || EPI == EPI_SUM) o[e] = shoup(a[e] + q - o[e], scale.x, scale.y, q);
+    }
+    if (EPI == EPI_SUM) {
+      uint32_t w[4];
+      ld_in4<DEP>(lb.T + j, w);
+#pragma unroll
+      for (int e = 0; e < 4; e++) o[e] = add_mod(o[e], w[e], q);
     }
     st4(lb.dst + j, o);
   }
@@ -233,7 +250,7 @@ __device__ __forceinline__ void blk_inverse(uint32_t (&x)[16], uint32_t *sm, int
   nb_round_hi<false>(x, hw, q);
 }
 
-// Forward: PRO_PLAIN with EPI_PLAIN, EPI_COMBINE or EPI_RESCALE; inverse: PRO_PLAIN,
+// Forward: PRO_PLAIN with EPI_PLAIN, EPI_COMBINE, EPI_RESCALE or EPI_SUM; inverse: PRO_PLAIN,
 // PRO_GATHER or PRO_MUL with EPI_LAZY.  Residency: 48 registers (16 values, 30 of twiddles), 40
 // warps per SM (32 and 48, and loading the lo twiddles after the hi round: within 1 % or slower).
 // Four blocks (two warps) per CTA: with no CTA barrier the size only sets how finely the launch
@@ -247,7 +264,7 @@ __global__ void __launch_bounds__(kBlkThreads, ((DEP && FWD) || PRO == PRO_MUL ?
   __shared__ __align__(16) uint2 hws[kBlkBlocks * 16];
   const int tid = threadIdx.x, c = tid >> 4, tau = tid & 15;
   const int v = blockIdx.x / TILES, tile = blockIdx.x % TILES;
-  const Limb lb = limb_at<EPI == EPI_COMBINE>(sl, v, tb.ninv, LOGN);
+  const Limb lb = limb_at<EPI == EPI_COMBINE || EPI == EPI_SUM>(sl, v, tb.ninv, LOGN);
   const PrimeC P = tb.pc[lb.prime];
   const uint32_t q = P.q;
   const int blk = tile * kBlkBlocks + c;
@@ -265,8 +282,8 @@ __global__ void __launch_bounds__(kBlkThreads, ((DEP && FWD) || PRO == PRO_MUL ?
     __syncwarp();  // the hi-round twiddles
     blk_forward(x, sm, c, tau, hw, tl, q);
     uint2 scale = make_uint2(0, 0);
-    if (EPI == EPI_COMBINE || EPI == EPI_RESCALE) scale = __ldg(lb.scale);
-    blk_store<EPI, DEP>(lb, blk, sm, c, tau, scale, q);
+    if (EPI != EPI_PLAIN) scale = __ldg(lb.scale);
+    blk_store<EPI, DEP>(sl, lb, blk, sm, c, tau, scale, q);
   } else {
     blk_load<LOGN, PRO, DEP>(x, lb, P, blk, sm, c, tau, [&] { hw[tau] = h1; });
     blk_inverse(x, sm, c, tau, hw, tl, q);

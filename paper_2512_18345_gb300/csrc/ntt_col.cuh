@@ -20,7 +20,7 @@ namespace fhe {
 template <bool FWD>
 constexpr int ntt_col_ctas() { return FWD ? 6 : 7; }
 
-// Forward: PRO_PLAIN or PRO_REDUCE with EPI_LAZY; inverse: PRO_PLAIN with EPI_SCALE.
+// Forward: PRO_PLAIN, PRO_REDUCE or PRO_SUM with EPI_LAZY; inverse: PRO_PLAIN with EPI_SCALE.
 template <int LOGN, bool FWD, int PRO, int EPI, bool DEP>
 __global__ void __launch_bounds__(kNttThreads, ntt_col_ctas<FWD>())
     k_ntt_col(const __grid_constant__ SegList sl, const NttTables tb) {
@@ -49,6 +49,19 @@ __global__ void __launch_bounds__(kNttThreads, ntt_col_ctas<FWD>())
   uint32_t x[16];
 #pragma unroll
   for (int e = 0; e < 16; e++) x[e] = ld_in<DEP>(lb.src + G::gidx(tile, c, kmap<R>(FWD, e, tau)));
+  if (PRO == PRO_SUM) {  // the other items' values (each lazy, in [0, 2q))
+    const size_t off = (size_t)(lb.src - sl.ks[0].r);
+#pragma unroll
+    for (int e = 0; e < 16; e++) x[e] = red2(x[e], q);
+    for (int i = 1; i < sl.sum_n; i++) {
+      const uint32_t *p = sl.ks[i].r + off;
+      uint32_t w[16];
+#pragma unroll
+      for (int e = 0; e < 16; e++) w[e] = ld_in<DEP>(p + G::gidx(tile, c, kmap<R>(FWD, e, tau)));
+#pragma unroll
+      for (int e = 0; e < 16; e++) x[e] = add_mod(x[e], red2(w[e], q), q);
+    }
+  }
   // (stored after the loads are on their way, so that their latencies overlap)
   if (lane < 16) hw[lane] = h1;
   if (R == 8) hw[16 + (lane >> 4) * kLo + (lane & 15)] = h2;

@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(kNttThreads, PRO == PRO_BCONV ? 2 : 4)
 #pragma unroll
   for (int e = 0; e < 16; e++) x[e] = s.sm[nb_blk_addr(c, (e << 4) | tau)];
   blk_forward(x, s.sm, c, tau, s.hws + c * 16, tl, q);
-  blk_store<EPI, DEP>(lb, c, s.sm, c, tau, scale, q);
+  blk_store<EPI, DEP>(sl, lb, c, s.sm, c, tau, scale, q);
 }
 
 // One CTA per extended limb and half: u_c = sum_j ModUp_j key_j[c] (+ P addp_c on the q-limbs),

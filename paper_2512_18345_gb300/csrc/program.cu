@@ -64,6 +64,11 @@ static void push_transform(fhe_ctx *c, Program &P, Stage first, Stage second) {
   P.stages.push_back(std::move(second));
 }
 
+bool merge_moddowns(const fhe_ctx *c) {
+  const DevTables &t = c->tabs;
+  return c->fused && c->logn == 16 && !t.ntt_otf && !t.ntt_single && !t.ntt_stream && !t.ntt_persist;
+}
+
 int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool fork, Program &P) {
   const size_t N = c->N;
   const int L = c->L, K = c->K, A = c->alpha;
@@ -90,6 +95,8 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
     memset(&k, 0, sizeof k);
     k.ext = S.EXT;
     k.key = it.key;
+    k.r = S.R;
+    k.u = S.U;
     k.pinv = c->d_pinv;
     k.pmod = c->d_pmod;
     k.level = it.level;
@@ -347,6 +354,20 @@ int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool f
       mbc.groups.push_back(g);
       mbc.max_in = std::max(mbc.max_in, K);
       mbc.max_out = std::max(mbc.max_out, level);
+      if (it.sum) {
+        // sum_g (u_g - NTT(r_g)) P^-1 = (sum_g u_g - NTT(sum_g r_g)) P^-1: the first item's limbs
+        // alone are transformed, summing every item's r in the loads and u in the combine
+        if (i > 0) continue;
+        r1.pro = PRO_SUM;
+        r2.epi = EPI_SUM;
+        add(r1, seg(r, r, level, 0, 0));
+        Seg z = seg(r, it.out + (size_t)cc * level * N, level, 0, 0);
+        z.src2 = U + (size_t)cc * n_ext * N;
+        z.T = it.in2 + (size_t)cc * level * N;
+        z.n_in = (int)N;
+        add(r2, z);
+        continue;
+      }
       add(r1, seg(r, r, level, 0, (int)i));
       Seg z = fused ? seg(r, it.out + (size_t)cc * level * N, level, 0, (int)i) : seg(r, r, level, 0, (int)i);
       z.src2 = U + (size_t)cc * n_ext * N;
@@ -502,6 +523,7 @@ int run_program_inline(fhe_ctx *c, const Program &P, cudaStream_t s) {
         for (const Seg &x : segs) seg_push(l, x);
     };
     fill(sl, st.segs);
+    if (st.pro == PRO_SUM || st.epi == EPI_SUM) sl.sum_n = (int)P.ks.size();
     if (!st.segs2.empty()) {
       seg_clear(sl2);
       fill(sl2, st.segs2);

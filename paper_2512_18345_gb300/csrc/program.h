@@ -20,6 +20,8 @@ struct Item {
   uint32_t galois = 1;             // rotation Galois element (1: none)
   const uint32_t *in = nullptr;    // KS / MODUP: d [level][N]; ROTATE / MODDOWN: ct [2][level][N]; RELIN: a;
                                    // IPX: the polynomial that was ModUp'ed [level][N]; MDX: [npoly][level+K][N]
+  bool sum = false;                // ROTATE: every item of the program is summed into `out` over the first
+                                   // item's in2 [2][level][N], with one ModDown transform (merge_moddowns)
   const uint32_t *in2 = nullptr;   // RELIN: b; IPX: pass-through c0 [level][N] or null
   uint32_t *out = nullptr;         // [2][level][N]; MODUP: [beta][level+K][N], or null (the slot's)
   const uint32_t *key = nullptr;   // switching key (not for MODUP)
@@ -61,6 +63,8 @@ struct DevProgram {
 
 int ensure_slots(fhe_ctx *c, int n);
 // fork: the inner product of the ciphertext limbs on an auxiliary branch (complementary pipelining)
+// whether programs may merge the ModDowns of summed rotations (Item::sum)
+bool merge_moddowns(const fhe_ctx *c);
 int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool fork, Program &P);
 // whether the items' program fits by-value launch arguments (program_fits_inline of it, without
 // building it or growing the workspace)
