@@ -35,6 +35,12 @@ struct DiagArgs {
   int nb, giant, nlimb, level, L;    // limb i < level is modulo q_i, limb i >= level modulo p_{i - level}
   int16_t didx[kMaxGiant * kMaxBaby];  // [giant][nb]: index into diags, -1 where the pair has no diagonal
   uint32_t gmask[kMaxGiant];           // bit b of gmask[g]: didx[g][b] >= 0
+  // double-hoisted form: the baby steps without rotation, P ct in the extended basis, are read
+  // from ct itself and scaled by P in registers (their special limbs are zero: no step at all),
+  // which spares the kernel and the array that lifted them (14 us of a CoeffToSlot level)
+  uint32_t idmask;
+  const uint32_t *ct;                  // [2][level][N]
+  const uint2 *pmod;
 };
 
 static void diag_masks(DiagArgs &da) {
@@ -69,7 +75,8 @@ constexpr int kDiagStageBytes = kDiagRows * kDiagChunk * 4 + 16;  // rows, two m
 constexpr int kDiagStages = 8;
 static_assert(kDiagStages * kDiagStageBytes <= 227 * 1024, "diagonal kernel: stages exceed shared memory");
 
-template <bool DEP>
+// ID: some baby step is the identity (idmask).
+template <bool ID, bool DEP>
 __global__ void __launch_bounds__(kDiagThreads + 32, 1) k_diag_bulk(const __grid_constant__ DiagArgs a, const PrimeC *pc,
                                                                    int logn, unsigned int *status) {
   constexpr int stages = kDiagStages;
@@ -91,12 +98,13 @@ __global__ void __launch_bounds__(kDiagThreads + 32, 1) k_diag_bulk(const __grid
       mbar_init(&ebar[st], kDiagThreads);
     }
   __syncthreads();
-  // the baby steps of group grp that meet a diagonal
-  auto group_mask = [&](int grp, uint32_t (&gm)[kGsub]) {
+  // the baby steps of limb i and group grp that meet a diagonal
+  auto group_mask = [&](int grp, int i, uint32_t (&gm)[kGsub]) {
+    const uint32_t in = !ID || i < a.level ? ~0u : ~a.idmask;
     uint32_t any = 0;
 #pragma unroll
     for (int g = 0; g < kGsub; g++) {
-      gm[g] = grp * kGsub + g < a.giant ? a.gmask[grp * kGsub + g] : 0u;
+      gm[g] = grp * kGsub + g < a.giant ? a.gmask[grp * kGsub + g] & in : 0u;
       any |= gm[g];
     }
     return any;
@@ -114,7 +122,7 @@ __global__ void __launch_bounds__(kDiagThreads + 32, 1) k_diag_bulk(const __grid
       const int grp = u % groups, ch = (u / groups) % chunks, i = u / (groups * chunks);
       const size_t off = (size_t)i * N + (size_t)ch * kDiagChunk;
       uint32_t gm[kGsub];
-      for (uint32_t live = group_mask(grp, gm); live; live &= live - 1) {
+      for (uint32_t live = group_mask(grp, i, gm); live; live &= live - 1) {
         const int b = __ffs(live) - 1;
         const int st = k % stages;
         // the consumers released this stage's previous step (bounded: if they gave up, so do we)
@@ -125,8 +133,10 @@ __global__ void __launch_bounds__(kDiagThreads + 32, 1) k_diag_bulk(const __grid
         for (int g = 0; g < kGsub; g++) rows += (gm[g] >> b) & 1u;
         mbar_arrive_expect_tx(&bar[st], rows * kDiagChunk * 4u);
         uint32_t *dst = buf + (size_t)st * stage_words;
-        bulk_g2s(dst, a.babies[b] + off, kDiagChunk * 4u, &bar[st]);
-        bulk_g2s(dst + kDiagChunk, a.babies[b] + poly + off, kDiagChunk * 4u, &bar[st]);
+        const bool id = ID && ((a.idmask >> b) & 1u);
+        const uint32_t *x0 = (id ? a.ct : a.babies[b]) + off;
+        bulk_g2s(dst, x0, kDiagChunk * 4u, &bar[st]);
+        bulk_g2s(dst + kDiagChunk, x0 + (id ? (size_t)a.level * N : poly), kDiagChunk * 4u, &bar[st]);
 #pragma unroll
         for (int g = 0; g < kGsub; g++)
           if ((gm[g] >> b) & 1u)
@@ -148,7 +158,8 @@ __global__ void __launch_bounds__(kDiagThreads + 32, 1) k_diag_bulk(const __grid
     const PrimeC P = pc[limb_prime(i, a.level, a.L)];
     const uint32_t r34 = P.r34;
     uint32_t gm[kGsub];
-    uint32_t live = group_mask(grp, gm);
+    uint32_t live = group_mask(grp, i, gm);
+    const uint2 pm = ID && i < a.level ? a.pmod[i] : make_uint2(0, 0);
     uint64_t acc[2][kGsub][E];
 #pragma unroll
     for (int g = 0; g < kGsub; g++)
@@ -166,6 +177,9 @@ __global__ void __launch_bounds__(kDiagThreads + 32, 1) k_diag_bulk(const __grid
       uint32_t x0[E], x1[E];
       ld_words<E>(src, x0);
       ld_words<E>(src + kDiagChunk, x1);
+      if (ID && ((a.idmask >> b) & 1u))
+#pragma unroll
+        for (int e = 0; e < E; e++) x0[e] = shoup(x0[e], pm, P.q), x1[e] = shoup(x1[e], pm, P.q);
 #pragma unroll
       for (int g = 0; g < kGsub; g++)
         if ((gm[g] >> b) & 1u) {
@@ -211,7 +225,7 @@ __global__ void __launch_bounds__(kDiagThreads + 32, 1) k_diag_bulk(const __grid
     int issued = 0;  // steps of this CTA
     for (int u = blockIdx.x; u < total; u += gridDim.x) {
       uint32_t gm[kGsub];
-      issued += __popc(group_mask(u % groups, gm));
+      issued += __popc(group_mask(u % groups, u / (groups * chunks), gm));
     }
     for (int k2 = k; k2 < min(issued, k + stages); k2++)
       mbar_wait_bounded(&bar[k2 % stages], (uint32_t)(k2 / stages) & 1u);
@@ -219,44 +233,27 @@ __global__ void __launch_bounds__(kDiagThreads + 32, 1) k_diag_bulk(const __grid
 }
 
 
-static cudaError_t launch_diag(fhe_ctx *c, const DiagArgs &da, cudaStream_t s) {
+template <bool ID, bool DEP>
+static cudaError_t diag_go(fhe_ctx *c, const DiagArgs &da, unsigned grid, cudaStream_t s) {
   static PerDeviceOnce configured;
   const cudaError_t e = configured.run([] {
-    constexpr int kMax = kDiagStages * kDiagStageBytes;
-    const cudaError_t e0 = cudaFuncSetAttribute(k_diag_bulk<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
-    return e0 != cudaSuccess ? e0
-                             : cudaFuncSetAttribute(k_diag_bulk<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
+    return cudaFuncSetAttribute(k_diag_bulk<ID, DEP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kDiagStages * kDiagStageBytes);
   });
   if (e != cudaSuccess) return e;
+  return launch_dep(DEP, k_diag_bulk<ID, DEP>, grid, kDiagThreads + 32, kDiagStages * kDiagStageBytes, s, da, c->d_pc,
+                    c->logn, c->tabs.status);
+}
+
+static cudaError_t launch_diag(fhe_ctx *c, const DiagArgs &da, cudaStream_t s) {
   const int sms = c->tabs.sms;
   const int units = da.nlimb * (int)(c->N / kDiagChunk) * ((da.giant + kGsub - 1) / kGsub);
   const unsigned grid = (unsigned)std::min(units, std::max(1, sms));  // persistent: one CTA per SM
   const bool dep = c->dep_next((size_t)2 * da.giant * da.nlimb);
   note_launch();
   c->after_kernel = true;
-  return launch_dep(dep, dep ? k_diag_bulk<true> : k_diag_bulk<false>, grid, kDiagThreads + 32,
-                    kDiagStages * kDiagStageBytes, s, da, c->d_pc, c->logn, c->tabs.status);
-}
-
-// The identity baby step of a double-hoisted transform, in the extended basis:
-// out[c] = P ct[c] on the q-limbs and 0 on the special limbs (ModDown of it returns ct exactly).
-__global__ void __launch_bounds__(256) k_lift(const uint32_t *ct, uint32_t *out, const uint2 *pmod, const PrimeC *pc,
-                                              int level, int nlimb, int logn) {
-  const size_t N = (size_t)1 << logn;
-  const int per_limb = (int)(N / 1024);  // four consecutive coefficients per thread
-  const int i = blockIdx.x / per_limb;
-  const size_t n = (size_t)(blockIdx.x % per_limb) * 1024 + threadIdx.x * 4;
-#pragma unroll
-  for (int c = 0; c < 2; c++) {
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (i < level) {
-      const uint4 x = __ldg(reinterpret_cast<const uint4 *>(ct + ((size_t)c * level + i) * N + n));
-      const uint2 pm = pmod[i];
-      const uint32_t q = pc[i].q;
-      v = make_uint4(shoup(x.x, pm, q), shoup(x.y, pm, q), shoup(x.z, pm, q), shoup(x.w, pm, q));
-    }
-    *reinterpret_cast<uint4 *>(out + ((size_t)c * nlimb + i) * N + n) = v;
-  }
+  if (da.idmask) return dep ? diag_go<true, true>(c, da, grid, s) : diag_go<true, false>(c, da, grid, s);
+  return dep ? diag_go<false, true>(c, da, grid, s) : diag_go<false, false>(c, da, grid, s);
 }
 
 // Giant-step accumulation of a double-hoisted transform, in the extended basis:
@@ -487,7 +484,7 @@ extern "C" int fhe_linear_transform(fhe_ctx *c, const uint32_t *ct, int level, c
 //   out = sum_g rot_{giant[g]}( sum_b pt[idx[g][b]] (.) rot_{baby[b]}(ct) ).
 // (1) one ModUp of c1; every baby rotation's inner product stays in the
 //     extended basis Q_l u P, with P sigma_b(c0) folded onto its q-limbs
-//     (IT_IPX); a baby step without rotation is P ct (k_lift);
+//     (IT_IPX); a baby step without rotation is P ct (formed in the diagonal pass);
 // (2) the inner sums are formed in the extended basis (k_diag_bulk over l + K limbs);
 // (3) per rotating giant step, the c1 half of its inner sum goes down to Q_l
 //     (IT_MDX), is decomposed again (IT_MODUP) and key-switched with sigma_g on the
@@ -539,14 +536,7 @@ extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level
   // (1) baby steps
   std::vector<Item> its;
   for (int b = 0; b < n_baby; b++) {
-    if (gb[b] == 1u) {
-      TraceScope ts(c->tabs, "lt_lift", s);
-      k_lift<<<grid_x / 4, 256, 0, s>>>(ct, bab + b * xct, c->d_pmod, c->d_pc, level, n_ext, c->logn);
-      note_launch();
-      if (cudaGetLastError() != cudaSuccess) return fhe_fail(FHE_ECUDA, "%s: lift kernel", fn);
-      c->after_kernel = true;
-      continue;
-    }
+    if (gb[b] == 1u) continue;  // (the diagonal pass reads ct itself)
     Item it;
     it.kind = IT_IPX;
     it.level = level;
@@ -581,6 +571,10 @@ extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level
   da.L = c->L;
   for (int k = 0; k < n_baby * n_giant; k++) da.didx[k] = (int16_t)idx[k];
   diag_masks(da);
+  for (int b = 0; b < n_baby; b++)
+    if (gb[b] == 1u) da.idmask |= 1u << b;
+  da.ct = ct;
+  da.pmod = c->d_pmod;
   {
     TraceScope ts(c->tabs, "diag_mac", s);
     if (launch_diag(c, da, s) != cudaSuccess) return fhe_fail(FHE_ECUDA, "%s: diagonal kernel", fn);
