@@ -80,6 +80,64 @@ extern "C" int fhe_ctx_set_batch(fhe_ctx *c, size_t l2_budget_bytes, int max_gro
   return FHE_OK;
 }
 
+// Group the items, in order.  With a budget or a group cap set (fhe_ctx_set_batch), consecutive
+// items while their stage-1 working sets stay within the budget, so that the groups in flight do.
+// By default: one group while the working set is within twice the L2 over the lanes; above that
+// equal shares of at least one group per lane, of about twice that size or kWideGroup items --
+// the stage kernels are bound by instruction issue, and large launches amortise their ramp and
+// their last wave better than L2 residency saves (64 mixed items at N = 2^16: groups of 16 on two
+// lanes 2342 us, of 8 2422; 8 rotations: 4 + 4 and 5 + 3 within 0.3 %).  Every group item of every
+// lane holds a workspace slot; where memory (or the context's limit) is short of the default's,
+// the smaller groups of twice the L2 and 8 items are taken.
+static constexpr int kWideGroup = 16;
+static std::vector<std::vector<int>> make_groups(const fhe_ctx *c, const fhe_ks_item *items, int n) {
+  const int nl = std::max(1, c->batch_lanes);
+  size_t l2x2 = 0, total = 0;
+  {
+    int l2 = 0;
+    cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, c->device);
+    l2x2 = (size_t)l2 * 2;
+  }
+  std::vector<size_t> fp(n);
+  for (int i = 0; i < n; i++) total += fp[i] = (size_t)c->beta(items[i].level) * (items[i].level + c->K) * 4 * c->N;
+  // groups on different lanes are resident in L2 at the same time
+  const size_t budget = (c->batch_budget ? c->batch_budget : l2x2) / nl;
+  auto split = [&](size_t most, int cap) {
+    std::vector<std::vector<int>> groups(1);
+    size_t used = 0;
+    for (int i = 0; i < n; i++) {
+      if (!groups.back().empty() && (used + fp[i] > most || (int)groups.back().size() >= cap)) {
+        groups.emplace_back();
+        used = 0;
+      }
+      groups.back().push_back(i);
+      used += fp[i];
+    }
+    return groups;
+  };
+  if (!c->batch_budget && c->batch_max_group <= 0 && total > budget) {
+    size_t count = std::max<size_t>(nl, (total + 2 * budget - 1) / (2 * budget));
+    count = std::max<size_t>(count, (n + kWideGroup - 1) / kWideGroup);
+    count = std::min<size_t>((count + nl - 1) / nl * nl, n);  // the same number on every lane
+    std::vector<std::vector<int>> groups(count);
+    size_t before = 0;
+    for (int i = 0; i < n; i++) {  // item i's middle decides its share (shares are never left empty)
+      size_t g = std::min(count - 1, (size_t)((before + fp[i] / 2) * (double)count / total));
+      before += fp[i];
+      groups[g].push_back(i);
+    }
+    size_t most = 0;
+    bool ok = true;
+    for (auto &g : groups) most = std::max(most, g.size()), ok = ok && !g.empty();
+    const size_t lanes = std::min<size_t>(nl, count), have = c->slots.size(), need = lanes * most;
+    const size_t grow = need > have ? (need - have) * c->slot_bytes : 0;
+    size_t avail = 0, all = 0;
+    if (cudaMemGetInfo(&avail, &all) != cudaSuccess) avail = 0;
+    if (ok && grow < avail / 2 && !(c->mem_limit && c->grown_bytes + grow > c->mem_limit)) return groups;
+  }
+  return split(budget, c->batch_max_group > 0 ? c->batch_max_group : 8);
+}
+
 extern "C" int fhe_batch_plan(fhe_ctx *c, const fhe_ks_item *items, int n, int flags, fhe_plan **out) {
   if (!c || !out || n < 1 || !items) return fhe_fail(FHE_EINVAL, "fhe_batch_plan: bad arguments (n >= 1 items)");
   *out = nullptr;
@@ -112,30 +170,8 @@ extern "C" int fhe_batch_plan(fhe_ctx *c, const fhe_ks_item *items, int n, int f
   p->ctx = c;
   p->items.assign(items, items + n);
   p->flags = flags;
-  // group items so that the stage-1 working sets of the groups in flight stay within
-  // the budget (default: twice the L2 -- the stage kernels are bound by the integer
-  // pipes, and larger launches amortise their ramp more than L2 residency saves)
-  size_t budget = c->batch_budget;
-  if (!budget) {
-    int l2 = 0;
-    cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, c->device);
-    budget = (size_t)l2 * 2;
-  }
-  const int max_group = c->batch_max_group > 0 ? c->batch_max_group : 8;
+  const std::vector<std::vector<int>> groups = make_groups(c, items, n);
   const int nl = std::max(1, c->batch_lanes);
-  budget /= nl;  // groups on different lanes are resident in L2 at the same time
-  std::vector<std::vector<int>> groups(1);
-  size_t used = 0;
-  for (int i = 0; i < n; i++) {
-    const int lv = items[i].level;
-    const size_t fp = (size_t)c->beta(lv) * (lv + c->K) * 4 * N;
-    if (!groups.back().empty() && (used + fp > budget || (int)groups.back().size() >= max_group)) {
-      groups.emplace_back();
-      used = 0;
-    }
-    groups.back().push_back(i);
-    used += fp;
-  }
   int rc = FHE_OK;
   p->nlanes = std::min<int>(nl, (int)groups.size());
   if (p->nlanes < 1) p->nlanes = 1;
