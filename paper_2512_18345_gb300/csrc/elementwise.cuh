@@ -204,16 +204,15 @@ __global__ void __launch_bounds__(kIpThreads + 32, 2) k_ip_bulk(const __grid_con
     const uint32_t copies = GEXT ? 2u * (uint32_t)ks.beta : 3u * (uint32_t)ks.beta - (d.gjd >= 0 ? 1u : 0u);
     mbar_arrive_expect_tx(&bar[st], copies * kIpChunk * 4u);
     uint32_t *dst = buf + (size_t)st * stage_words;
-    auto digits = [&] {
-      for (int jd = 0; jd < ks.beta; jd++)
-        if (!GEXT && jd != d.gjd) {
-          const bool own = t < ks.level && t >= jd * ks.alpha && t < (jd + 1) * ks.alpha;
-          const uint32_t *e = own ? ks.own + (size_t)t * N : ks.ext + ((size_t)jd * ks.n_ext + t) * N;
-          bulk_g2s(dst + (size_t)(RPD * jd) * kIpChunk, e + c0, kIpChunk * 4u, &bar[st]);
-        }
+    auto digit = [&](int jd) {
+      if (!GEXT && jd != d.gjd) {
+        const bool own = t < ks.level && t >= jd * ks.alpha && t < (jd + 1) * ks.alpha;
+        const uint32_t *e = own ? ks.own + (size_t)t * N : ks.ext + ((size_t)jd * ks.n_ext + t) * N;
+        bulk_g2s(dst + (size_t)(RPD * jd) * kIpChunk, e + c0, kIpChunk * 4u, &bar[st]);
+      }
     };
-    if (!first) digits();
     for (int jd = 0; jd < ks.beta; jd++) {
+      if (!first) digit(jd);
       const uint32_t *kp = ks.key + jd * kstride + (size_t)row * N + c0;
       bulk_g2s_hint(dst + (size_t)(RPD * jd + KR) * kIpChunk, kp, kIpChunk * 4u, &bar[st], key_policy);
       bulk_g2s_hint(dst + (size_t)(RPD * jd + KR + 1) * kIpChunk, kp + half, kIpChunk * 4u, &bar[st], key_policy);
@@ -221,7 +220,7 @@ __global__ void __launch_bounds__(kIpThreads + 32, 2) k_ip_bulk(const __grid_con
     if (first) {
       dep_wait();
       asm volatile("fence.proxy.async;" ::: "memory");  // bulk copies read what earlier kernels wrote
-      digits();
+      for (int jd = 0; jd < ks.beta; jd++) digit(jd);
     }
   };
   // Warp specialisation: warps 0..7 reduce units, warp 8 (one lane) produces them.  The

@@ -53,22 +53,15 @@ static const char *ntt_name() {
   return name.c_str();
 }
 
-template <int LOGN, bool COLUMN, bool FWD, int PRO, int EPI, bool OTF>
-static cudaError_t ntt_go(const DevTables &t, const SegList &sl, cudaStream_t s) {
-  using G = NttGeom<LOGN, COLUMN>;
+template <int LOGN, bool FWD, int PRO, int EPI>
+static cudaError_t ntt_otf_go(const DevTables &t, const SegList &sl, cudaStream_t s) {
+  using G = NttGeom<LOGN, false>;
   const unsigned grid = (unsigned)(sl.total * G::TILES);
   if (grid == 0) return cudaSuccess;
-  constexpr int smem = ntt_twiddle_smem(COLUMN, G::S);
-  static PerDeviceOnce configured;  // opt in to > 48 KB of shared memory once per instantiation and device
-  cudaError_t e = configured.run([] {
-    return cudaFuncSetAttribute(k_ntt<LOGN, COLUMN, FWD, PRO, EPI, OTF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                smem);
-  });
-  if (e != cudaSuccess) return e;
-  TraceScope ts(t, ntt_name<LOGN, COLUMN, FWD, PRO, EPI, OTF>(), s);
-  k_ntt<LOGN, COLUMN, FWD, PRO, EPI, OTF><<<grid, kNttThreads, smem, s>>>(sl, t.ntt);
+  constexpr int smem = ntt_twiddle_smem(false, G::S);
+  TraceScope ts(t, ntt_name<LOGN, false, FWD, PRO, EPI, true>(), s);
   g_launches++;
-  return cudaGetLastError();
+  return launch_dep(false, k_ntt_otf<LOGN, FWD, PRO, EPI>, grid, kNttThreads, smem, s, sl, t.ntt);
 }
 
 // Block pass with each half-warp on its own (ntt_blk.cuh).
@@ -142,7 +135,7 @@ static cudaError_t ntt_dispatch(const DevTables &t, bool column, bool fwd, int p
 #define NTT_CASE(COL, FWDV, P, E)                                                              \
   if (column == COL && fwd == FWDV && pro == P && epi == E) {                                  \
     if constexpr (COL) return ntt_col_go<LOGN, FWDV, P, E>(t, sl, s);                          \
-    else if (otf) return ntt_go<LOGN, COL, FWDV, P, E, true>(t, sl, s);                        \
+    else if (otf) return ntt_otf_go<LOGN, FWDV, P, E>(t, sl, s);                               \
     else return ntt_blk_go<LOGN, FWDV, P, E>(t, sl, s);                                        \
   }
   NTT_CASE(true, true, PRO_PLAIN, EPI_LAZY)
@@ -157,8 +150,8 @@ static cudaError_t ntt_dispatch(const DevTables &t, bool column, bool fwd, int p
   if constexpr (LOGN == 16) {
     if (column && fwd && pro == PRO_SUM && epi == EPI_LAZY) return ntt_col_go<LOGN, true, PRO_SUM, EPI_LAZY>(t, sl, s);
     if (!column && fwd && pro == PRO_PLAIN && epi == EPI_SUM) return ntt_blk_go<LOGN, true, PRO_PLAIN, EPI_SUM>(t, sl, s);
+    if (!column && !fwd && pro == PRO_MUL && epi == EPI_LAZY) return ntt_blk_go<LOGN, false, PRO_MUL, EPI_LAZY>(t, sl, s);
   }
-  if (!column && !fwd && pro == PRO_MUL && epi == EPI_LAZY) return ntt_blk_go<LOGN, false, PRO_MUL, EPI_LAZY>(t, sl, s);
   return cudaErrorInvalidValue;
 }
 

@@ -14,7 +14,9 @@
 //   256-element blocks.  The inverse runs B then A.  A tile is 4096 elements
 //   (16 KB of shared memory), 256 threads, 16 elements per thread held in
 //   registers through 4 butterfly stages per shared-memory round trip.
-//   Butterflies keep values lazily in [0, 2q) (q < 2^31).
+//   Butterflies keep values lazily in [0, 2q) (q < 2^31).  The default passes are
+//   the kernels of ntt_col.cuh and ntt_blk.cuh (and ntt_small.cuh at N = 2^12);
+//   ntt_pass below is the variants' form of both.
 //
 // Variants (chosen per context, measured by the autotuner):
 //   * on-the-fly twiddles (Section III-C cites them for the second NTT kernel):
@@ -385,31 +387,17 @@ __device__ __forceinline__ void ntt_pass(const Limb &lb, const NttTables &tb, in
   }
 }
 
-// Resident CTAs per SM asked of the register allocator for each pass (the occupancy the
-// passes were measured best at: 8 for the forward column passes, 6 for the inverse column
-// pass, 5 or 4 for the block passes; 6 for ModUp's forward block pass cost a register
-// spill and 1.5 % of its time).
-template <bool COLUMN, bool FWD, int PRO, int EPI, bool OTF>
-constexpr int ntt_min_blocks() {
-  if (COLUMN) return FWD ? 8 : 6;
-  if (!FWD) return 5;
-  return EPI == EPI_RESCALE ? 4 : 5;
-}
-
-template <int LOGN, bool COLUMN, bool FWD, int PRO, int EPI, bool OTF>
-__global__ void __launch_bounds__(kNttThreads, ntt_min_blocks<COLUMN, FWD, PRO, EPI, OTF>())
-    k_ntt(const __grid_constant__ SegList sl, const NttTables tb) {
-  using G = NttGeom<LOGN, COLUMN>;
-  constexpr int R = G::R;
-  // staged twiddles: the column pass needs the S - 1 twiddles of stages 0..R-1 (shared
-  // by all columns); the block pass needs, per stage sigma of its 8, the 16 2^sigma
-  // twiddles of its 16 blocks, stored at 16 (2^sigma - 1).
-  __shared__ uint32_t sm[R == 8 ? G::SMEM : 1];
-  extern __shared__ __align__(16) uint2 tws[];  // dynamic: ntt_twiddle_smem(COLUMN, S) bytes (+ the small table)
-
+// A block pass with on-the-fly twiddles (FHE_NTT_OTF), one CTA per 4096-element tile; the default
+// passes are the kernels of ntt_col.cuh and ntt_blk.cuh.
+template <int LOGN, bool FWD, int PRO, int EPI>
+__global__ void __launch_bounds__(kNttThreads, EPI == EPI_RESCALE ? 4 : 5)
+    k_ntt_otf(const __grid_constant__ SegList sl, const NttTables tb) {
+  using G = NttGeom<LOGN, false>;
+  __shared__ uint32_t sm[G::SMEM];
+  extern __shared__ __align__(16) uint2 tws[];  // dynamic: ntt_twiddle_smem(false, S) bytes
   const int v = blockIdx.x / G::TILES, tile = blockIdx.x % G::TILES;
   const Limb lb = limb_at<EPI == EPI_COMBINE>(sl, v, tb.ninv, LOGN);
-  ntt_pass<LOGN, COLUMN, FWD, PRO, EPI, OTF, SRC_GLOBAL, DST_GLOBAL>(lb, tb, tile, sm, tws, nullptr);
+  ntt_pass<LOGN, false, FWD, PRO, EPI, true, SRC_GLOBAL, DST_GLOBAL>(lb, tb, tile, sm, tws, nullptr);
 }
 
 // Both passes of a 2^16-point transform in one launch: a cluster of 16 CTAs per limb, CTA
