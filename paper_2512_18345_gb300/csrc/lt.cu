@@ -20,6 +20,7 @@
 #include "../../include/fhe.h"
 #include "ctx.h"
 #include "elementwise.cuh"
+#include "ip_diag.cuh"
 #include "internal.h"
 #include "program.h"
 
@@ -256,6 +257,32 @@ static cudaError_t launch_diag(fhe_ctx *c, const DiagArgs &da, cudaStream_t s) {
   return dep ? diag_go<false, true>(c, da, grid, s) : diag_go<false, false>(c, da, grid, s);
 }
 
+// The baby rotations and the diagonals in one kernel (ip_diag.cuh), up to the kBdGiant giant steps
+// whose sums a warp holds in registers: every further group would read the keys again (1.9 GB of a
+// CoeffToSlot level at L = 48) to spare the baby rotations' 0.9 GB, so more keep the two kernels.
+static bool baby_diag_fits(const fhe_ctx *c, int level, int n_giant) {
+  return c->tabs.ip_staged && n_giant <= kBdGiant && c->beta(level) <= 4 && c->N % kIpChunk == 0;
+}
+
+static cudaError_t launch_baby_diag(fhe_ctx *c, const BabyDiagArgs &a, cudaStream_t s) {
+  static PerDeviceOnce configured;
+  const cudaError_t e = configured.run([] {
+    constexpr int kMax = 227 * 1024;
+    const cudaError_t e0 = cudaFuncSetAttribute(k_baby_diag<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
+    return e0 != cudaSuccess ? e0
+                             : cudaFuncSetAttribute(k_baby_diag<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
+  });
+  if (e != cudaSuccess) return e;
+  const int units = a.nlimb * (int)(c->N / kIhUnit), sms = std::max(1, c->tabs.sms);
+  const int ws = kBdStages * baby_diag_stage_words(a.beta) * 4;  // one warp's ring
+  const int warps = std::max(1, std::min({kBdMaxWarps, 227 * 1024 / ws, (units + sms - 1) / sms}));
+  const unsigned grid = (unsigned)std::min((units + warps - 1) / warps, sms);
+  const bool dep = c->dep_next((size_t)2 * a.giant * a.nlimb);
+  note_launch();
+  c->after_kernel = true;
+  return launch_dep(dep, dep ? k_baby_diag<true> : k_baby_diag<false>, grid, warps * 32, warps * ws, s, a, c->d_pc, c->logn);
+}
+
 // Giant-step accumulation of a double-hoisted transform, in the extended basis:
 //   out_0 = sum_g sigma_g(inner_g,0) + v_g,0,   out_1 = sum_g v_g,1,
 // where v_g is the extended-basis key switch of sigma_g applied to ModDown(inner_g,1); a giant
@@ -483,9 +510,11 @@ extern "C" int fhe_linear_transform(fhe_ctx *c, const uint32_t *ct, int level, c
 // hoisted as well as ModUp):
 //   out = sum_g rot_{giant[g]}( sum_b pt[idx[g][b]] (.) rot_{baby[b]}(ct) ).
 // (1) one ModUp of c1; every baby rotation's inner product stays in the
-//     extended basis Q_l u P, with P sigma_b(c0) folded onto its q-limbs
-//     (IT_IPX); a baby step without rotation is P ct (formed in the diagonal pass);
-// (2) the inner sums are formed in the extended basis (k_diag_bulk over l + K limbs);
+//     extended basis Q_l u P, with P sigma_b(c0) folded onto its q-limbs;
+//     a baby step without rotation is P ct (formed in the diagonal pass);
+// (2) the inner sums are formed in the extended basis, by the kernel that forms
+//     the inner products (k_baby_diag, up to four giant steps), or after them
+//     (IT_IPX, then k_diag_bulk over l + K limbs);
 // (3) per rotating giant step, the c1 half of its inner sum goes down to Q_l
 //     (IT_MDX), is decomposed again (IT_MODUP) and key-switched with sigma_g on the
 //     extended digits (IT_IPX), again without ModDown;
@@ -548,12 +577,14 @@ extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level
     it.ext_slot = 0;
     its.push_back(it);
   }
+  const bool fused = !its.empty() && baby_diag_fits(c, level, n_giant);
   if (!its.empty()) {
     Item up;
     up.kind = IT_MODUP;
     up.level = level;
     up.in = ct + poly;
     up.slot = 0;
+    if (fused) its.clear();  // (their inner products are formed with the diagonals)
     its.insert(its.begin(), up);
     LT_CHECK(run_items_chunked(c, its, 1, s));
   }
@@ -575,7 +606,33 @@ extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level
     if (gb[b] == 1u) da.idmask |= 1u << b;
   da.ct = ct;
   da.pmod = c->d_pmod;
-  {
+  if (fused) {
+    BabyDiagArgs ba;
+    memset(&ba, 0, sizeof ba);
+    for (int b = 0; b < n_baby; b++) {
+      ba.key[b] = kb[b];
+      ba.gal[b] = gb[b];
+    }
+    ba.ct = ct;
+    ba.ext = c->slots[0].EXT;
+    ba.diags = diags;
+    ba.pmod = c->d_pmod;
+    ba.out = inner;
+    ba.giant = n_giant;
+    ba.nlimb = n_ext;
+    ba.level = level;
+    ba.L = c->L;
+    ba.K = K;
+    ba.alpha = c->alpha;
+    ba.beta = c->beta(level);
+    ba.idmask = da.idmask;
+    for (int g = 0; g < n_giant; g++) {
+      ba.gmask[g] = da.gmask[g];
+      for (int b = 0; b < n_baby; b++) ba.didx[g][b] = da.didx[g * n_baby + b];
+    }
+    TraceScope ts(c->tabs, "baby_diag", s);
+    if (launch_baby_diag(c, ba, s) != cudaSuccess) return fhe_fail(FHE_ECUDA, "%s: baby and diagonal kernel", fn);
+  } else {
     TraceScope ts(c->tabs, "diag_mac", s);
     if (launch_diag(c, da, s) != cudaSuccess) return fhe_fail(FHE_ECUDA, "%s: diagonal kernel", fn);
   }
