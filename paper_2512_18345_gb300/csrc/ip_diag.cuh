@@ -1,8 +1,10 @@
-// Baby rotations and diagonals of a double-hoisted transform in one pass: for one unit of an
-// extended limb, every baby step's inner product u_b = sum_j sigma_b(ModUp_j) key_b,j
-// (+ P sigma_b(c0) on the q-limbs) is formed in registers and multiplied at once by the
-// diagonals of up to kBdGiant giant steps, so the baby rotations (two extended polynomials
-// each) are neither written nor read back.
+// A double-hoisted transform's baby rotations and diagonals in one pass (k_baby_diag), and its giant
+// steps' key switches and sum in another (k_giant_ip).
+//
+// k_baby_diag: for one unit of an extended limb, every baby step's inner product
+// u_b = sum_j sigma_b(ModUp_j) key_b,j (+ P sigma_b(c0) on the q-limbs) is formed in registers
+// and multiplied at once by the diagonals of up to kBdGiant giant steps, so the baby rotations
+// (two extended polynomials each) are neither written nor read back.
 //
 // Bound by the keys and the diagonals, both read once, from HBM.  A CoeffToSlot level at N = 2^16,
 // L = 48, alpha = K = 12 (15 rotating baby and 4 giant steps, 63 diagonals): 3.0 GB in 510 us (5.9
@@ -180,6 +182,133 @@ __global__ void __launch_bounds__(kBdMaxWarps * 32, 1)
         }
   }
   cp_async_wait_group<0>();  // nothing in flight when the warp leaves
+}
+
+// Giant steps of a double-hoisted transform, in the extended basis:
+//   out_0 = sum_g sigma_g(inner_g,0) + u_g,0,   out_1 = sum_g u_g,1,
+// u_g the key switch's inner product over the digits of ModDown(inner_g,1) read through sigma_g; a
+// giant step without rotation adds inner_g itself.  The same warp pipelines, one giant step per
+// stage: beta digit rows, the c0 row, 2 beta key rows.  The sums stay in registers, so the u_g
+// (two extended polynomials each) are neither written nor read back.  Bound by HBM: the CoeffToSlot
+// level above (3 rotating giant steps) reads 0.38 GB of keys and 0.27 GB of digits and c0 halves in
+// 113 us, where an inner product and a sum kernel took 150 us (the level 1105 -> 1062 us, the one at
+// N = 2^12 58 -> 50 us); 12 warps instead of 16 differ by less than the runs do.
+constexpr int kGiMaxGiant = 16, kGiMaxWarps = 16, kGiStages = 2;
+struct GiantIpArgs {
+  const uint32_t *key[kGiMaxGiant];    // null: no rotation
+  const uint32_t *ext[kGiMaxGiant];    // [beta][nlimb][N]
+  const uint32_t *own[kGiMaxGiant];    // [level][N]
+  const uint32_t *inner[kGiMaxGiant];  // [2][nlimb][N]
+  uint32_t gal[kGiMaxGiant];
+  uint32_t *out;                       // [2][nlimb][N]
+  int giant, nlimb, level, L, K, alpha, beta;
+};
+__host__ __device__ constexpr int giant_ip_stage_words(int beta) { return kIhUnit * (3 * beta + 1); }
+
+template <bool DEP>
+__global__ void __launch_bounds__(kGiMaxWarps * 32, 1)
+    k_giant_ip(const __grid_constant__ GiantIpArgs a, const PrimeC *pc, int logn) {
+  constexpr int D = kGiStages;
+  extern __shared__ __align__(128) uint8_t smem[];
+  const int warp = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const size_t N = (size_t)1 << logn, poly = (size_t)a.nlimb * N, half = (size_t)(a.L + a.K) * N;
+  const int lpl = logn - 7;
+  const int total = a.nlimb << lpl;
+  const int beta = a.beta, sw = giant_ip_stage_words(beta);
+  const int PR = beta * kIhUnit, KR = PR + kIhUnit;
+  uint32_t *ring = reinterpret_cast<uint32_t *>(smem) + (size_t)warp * D * sw;
+  const uint32_t ring_s = smem_addr(ring);
+  const int wpc = (int)(blockDim.x >> 5);
+  const int gw = (int)blockIdx.x * wpc + warp, nw = (int)gridDim.x * wpc;
+  const uint64_t once = l2_evict_first_policy();  // keys are read exactly once
+  const int eb = l >> 3, part = l & 7;
+  const uint32_t pw = (uint32_t)(eb * 32 + 4 * part);
+
+  int su = gw, sg = 0, ring_at = 0;  // the staging cursor: unit and giant step
+  auto stage = [&] {
+    if (su < total) {
+      const int i = su >> lpl;
+      const uint32_t c0 = (uint32_t)(su & ((1 << lpl) - 1)) * kIhUnit;
+      const uint32_t dst = ring_s + (uint32_t)(ring_at * sw + pw) * 4u;
+      auto row = [&](int words) { return dst + (uint32_t)words * 4u; };
+      const size_t lim = (size_t)i * N;
+      const size_t at = ((size_t)(galois_src(c0 + 32u * (uint32_t)eb, a.gal[sg], logn) >> 5) << 5) + 4 * part;
+      cp_async_plain16(row(PR), a.inner[sg] + lim + at);
+      if (!a.key[sg]) {
+        cp_async_plain16(row(0), a.inner[sg] + poly + lim + at);
+      } else {
+        const int jown = i < a.level ? i / a.alpha : -1;
+        const uint32_t *kp = a.key[sg] + (size_t)(i < a.level ? i : a.L + (i - a.level)) * N + c0 + pw;
+#pragma unroll
+        for (int r = 0; r < 4; r++)
+          if (r < beta) {
+            cp_async_plain16(row(r * kIhUnit), (r == jown ? a.own[sg] : a.ext[sg] + (size_t)r * poly) + lim + at);
+            cp_async16_hint(row(KR + 2 * r * kIhUnit), kp + (size_t)(2 * r) * half, once);
+            cp_async16_hint(row(KR + (2 * r + 1) * kIhUnit), kp + (size_t)(2 * r + 1) * half, once);
+          }
+      }
+      if (++sg == a.giant) {
+        sg = 0;
+        su += nw;
+      }
+    }
+    if (++ring_at == D) ring_at = 0;
+    cp_async_commit();
+  };
+
+  if (DEP) dep_wait();
+#pragma unroll
+  for (int k = 0; k < D - 1; k++) stage();
+  int at = 0;
+  for (int u = gw; u < total; u += nw) {
+    const int i = u >> lpl;
+    const uint32_t c0 = (uint32_t)(u & ((1 << lpl) - 1)) * kIhUnit;
+    const PrimeC P = pc[i < a.level ? i : a.L + (i - a.level)];
+    uint32_t s0[4] = {}, s1[4] = {};
+    for (int g = 0; g < a.giant; g++) {
+      stage();
+      cp_async_wait_group<D - 1>();
+      __syncwarp();
+      const uint32_t *st = ring + (size_t)at * sw;
+      if (++at == D) at = 0;
+      if (!a.key[g]) {
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+          s0[e] = add_mod(s0[e], st[PR + 32 * e + l], P.q);
+          s1[e] = add_mod(s1[e], st[32 * e + l], P.q);
+        }
+      } else {
+        int off[4];
+        uint64_t a0[4] = {}, a1[4] = {};
+#pragma unroll
+        for (int e = 0; e < 4; e++) off[e] = e * 32 + (int)(galois_src(c0 + 32u * e + l, a.gal[g], logn) & 31u);
+#pragma unroll
+        for (int r = 0; r < 4; r++)
+          if (r < beta) {
+            const uint32_t *dr = st + r * kIhUnit, *kb = st + KR + 2 * r * kIhUnit + l;
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+              const uint32_t ev = dr[off[e]];
+              a0[e] += (uint64_t)ev * kb[32 * e];
+              a1[e] += (uint64_t)ev * kb[kIhUnit + 32 * e];
+            }
+          }
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+          s0[e] = add_mod(s0[e], add_mod(reduce_u64(a0[e], P), st[PR + off[e]], P.q), P.q);
+          s1[e] = add_mod(s1[e], reduce_u64(a1[e], P), P.q);
+        }
+      }
+      __syncwarp();
+    }
+    uint32_t *o = a.out + (size_t)i * N + c0 + l;
+#pragma unroll
+    for (int e = 0; e < 4; e++) {
+      o[32 * e] = s0[e];
+      o[poly + 32 * e] = s1[e];
+    }
+  }
+  cp_async_wait_group<0>();
 }
 
 }  // namespace fhe

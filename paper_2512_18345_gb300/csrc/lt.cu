@@ -283,6 +283,32 @@ static cudaError_t launch_baby_diag(fhe_ctx *c, const BabyDiagArgs &a, cudaStrea
   return launch_dep(dep, dep ? k_baby_diag<true> : k_baby_diag<false>, grid, warps * 32, warps * ws, s, a, c->d_pc, c->logn);
 }
 
+// The key switches of the giant steps and their sum in one kernel (ip_diag.cuh), wherever the staged
+// gather is on and the digits fit its rows; else IT_IPX items and k_gsum, which also sums a
+// transform without rotating giant steps (nothing to key-switch).
+static bool giant_ip_fits(const fhe_ctx *c, int level) {
+  return c->tabs.ip_staged && c->beta(level) <= 4 && c->N % kIpChunk == 0;
+}
+
+static cudaError_t launch_giant_ip(fhe_ctx *c, const GiantIpArgs &a, cudaStream_t s) {
+  static PerDeviceOnce configured;
+  const cudaError_t e = configured.run([] {
+    constexpr int kMax = 227 * 1024;
+    const cudaError_t e0 = cudaFuncSetAttribute(k_giant_ip<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
+    return e0 != cudaSuccess ? e0
+                             : cudaFuncSetAttribute(k_giant_ip<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
+  });
+  if (e != cudaSuccess) return e;
+  const int units = a.nlimb * (int)(c->N / kIhUnit), sms = std::max(1, c->tabs.sms);
+  const int ws = kGiStages * giant_ip_stage_words(a.beta) * 4;
+  const int warps = std::max(1, std::min({kGiMaxWarps, 227 * 1024 / ws, (units + sms - 1) / sms}));
+  const unsigned grid = (unsigned)std::min((units + warps - 1) / warps, sms);
+  const bool dep = c->dep_next((size_t)2 * a.nlimb);
+  note_launch();
+  c->after_kernel = true;
+  return launch_dep(dep, dep ? k_giant_ip<true> : k_giant_ip<false>, grid, warps * 32, warps * ws, s, a, c->d_pc, c->logn);
+}
+
 // Giant-step accumulation of a double-hoisted transform, in the extended basis:
 //   out_0 = sum_g sigma_g(inner_g,0) + v_g,0,   out_1 = sum_g v_g,1,
 // where v_g is the extended-basis key switch of sigma_g applied to ModDown(inner_g,1); a giant
@@ -517,8 +543,9 @@ extern "C" int fhe_linear_transform(fhe_ctx *c, const uint32_t *ct, int level, c
 //     (IT_IPX, then k_diag_bulk over l + K limbs);
 // (3) per rotating giant step, the c1 half of its inner sum goes down to Q_l
 //     (IT_MDX), is decomposed again (IT_MODUP) and key-switched with sigma_g on the
-//     extended digits (IT_IPX), again without ModDown;
-// (4) k_gsum adds sigma_g of the c0 halves and the key-switch outputs;
+//     extended digits, again without ModDown;
+// (4) sigma_g of the c0 halves and the key-switch outputs are added: k_giant_ip for
+//     both, or IT_IPX items, then k_gsum;
 // (5) one ModDown of both halves (IT_MDX).
 extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level, const int32_t *baby, int n_baby,
                                        const int32_t *giant, int n_giant, const uint32_t *diags, int n_diag,
@@ -638,6 +665,7 @@ extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level
   }
 
   // (3) rotating giant steps: ModDown of the c1 halves, then ModUp + extended-basis key switch
+  const bool gip = giant_ip_fits(c, level);
   std::vector<int> rg;
   for (int g = 0; g < n_giant; g++)
     if (gg[g] != 1u) rg.push_back(g);
@@ -663,7 +691,7 @@ extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level
       up.slot = 1 + j;
       ks.push_back(up);
     }
-    for (int j = 0; j < ng; j++) {
+    for (int j = 0; j < ng && !gip; j++) {
       const int g = rg[j];
       Item it;
       it.kind = IT_IPX;
@@ -679,25 +707,50 @@ extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level
   }
 
   // (4) giant-step accumulation, (5) one ModDown of both halves
-  GsumArgs ga;
-  memset(&ga, 0, sizeof ga);
-  for (int g = 0; g < n_giant; g++) {
-    ga.inner[g] = inner + g * xct;
-    ga.v[g] = gg[g] != 1u ? v + g * xct : nullptr;
-    ga.galois[g] = gg[g];
-  }
-  ga.out = acc;
-  ga.count = n_giant;
-  ga.nlimb = n_ext;
-  ga.level = level;
-  ga.L = c->L;
-  {
-    TraceScope ts(c->tabs, "lt_gsum", s);
-    const bool dep = c->dep_next((size_t)2 * n_ext);
-    note_launch();
-    c->after_kernel = true;
-    if (launch_dep(dep, dep ? k_gsum<true> : k_gsum<false>, grid_x / kGsumEpt, 256, 0, s, ga, c->d_pc, c->logn) != cudaSuccess)
-      return fhe_fail(FHE_ECUDA, "%s: giant-step sum kernel", fn);
+  if (gip && !rg.empty()) {
+    GiantIpArgs ga;
+    memset(&ga, 0, sizeof ga);
+    for (int g = 0; g < n_giant; g++) {
+      ga.inner[g] = inner + g * xct;
+      ga.gal[g] = gg[g];
+    }
+    for (size_t j = 0; j < rg.size(); j++) {
+      const int g = rg[j];
+      ga.key[g] = kg[g];
+      ga.ext[g] = c->slots[1 + j].EXT;
+      ga.own[g] = c1d + g * poly;
+    }
+    ga.out = acc;
+    ga.giant = n_giant;
+    ga.nlimb = n_ext;
+    ga.level = level;
+    ga.L = c->L;
+    ga.K = K;
+    ga.alpha = c->alpha;
+    ga.beta = c->beta(level);
+    TraceScope ts(c->tabs, "giant_ip", s);
+    if (launch_giant_ip(c, ga, s) != cudaSuccess) return fhe_fail(FHE_ECUDA, "%s: giant-step kernel", fn);
+  } else {
+    GsumArgs ga;
+    memset(&ga, 0, sizeof ga);
+    for (int g = 0; g < n_giant; g++) {
+      ga.inner[g] = inner + g * xct;
+      ga.v[g] = gg[g] != 1u ? v + g * xct : nullptr;
+      ga.galois[g] = gg[g];
+    }
+    ga.out = acc;
+    ga.count = n_giant;
+    ga.nlimb = n_ext;
+    ga.level = level;
+    ga.L = c->L;
+    {
+      TraceScope ts(c->tabs, "lt_gsum", s);
+      const bool dep = c->dep_next((size_t)2 * n_ext);
+      note_launch();
+      c->after_kernel = true;
+      if (launch_dep(dep, dep ? k_gsum<true> : k_gsum<false>, grid_x / kGsumEpt, 256, 0, s, ga, c->d_pc, c->logn) != cudaSuccess)
+        return fhe_fail(FHE_ECUDA, "%s: giant-step sum kernel", fn);
+    }
   }
   Item fin;
   fin.kind = IT_MDX;

@@ -1,5 +1,5 @@
 """The double-hoisted transform's baby rotations and diagonals in one kernel (at most four giant
-steps) and in two (more): one to four digits, partial last digits, one to 32 baby steps, identity
+steps) and in two (more), and its giant steps' key switches and sum in one, up to 16 of them: one to four digits, partial last digits, one to 32 baby steps, identity
 and repeated baby steps, special limbs that meet no step, sparse and full index tables, maximal
 residues (the folds of the accumulators).  Residue for residue against the C oracle on the small
 ring, and on the large one against the two-kernel form, which the oracle checks elsewhere."""
@@ -39,6 +39,9 @@ CASES = [
     ((6, 2, 3, 4), (2, 9, 0), (0, 1, 5, 64), lambda i, b: i == 2, "random"),   # giant steps without any
     ((12, 3, 4, 11), tuple(range(-15, 17)), (0, 100, 200, 300), FULL, "max"),  # 32 baby steps, 4 digits
     ((6, 2, 3, 6), (0, 1, 2, 3), (0, 4, 8, 12, 16), FULL, "max"),              # five giant steps: two kernels
+    ((7, 2, 4, 7), (0, 1), tuple(range(-8, 8)), FULL, "max"),                  # 16 giant steps
+    ((5, 3, 2, 4), (0, 1, 2), (7, 0, 0, 7), FULL, "random"),                   # repeated and identity giant steps
+    ((3, 1, 3, 3), (0, 0), (4, 9), FULL, "max"),                               # no rotating baby step
 ]
 
 
