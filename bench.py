@@ -369,34 +369,28 @@ def bench_bootstrap_lt(binding, inputs, dev, timed, hbm_peak, only=None, runs=0)
         n_ks = sum(sum(1 for r in pl.baby if r % (P.N // 2)) + sum(1 for r in pl.giant if r % (P.N // 2))
                    for pl in plans)
         diag_bytes = sum(pl.n_diag * (lv + P.K) * P.N * 4 for pl, lv in zip(plans, levels))
-        # the diagonal kernel's algorithmic bytes: each diagonal once, each baby rotation once per
-        # group of 4 giant steps, each inner sum written once (extended basis, both halves)
-        mac_bytes = sum((pl.n_diag + 2 * len(pl.baby) * -(-len(pl.giant) // 4) + 2 * len(pl.giant)) *
-                        (lv + P.K) * P.N * 4 for pl, lv in zip(plans, levels))
-        mac_ms = stats.get("diag_mac", (0, 0.0))[1]
-        # the hoisted inner products' algorithmic bytes: per rotating baby step its key and its u
-        # over the extended basis, the shared digit set and pass-through once per level; per
-        # rotating giant step its key, its own digit set and its u
-        ip_words = 0
+        # algorithmic bytes of the two HBM-bound kernels.  Baby inner products and diagonals (at
+        # most 4 giant steps): each rotating baby step's key and each diagonal once, the shared
+        # digit set and the pass-through limbs once, each inner sum written once.  Giant steps:
+        # per rotating one its key, its digits and its c0 half, else both halves; one output.
+        bd_words = gi_words = 0
         for pl, lv in zip(plans, levels):
             beta, ext = P.beta(lv), lv + P.K
             nb = sum(1 for r in pl.baby if r % (P.N // 2))
             ng = sum(1 for r in pl.giant if r % (P.N // 2))
-            if nb:
-                ip_words += nb * (2 * beta + 2) * ext + beta * ext + lv
-            ip_words += ng * (3 * beta + 2) * ext
-        ip_bytes = ip_words * P.N * 4
-        ip_ms = stats.get("inner_product", (0, 0.0))[1]
+            bd_words += (2 * beta * nb + beta + pl.n_diag + 2 * len(pl.giant)) * ext + lv
+            gi_words += ((3 * beta + 1) * ng + 2 * (len(pl.giant) - ng) + 2) * ext
+
+        def streamed(kernel, words):
+            nbytes, kms = words * P.N * 4, stats.get(kernel, (0, 0.0))[1]
+            gbs = nbytes / (kms / 1e3) / 1e9 if kms else None
+            return {"bytes": nbytes, "ms_traced": kms, "gbs": gbs, "frac_of_measured_hbm": gbs / hbm_peak if kms else None}
+
         res[kind] = {
             "ms": ms, "levels": levels, "key_switches": n_ks, "ks_per_s": n_ks / (ms / 1e3),
             "diagonals": [pl.n_diag for pl in plans], "baby_giant": [[len(pl.baby), len(pl.giant)] for pl in plans],
             "diagonal_bytes": diag_bytes, "hbm_floor_ms": diag_bytes / (hbm_peak * 1e9) * 1e3,
-            "diag_mac": {"bytes": mac_bytes, "ms_traced": mac_ms,
-                         "gbs": mac_bytes / (mac_ms / 1e3) / 1e9 if mac_ms else None,
-                         "frac_of_measured_hbm": (mac_bytes / (mac_ms / 1e3) / 1e9) / hbm_peak if mac_ms else None},
-            "inner_product": {"bytes": ip_bytes, "ms_traced": ip_ms,
-                              "gbs": ip_bytes / (ip_ms / 1e3) / 1e9 if ip_ms else None,
-                              "frac_of_measured_hbm": (ip_bytes / (ip_ms / 1e3) / 1e9) / hbm_peak if ip_ms else None},
+            "baby_diag": streamed("baby_diag", bd_words), "giant_ip": streamed("giant_ip", gi_words),
             "kernels_ms": {k2: round(v[1], 4) for k2, v in sorted(stats.items(), key=lambda kv: -kv[1][1])}}
         del pts, outs, resc
     ctx.close()
