@@ -192,7 +192,10 @@ FHE_API int fhe_ctx_set_ntt(fhe_ctx *ctx, int flags);
  *     32-coefficient blocks into shared memory with bulk copies, so that every
  *     digit value is a shared-memory read; 0 gathers them with 4-byte global
  *     loads.  Launches that add the pass-through polynomial to both halves
- *     (relinearisation) use the gathering kernel either way;
+ *     (relinearisation) use the gathering kernel either way; with 1
+ *     fhe_linear_transform_dh also forms its inner products inside the kernels
+ *     that use them (baby steps: up to 4 giant steps), with 0 in kernels of
+ *     their own.  Results are the same;
  *   ip_staged_ctas, ip_staged_depth: resident CTAs per SM (1: one CTA of up
  *     to 227 KB of shared memory; 2: two of up to 113 KB) and stages per warp
  *     (2..4; 0: 2) of that staged kernel, whose warps each run their own
