@@ -433,7 +433,7 @@ cudaError_t launch_ip(const DevTables &t, const SegList &sl, bool gather_own, bo
     return t.dep ? IP_GO(false, false, false, true) : IP_GO(false, false, false, false);
 #undef IP_GO
   }
-  return cudaErrorInvalidValue;  // (contexts have at most four digits)
+  return cudaErrorInvalidValue;  // (a context's polynomials have at most four digits, whatever its dnum)
 }
 
 cudaError_t launch_ew(const DevTables &t, int op, const SegList &sl, cudaStream_t s) {

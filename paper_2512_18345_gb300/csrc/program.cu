@@ -448,10 +448,10 @@ static cudaError_t launch_stage(fhe_ctx *c, const Stage &st, const SegList &sl, 
     case Stage::NTT: return launch_ntt_pass(c->tabs, st.column, st.fwd, st.pro, st.epi, sl, q);
     case Stage::NTT1: return launch_ntt_single(c->tabs, st.fwd, st.pro, st.epi, sl, *sl2, q);
     case Stage::EW: return launch_ew(c->tabs, st.ewop, sl, q);
-    case Stage::IP: return launch_ip(c->tabs, sl, st.gather_own, st.gather_ext, st.add_c1, st.mul, c->dnum, q);
+    case Stage::IP: return launch_ip(c->tabs, sl, st.gather_own, st.gather_ext, st.add_c1, st.mul, c->beta(c->L), q);
     case Stage::SNTT: return launch_small_ntt(c->tabs, st.fwd, st.pro, st.epi, sl, q);
     case Stage::SIP: return launch_small_ip(c->tabs, sl, st.mul, q);
-    case Stage::IPN: return launch_ip_intt(c->tabs, sl, std::min(c->dnum, 4), q);
+    case Stage::IPN: return launch_ip_intt(c->tabs, sl, c->beta(c->L), q);
     case Stage::BCONV:
       return c->bconv_mode == FHE_BCONV_TC ? launch_bconv_tc(c->tabs, ba, st.max_in, st.max_out, q, c->tabs.tc_k)
                                            : launch_bconv(c->tabs, ba, st.max_in, st.max_out, q);
