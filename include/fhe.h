@@ -387,8 +387,9 @@ FHE_API int fhe_ctx_set_batch(fhe_ctx *ctx, size_t l2_budget_bytes, int max_grou
 /*
  * Schedule autotuner (Section IV-A batching, Section IV-C graphs): measures
  * graph-captured plans of n_items (1..64) synthetic key switches at `level`
- * on `stream` for every candidate schedule -- lanes 1..4, group budgets of
- * 3/4, 1, 2 and 4 times the device's L2, one or two resident CTAs per SM for
+ * on `stream` for every candidate schedule -- lanes 1..4, the default grouping
+ * (budget 0 of fhe_ctx_set_batch; kept where an explicit budget ties with it)
+ * and group budgets of 3/4, 1, 2 and 4 times the device's L2, one or two resident CTAs per SM for
  * the streaming inner product (one leaves room for transforms beside it; it is
  * chosen only when more than 2 % faster than the best two-CTA schedule),
  * complementary pipelining (Section IV-B) on or off, and,
@@ -405,12 +406,12 @@ FHE_API int fhe_ctx_set_batch(fhe_ctx *ctx, size_t l2_budget_bytes, int max_grou
 #define FHE_TUNE_SHAPE 4 /* then also measure kernel shapes (fhe_ctx_set_kernel_shape) one parameter at a time */
 typedef struct {
   int lanes;              /* chosen lane count */
-  size_t l2_budget_bytes; /* chosen group budget */
+  size_t l2_budget_bytes; /* chosen group budget (0: the default grouping) */
   int max_group;          /* chosen group cap (0: default) */
   int bconv_mode;         /* chosen BConv kernel */
   int n_groups;           /* groups of the measured plan */
   double us_per_ks;       /* measured time per key switch of the chosen schedule, microseconds */
-  double default_us_per_ks; /* the same for the default schedule (2 lanes, 2 x L2, 2 CTAs), 0 if not measured */
+  double default_us_per_ks; /* the same for the default schedule (2 lanes, default grouping, 2 CTAs), 0 if not measured */
   int candidates;         /* distinct schedules measured */
   int ip_ctas_per_sm;     /* chosen residency of the streaming inner product */
   int comp_pipe;          /* 1: complementary pipelining (q-limb inner product on its own branch) */
@@ -423,8 +424,8 @@ FHE_API int fhe_autotune(fhe_ctx *ctx, int level, int n_items, int flags, fhe_tu
  * an entry for this context's (N, level, K, alpha, dnum), n_items, flags and
  * GPU (name and SM count) is applied without measuring (out->candidates = 0);
  * otherwise the schedules are measured as by fhe_autotune and the choice is
- * appended to the file.  Malformed lines are skipped; the last matching entry
- * wins.  FHE_EINVAL if the file cannot be appended to.
+ * appended to the file.  Malformed lines, and entries recorded before the default
+ * grouping was a candidate, are skipped; the last matching entry wins.  FHE_EINVAL if the file cannot be appended to.
  */
 FHE_API int fhe_autotune_cached(fhe_ctx *ctx, const char *path, int level, int n_items, int flags,
                                 fhe_tune_result *out, fhe_stream stream);

@@ -96,7 +96,9 @@ extern "C" int fhe_autotune(fhe_ctx *c, int level, int n_items, int flags, fhe_t
     if (fhe_ctx_set_bconv(c, FHE_BCONV_TC) == FHE_OK) modes.push_back(FHE_BCONV_TC);
     c->bconv_mode = saved_mode;
   }
-  const size_t budgets[] = {(size_t)l2 * 3 / 4, (size_t)l2, (size_t)l2 * 2, (size_t)l2 * 4};
+  // budget 0 is the default grouping (fhe_ctx_set_batch), which no explicit budget gives beyond
+  // 8 items; first, so that it is the one kept where another budget forms the same groups
+  const size_t budgets[] = {0, (size_t)l2 * 3 / 4, (size_t)l2, (size_t)l2 * 2, (size_t)l2 * 4};
   std::map<std::tuple<int, int, std::vector<int>>, double> seen;  // (mode, lanes, group sizes) -> us per KS
   fhe_tune_result best;
   memset(&best, 0, sizeof best);
@@ -148,7 +150,7 @@ extern "C" int fhe_autotune(fhe_ctx *c, int level, int n_items, int flags, fhe_t
         const int ng = fhe_plan_groups(p, gs.data(), 64);
         gs.resize(std::min(ng, 64));
         const int eff_lanes = std::min(lanes, ng);
-        const bool is_default = mode == saved_mode && comp == 1 && ipc == 2 && lanes == 2 && budget == budgets[2];
+        const bool is_default = mode == saved_mode && comp == 1 && ipc == 2 && lanes == 2 && budget == 0;
         const auto key = std::make_tuple(mode * 8 + comp * 4 + ipc, eff_lanes, gs);
         auto found = seen.find(key);
         if (found != seen.end()) {  // the same schedule as one already measured
@@ -304,8 +306,10 @@ extern "C" int fhe_autotune(fhe_ctx *c, int level, int n_items, int flags, fhe_t
   return rc;
 }
 
-// ---- tuning cache: one text line per (ring, level, special primes, digit size, batch,
-// flags, GPU) -> chosen schedule; the last matching line wins, unreadable lines are skipped.
+// ---- tuning cache: one text line per (set of candidates, ring, level, special primes, digit size,
+// batch, flags, GPU) -> chosen schedule; the last matching line wins, unreadable lines are skipped.
+// sched=2: the candidates include the default grouping; entries without it were chosen among
+// explicit budgets alone and are measured again.
 
 static std::string tune_key(const fhe_ctx *c, int level, int n_items, int flags) {
   cudaDeviceProp prop;
@@ -315,7 +319,7 @@ static std::string tune_key(const fhe_ctx *c, int level, int n_items, int flags)
   for (char &ch : gpu)
     if (ch == ' ' || ch == '|') ch = '_';
   char buf[384];
-  snprintf(buf, sizeof buf, "N=%zu level=%d K=%d alpha=%d dnum=%d items=%d flags=%d gpu=%s sms=%d", (size_t)c->N,
+  snprintf(buf, sizeof buf, "sched=2 N=%zu level=%d K=%d alpha=%d dnum=%d items=%d flags=%d gpu=%s sms=%d", (size_t)c->N,
            level, c->K, c->alpha, c->dnum, n_items, flags, gpu.c_str(), prop.multiProcessorCount);
   return buf;
 }
