@@ -86,10 +86,14 @@ extern "C" int fhe_ctx_set_batch(fhe_ctx *c, size_t l2_budget_bytes, int max_gro
 // equal shares of at least one group per lane, of about twice that size or kWideGroup items --
 // the stage kernels are bound by instruction issue, and large launches amortise their ramp and
 // their last wave better than L2 residency saves (64 mixed items at N = 2^16: groups of 16 on two
-// lanes 2342 us, of 8 2422; 8 rotations: 4 + 4 and 5 + 3 within 0.3 %).  Every group item of every
-// lane holds a workspace slot; where memory (or the context's limit) is short of the default's,
-// the smaller groups of twice the L2 and 8 items are taken.
-static constexpr int kWideGroup = 16;
+// lanes 2342 us, of 8 2422; 8 rotations: 4 + 4 and 5 + 3 within 0.3 %).  Shares are of equal working
+// set, so items of low levels may crowd one (10 items at level 24 and 54 at level 1: 40 in the last).
+// Every group item of every lane holds a workspace slot sized for the top level, so a share of more
+// than kMostGroup items (kMostSlots over the lanes) is cut into equal parts; 64 items spread evenly
+// over levels 4..24 have shares of up to 23.  The smaller groups of twice the L2 and 8 items are
+// taken where a share comes out empty and where memory (or the context's limit) is short of the
+// larger ones' slots.
+static constexpr int kWideGroup = 16, kMostGroup = 24, kMostSlots = 2 * kMostGroup;
 static std::vector<std::vector<int>> make_groups(const fhe_ctx *c, const fhe_ks_item *items, int n) {
   const int nl = std::max(1, c->batch_lanes);
   size_t l2x2 = 0, total = 0;
@@ -119,17 +123,25 @@ static std::vector<std::vector<int>> make_groups(const fhe_ctx *c, const fhe_ks_
     size_t count = std::max<size_t>(nl, (total + 2 * budget - 1) / (2 * budget));
     count = std::max<size_t>(count, (n + kWideGroup - 1) / kWideGroup);
     count = std::min<size_t>((count + nl - 1) / nl * nl, n);  // the same number on every lane
-    std::vector<std::vector<int>> groups(count);
     size_t before = 0;
-    for (int i = 0; i < n; i++) {  // item i's middle decides its share (shares are never left empty)
+    std::vector<std::vector<int>> shares(count), groups;
+    for (int i = 0; i < n; i++) {  // item i's middle decides its share
       size_t g = std::min(count - 1, (size_t)((before + fp[i] / 2) * (double)count / total));
       before += fp[i];
-      groups[g].push_back(i);
+      shares[g].push_back(i);
     }
+    const size_t cap = std::max(8, std::min(kMostGroup, kMostSlots / nl));
     size_t most = 0;
     bool ok = true;
-    for (auto &g : groups) most = std::max(most, g.size()), ok = ok && !g.empty();
-    const size_t lanes = std::min<size_t>(nl, count), have = c->slots.size(), need = lanes * most;
+    for (auto &s : shares) {
+      ok = ok && !s.empty();
+      const size_t parts = (s.size() + cap - 1) / cap;
+      for (size_t k = 0; k < parts; k++) {
+        groups.emplace_back(s.begin() + s.size() * k / parts, s.begin() + s.size() * (k + 1) / parts);
+        most = std::max(most, groups.back().size());
+      }
+    }
+    const size_t lanes = std::min<size_t>(nl, groups.size()), have = c->slots.size(), need = lanes * most;
     const size_t grow = need > have ? (need - have) * c->slot_bytes : 0;
     size_t avail = 0, all = 0;
     if (cudaMemGetInfo(&avail, &all) != cudaSuccess) avail = 0;
