@@ -378,7 +378,9 @@ FHE_API int fhe_plan_groups(const fhe_plan *plan, int *sizes, int max);
  * the device's L2), a group holds at most max_group items (0: 8; with both 0,
  * plans beyond that budget get equal groups of about 16 items or twice the
  * budget, the same number on every lane, none of more than 24 items, or of 48
- * over the lanes (8 at least), where memory allows), and groups
+ * over the lanes (8 at least); the smaller groups where half of the device's
+ * free memory is short of their workspace, and under fhe_ctx_set_memory_limit
+ * unless the context holds that workspace already), and groups
  * run round-robin on `lanes` concurrent streams (0: 2), each lane with its own
  * workspace, so that one group's DRAM-bound inner product overlaps another
  * group's transforms.  fhe_autotune measures and sets these.

@@ -91,8 +91,9 @@ extern "C" int fhe_ctx_set_batch(fhe_ctx *c, size_t l2_budget_bytes, int max_gro
 // Every group item of every lane holds a workspace slot sized for the top level, so a share of more
 // than kMostGroup items (kMostSlots over the lanes) is cut into equal parts; 64 items spread evenly
 // over levels 4..24 have shares of up to 23.  The smaller groups of twice the L2 and 8 items are
-// taken where a share comes out empty and where memory (or the context's limit) is short of the
-// larger ones' slots.
+// taken where a share comes out empty, where half of the device's free memory is short of the
+// larger ones' slots, and under a memory limit unless the context holds those slots already (the
+// room is later calls').
 static constexpr int kWideGroup = 16, kMostGroup = 24, kMostSlots = 2 * kMostGroup;
 static std::vector<std::vector<int>> make_groups(const fhe_ctx *c, const fhe_ks_item *items, int n) {
   const int nl = std::max(1, c->batch_lanes);
@@ -144,8 +145,8 @@ static std::vector<std::vector<int>> make_groups(const fhe_ctx *c, const fhe_ks_
     const size_t lanes = std::min<size_t>(nl, groups.size()), have = c->slots.size(), need = lanes * most;
     const size_t grow = need > have ? (need - have) * c->slot_bytes : 0;
     size_t avail = 0, all = 0;
-    if (cudaMemGetInfo(&avail, &all) != cudaSuccess) avail = 0;
-    if (ok && grow < avail / 2 && !(c->mem_limit && c->grown_bytes + grow > c->mem_limit)) return groups;
+    if (grow && cudaMemGetInfo(&avail, &all) != cudaSuccess) avail = 0;
+    if (ok && (!grow || (!c->mem_limit && grow < avail / 2))) return groups;
   }
   return split(budget, c->batch_max_group > 0 ? c->batch_max_group : 8);
 }

@@ -1,6 +1,6 @@
-"""What a default plan may hold: groups stay within a bound whatever the mix of levels, and a share
-that comes out empty falls back to the smaller groups.  Every grouping gives the single calls'
-residues."""
+"""What a default plan may hold: groups stay within a bound whatever the mix of levels, a context
+with a memory limit keeps the smaller groups (room that later calls need), and a share that comes
+out empty falls back to them.  Every grouping gives the single calls' residues."""
 import pytest
 
 from paper_2512_18345_gb300 import inputs
@@ -63,5 +63,32 @@ def test_empty_share_falls_back(fhe_lib):
     items = rotations(P, residues, [24, 24, 24, 1, 1])
     plan = ctx.batch_plan(items)
     assert sum(plan.groups) == 5 and min(plan.groups) > 0
+    check(ctx, plan, items)
+    ctx.close()
+
+
+def test_a_limit_leaves_room_for_later_calls(fhe_lib):
+    """A limit that holds what a plan of 33 items takes without one, and less than a transform's
+    scratch beside it: the limited plan takes less, and the transform finds room."""
+    import torch
+    P, ctx, residues = context()
+    info, level, baby, giant = ctx.info(), 6, 1, 2
+    items = rotations(P, residues, [3 + (k * 7) % 22 for k in range(33)])
+    rk = residues(P.primes, P.dnum, 2)
+    ct, diags = residues(P.q[:level], 2), residues(P.q[:level], baby * giant)
+    plan = ctx.batch_plan(items)
+    slots = 2 * max(plan.groups)
+    assert slots > 16
+    check(ctx, plan, items)
+    ctx.set_rot_key(1, rk)
+    want = ctx.linear_transform(ct, level, diags, baby, giant)
+    ctx.close()
+    P, ctx, _ = context()
+    ctx.set_rot_key(1, rk)
+    ctx.set_memory_limit(2 * info["key_bytes"] + slots * info["workspace_bytes"] + 2 * level * P.N * 4)
+    plan = ctx.batch_plan(items)
+    assert max(plan.groups) <= 8
+    assert torch.equal(ctx.linear_transform(ct, level, diags, baby, giant), want)
+    ctx.set_memory_limit(0)
     check(ctx, plan, items)
     ctx.close()
