@@ -514,15 +514,13 @@ static cudaError_t bconv_tc_go(const DevTables &t, const BconvArgs &a, int max_o
         [] { return cudaFuncSetAttribute(k_bconv_tc_pipe<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448); });
     if (ce2 != cudaSuccess) return ce2;
     const int grid2 = std::min(total, std::max(1, sms * per_sm2));
-    k_bconv_tc_pipe<KT><<<grid2, kTcThreads, smem2, s>>>(a, t.pc, t.logn, t.status, npad, tiles_per_group);
-  } else {
-    const int grid = std::min(total, std::max(1, sms * per_sm));
-    const cudaError_t le = launch_dep(t.dep, t.dep ? k_bconv_tc<KT, true> : k_bconv_tc<KT, false>, grid, kTcThreads, smem, s, a, t.pc, t.logn, t.status, npad,
-                                      tiles_per_group);
-    if (le != cudaSuccess) return le;
+    note_launch();
+    return launch_dep(false, k_bconv_tc_pipe<KT>, grid2, kTcThreads, smem2, s, a, t.pc, t.logn, t.status, npad, tiles_per_group);
   }
+  const int grid = std::min(total, std::max(1, sms * per_sm));
   note_launch();
-  return cudaGetLastError();
+  return launch_dep(t.dep, t.dep ? k_bconv_tc<KT, true> : k_bconv_tc<KT, false>, grid, kTcThreads, smem, s, a, t.pc, t.logn,
+                    t.status, npad, tiles_per_group);
 }
 
 cudaError_t launch_bconv_tc(const DevTables &t, const BconvArgs &a, int max_in, int max_out, cudaStream_t s, int kt) {

@@ -100,7 +100,11 @@ void fhe_ctx::order_stream(cudaStream_t s) {
   // would mix with programmatic edges
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   after_kernel = false;
-  dep_ok = !capturing && !tabs.tracer && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+    cudaGetLastError();  // (the call's own launches report it)
+    cap = cudaStreamCaptureStatusInvalidated;
+  }
+  dep_ok = !capturing && !tabs.tracer && cap == cudaStreamCaptureStatusNone;
   if (capturing) return;
   if (have_last && s != last_stream) {
     cudaEventRecord(order_ev, last_stream);

@@ -94,7 +94,8 @@ struct TraceScope {
 void note_launch();
 
 // Launch a kernel; with `dep` (only for a kernel that begins with dep_wait, common.cuh) it may
-// start while the kernel before it on the stream is still running.
+// start while the kernel before it on the stream is still running.  A refused launch is reported
+// here alone: left pending on the thread it would fail the next call that asks.
 template <class... P, class... A>
 cudaError_t launch_dep(bool dep, void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s,
                        const A &...args) {
@@ -108,7 +109,9 @@ cudaError_t launch_dep(bool dep, void (*kern)(P...), dim3 grid, unsigned block, 
   cfg.stream = s;
   cfg.attrs = &attr;
   cfg.numAttrs = dep ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
 }
 // the block passes' lo-round twiddles in thread order, from the bit-reversed table (legacy stream)
 cudaError_t build_lo_table(const uint2 *tw, uint4 *lo, int logn, int nprimes);

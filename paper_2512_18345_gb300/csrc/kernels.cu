@@ -86,10 +86,8 @@ static cudaError_t ntt_col_go(const DevTables &t, const SegList &sl, cudaStream_
 
 cudaError_t build_lo_table(const uint2 *tw, uint4 *lo, int logn, int nprimes) {
   const size_t n = (size_t)nprimes << (logn - 1);
-  cudaLaunchConfig_t cfg = {};  // (its own status: an earlier call's error may be pending on this thread)
-  cfg.gridDim = dim3((unsigned)((n + 255) / 256));
-  cfg.blockDim = dim3(256);
-  return cudaLaunchKernelEx(&cfg, k_lo_table, tw, lo, logn, nprimes);
+  // (its own status: an earlier call's error may be pending on this thread)
+  return launch_dep(false, k_lo_table, dim3((unsigned)((n + 255) / 256)), 256, 0, nullptr, tw, lo, logn, nprimes);
 }
 
 // Streaming pass (ntt_bulk.cuh): persistent CTAs, two per SM, each walking a contiguous
