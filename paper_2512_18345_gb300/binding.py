@@ -170,7 +170,7 @@ def check(rc: int) -> None:
 # integers for pointers and streams, torch looked up once, the current stream's handle without a
 # Stream object, devices by their cached torch.device (11 -> 4 us a call).
 _torch = None
-_devices: dict = {}
+_devices: dict = {}  # by name
 
 
 def _cuda():
@@ -215,10 +215,11 @@ def to_numpy(t) -> np.ndarray:
 
 def empty(shape, device: int = 0):
     torch = _cuda()
-    dev = _devices.get(device)
+    name = f"cuda:{device}"
+    dev = _devices.get(name)
     if dev is None:
-        dev = _devices[device] = torch.device("cuda", device)
-    return torch.empty(shape, dtype=torch.int32, device=dev)
+        dev = _devices[name] = torch.device(name)
+    return torch.empty(tuple(shape), dtype=torch.int32, device=dev)
 
 
 def probe_bandwidth(device: int = 0, nbytes: int = 64 << 20, reps: int = 50) -> dict:
