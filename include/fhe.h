@@ -274,7 +274,10 @@ FHE_API int fhe_rotate_hoisted(fhe_ctx *ctx, const uint32_t *ct, int level, cons
  * out [2][level][N] (must not overlap ct).  The baby rotations share one ModUp
  * (as fhe_rotate_hoisted); the giant rotations are ordinary rotations.  Needs the
  * rotation keys of 1..baby-1 and baby g (g = 1..giant-1).  baby <= 32, giant <= 16.
- * No rescale.  The context grows a scratch buffer of (baby + 2 giant) ciphertexts.
+ * No rescale.  The context grows a scratch buffer of (baby + giant) ciphertexts,
+ * and giant - 1 more for the giant rotations where these are formed one by one
+ * (N = 2^12, the plain pipeline, fhe_ctx_set_ntt modes other than 0, a giant step
+ * that is the identity).
  */
 FHE_API int fhe_linear_transform(fhe_ctx *ctx, const uint32_t *ct, int level, const uint32_t *diags, int baby,
                                  int giant, uint32_t *out, fhe_stream stream);
@@ -299,8 +302,11 @@ FHE_API int fhe_linear_transform(fhe_ctx *ctx, const uint32_t *ct, int level, co
  *   idx    [n_giant][n_baby] (host) index into diags, or -1 where the pair has
  *          no diagonal;
  *   out    [2][level][N] (device), must not overlap ct or diags.
- * No rescale.  The context grows a scratch buffer of (n_baby + 2 n_giant + 1)
- * extended-basis ciphertexts plus n_giant polynomials.  Errors: FHE_EINVAL (null,
+ * No rescale.  The context grows a scratch buffer of (n_giant + 1) extended-basis
+ * ciphertexts and one polynomial per rotating giant step; with more than 4 giant
+ * steps, or ip_staged_gather = 0 (fhe_ctx_set_kernel_shape), one more
+ * extended-basis ciphertext per rotating baby step, and with ip_staged_gather = 0
+ * one per rotating giant step.  Errors: FHE_EINVAL (null,
  * misaligned, counts or idx out of range, n_diag > 32767), FHE_ELEVEL, FHE_ENOKEY, FHE_EALIAS,
  * FHE_ENOMEM, FHE_ECUDA.
  */

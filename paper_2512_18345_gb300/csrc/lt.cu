@@ -434,8 +434,11 @@ extern "C" int fhe_linear_transform(fhe_ctx *c, const uint32_t *ct, int level, c
   const size_t N = c->N, poly = (size_t)level * N, ct_words = 2 * poly;
   cudaSetDevice(c->device);
   cudaStream_t s = (cudaStream_t)stream;
-  // scratch: baby rotations, inner sums, giant rotations
-  int rc = ensure_lt_scratch(c, ct_words * ((size_t)baby + 2 * giant));
+  int rotating = 0;  // giant steps
+  for (int g = 1; g < giant; g++) rotating += fhe_galois_elt(baby * g, c->N) != 1u;
+  const bool merged = merge_moddowns(c) && rotating == giant - 1 && giant > 1;
+  // scratch: baby rotations, inner sums and, where their ModDowns are not merged, giant rotations
+  int rc = ensure_lt_scratch(c, ct_words * ((size_t)baby + giant + (merged ? 0 : giant - 1)));
   if (rc != FHE_OK) return rc;
   uint32_t *babies = c->lt_scratch, *inner = babies + baby * ct_words, *grot = inner + giant * ct_words;
   std::vector<int32_t> rots(baby);
@@ -467,7 +470,7 @@ extern "C" int fhe_linear_transform(fhe_ctx *c, const uint32_t *ct, int level, c
   for (int g = 1; g < giant; g++) {
     const uint32_t k = fhe_galois_elt(baby * g, c->N);
     if (k == 1u) {
-      if (cudaMemcpyAsync(grot + g * ct_words, inner + g * ct_words, 4 * ct_words, cudaMemcpyDeviceToDevice, s) !=
+      if (cudaMemcpyAsync(grot + (g - 1) * ct_words, inner + g * ct_words, 4 * ct_words, cudaMemcpyDeviceToDevice, s) !=
           cudaSuccess)
         return fhe_fail(FHE_ECUDA, "fhe_linear_transform: copy");
       c->after_kernel = false;
@@ -478,11 +481,11 @@ extern "C" int fhe_linear_transform(fhe_ctx *c, const uint32_t *ct, int level, c
     it.level = level;
     it.galois = k;
     it.in = inner + g * ct_words;
-    it.out = grot + g * ct_words;
+    it.out = grot + (g - 1) * ct_words;
     it.key = c->find_key(baby * g);
     its.push_back(it);
   }
-  if (merge_moddowns(c) && (int)its.size() == giant - 1 && giant > 1) {
+  if (merged) {
     // out = inner_0 + sum_g rot_{B g}(inner_g) with the rotations' ModDowns merged into one
     // transform of the output's limbs (as many rotations per program as its launch arguments
     // hold; a further program adds to out)
@@ -515,7 +518,7 @@ extern "C" int fhe_linear_transform(fhe_ctx *c, const uint32_t *ct, int level, c
   SumArgs sa;
   memset(&sa, 0, sizeof sa);
   sa.in[0] = inner;
-  for (int g = 1; g < giant; g++) sa.in[g] = grot + g * ct_words;
+  for (int g = 1; g < giant; g++) sa.in[g] = grot + (g - 1) * ct_words;
   sa.count = giant;
   sa.out = out;
   sa.level = level;
@@ -580,46 +583,50 @@ extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level
   cudaSetDevice(c->device);
   cudaStream_t s = (cudaStream_t)stream;
   c->order_stream(s);
-  // scratch: baby rotations, inner sums and giant key switches (extended basis, two
-  // halves each), the giant steps' c1 halves in Q_l, the accumulator
-  const size_t xct = 2 * xpoly;
-  int rc = ensure_lt_scratch(c, xct * ((size_t)n_baby + 2 * n_giant + 1) + poly * n_giant);
+  std::vector<int> rb, rg;  // the rotating baby and giant steps
+  for (int b = 0; b < n_baby; b++)
+    if (gb[b] != 1u) rb.push_back(b);
+  for (int g = 0; g < n_giant; g++)
+    if (gg[g] != 1u) rg.push_back(g);
+  const bool fused = !rb.empty() && baby_diag_fits(c, level, n_giant), gip = giant_ip_fits(c, level);
+  // scratch: inner sums and the accumulator (extended basis, two halves each), the rotating giant
+  // steps' c1 halves in Q_l and, where the kernels that use them do not form them, the rotating
+  // baby steps and the giant key switches
+  const size_t xct = 2 * xpoly, n_bab = fused ? 0 : rb.size(), n_v = gip ? 0 : rg.size();
+  int rc = ensure_lt_scratch(c, xct * (n_bab + n_giant + n_v + 1) + poly * rg.size());
   if (rc != FHE_OK) return rc;
-  uint32_t *bab = c->lt_scratch, *inner = bab + n_baby * xct, *v = inner + n_giant * xct, *acc = v + n_giant * xct,
+  uint32_t *bab = c->lt_scratch, *inner = bab + n_bab * xct, *v = inner + n_giant * xct, *acc = v + n_v * xct,
            *c1d = acc + xct;
   const unsigned grid_x = (unsigned)(n_ext * (N / 256));
 
   // (1) baby steps
-  std::vector<Item> its;
-  for (int b = 0; b < n_baby; b++) {
-    if (gb[b] == 1u) continue;  // (the diagonal pass reads ct itself)
-    Item it;
-    it.kind = IT_IPX;
-    it.level = level;
-    it.galois = gb[b];
-    it.in = ct + poly;
-    it.in2 = ct;
-    it.out = bab + b * xct;
-    it.key = kb[b];
-    it.ext_slot = 0;
-    its.push_back(it);
-  }
-  const bool fused = !its.empty() && baby_diag_fits(c, level, n_giant);
-  if (!its.empty()) {
+  // (the diagonal pass reads ct itself for a step without rotation)
+  if (!rb.empty()) {
     Item up;
     up.kind = IT_MODUP;
     up.level = level;
     up.in = ct + poly;
     up.slot = 0;
-    if (fused) its.clear();  // (their inner products are formed with the diagonals)
-    its.insert(its.begin(), up);
+    std::vector<Item> its{up};
+    for (size_t j = 0; j < n_bab; j++) {
+      Item it;
+      it.kind = IT_IPX;
+      it.level = level;
+      it.galois = gb[rb[j]];
+      it.in = ct + poly;
+      it.in2 = ct;
+      it.out = bab + j * xct;
+      it.key = kb[rb[j]];
+      it.ext_slot = 0;
+      its.push_back(it);
+    }
     LT_CHECK(run_items_chunked(c, its, 1, s));
   }
 
   // (2) inner sums in the extended basis
   DiagArgs da;
   memset(&da, 0, sizeof da);
-  for (int b = 0; b < n_baby; b++) da.babies[b] = bab + b * xct;
+  for (size_t j = 0; j < n_bab; j++) da.babies[rb[j]] = bab + j * xct;
   da.diags = diags;
   da.out = inner;
   da.nb = n_baby;
@@ -665,29 +672,25 @@ extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level
   }
 
   // (3) rotating giant steps: ModDown of the c1 halves, then ModUp + extended-basis key switch
-  const bool gip = giant_ip_fits(c, level);
-  std::vector<int> rg;
-  for (int g = 0; g < n_giant; g++)
-    if (gg[g] != 1u) rg.push_back(g);
   if (!rg.empty()) {
+    const int ng = (int)rg.size();
     std::vector<Item> md;
-    for (int g : rg) {
+    for (int j = 0; j < ng; j++) {
       Item it;
       it.kind = IT_MDX;
       it.level = level;
       it.npoly = 1;
-      it.in = inner + g * xct + xpoly;
-      it.out = c1d + g * poly;
+      it.in = inner + rg[j] * xct + xpoly;
+      it.out = c1d + j * poly;
       md.push_back(it);
     }
     LT_CHECK(run_items_chunked(c, md, 1, s));
     std::vector<Item> ks;
-    const int ng = (int)rg.size();
     for (int j = 0; j < ng; j++) {
       Item up;
       up.kind = IT_MODUP;
       up.level = level;
-      up.in = c1d + rg[j] * poly;
+      up.in = c1d + j * poly;
       up.slot = 1 + j;
       ks.push_back(up);
     }
@@ -697,8 +700,8 @@ extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level
       it.kind = IT_IPX;
       it.level = level;
       it.galois = gg[g];
-      it.in = c1d + g * poly;
-      it.out = v + g * xct;
+      it.in = c1d + j * poly;
+      it.out = v + j * xct;
       it.key = kg[g];
       it.ext_slot = 1 + j;
       ks.push_back(it);
@@ -718,7 +721,7 @@ extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level
       const int g = rg[j];
       ga.key[g] = kg[g];
       ga.ext[g] = c->slots[1 + j].EXT;
-      ga.own[g] = c1d + g * poly;
+      ga.own[g] = c1d + j * poly;
     }
     ga.out = acc;
     ga.giant = n_giant;
@@ -735,9 +738,9 @@ extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level
     memset(&ga, 0, sizeof ga);
     for (int g = 0; g < n_giant; g++) {
       ga.inner[g] = inner + g * xct;
-      ga.v[g] = gg[g] != 1u ? v + g * xct : nullptr;
       ga.galois[g] = gg[g];
     }
+    for (size_t j = 0; j < n_v; j++) ga.v[rg[j]] = v + j * xct;
     ga.out = acc;
     ga.count = n_giant;
     ga.nlimb = n_ext;
