@@ -146,7 +146,6 @@ extern "C" int fhe_bconv_noalloc(fhe_ctx *c, const uint32_t *in, const int *in_i
     x.n = 1;
     x.prime = in_idx[j];
     x.src_stride = 1;
-    x.src_prime = -1;
     x.scale = dPre + j;
     x.galois = 1;
     seg_push(sl, x);

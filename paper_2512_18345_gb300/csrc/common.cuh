@@ -108,7 +108,6 @@ struct Seg {
   int n;             // limbs in the run
   int prime;         // prime index (into q_0.., p_0..) of the first limb
   int src_stride;    // in limbs (0: every limb reads the same source limb)
-  int src_prime;     // prime of the source limb if it differs (rescale), else -1
   const uint2 *scale;  // per-limb Shoup constant pairs (inverse-NTT output scale), or null
   int t0;            // extended-basis index of the first limb (inner product)
   int key_row0;      // key row of the first limb
@@ -182,7 +181,7 @@ struct SegList {
 static_assert(kMaxSeg <= 256, "segof holds a segment index in a byte");
 
 // an empty by-value list: the header alone (the arrays hold what their counts say; clearing the
-// 14 KB of them before each launch was a third of a small call's host time)
+// 12 KB of them before each launch was a third of a small call's host time)
 inline void seg_clear(SegList &l) {
   l.nseg = l.total = l.lm_groups = l.sum_n = 0;
   l.dev = nullptr;

@@ -18,8 +18,8 @@ struct fhe_ctx {
   int fused = 1;
   int comp_pipe = 1;  // complementary pipelining of the inner product (autotuned)
   int fuse_ip_md = 0; // special limbs' inner product fused with ModDown's first INTT pass (autotuned)
-  size_t batch_budget = 0;  // L2 bytes per batched group (0: 3/4 of the L2 size)
-  int batch_max_group = 0;  // items per batched group (0: 8)
+  size_t batch_budget = 0;  // bytes of the batched groups resident at once (0: twice the L2)
+  int batch_max_group = 0;  // items per batched group (0: 8; both 0: the default grouping, batch.cu)
 
   // device tables
   fhe::PrimeC *d_pc = nullptr;
@@ -34,9 +34,9 @@ struct fhe_ctx {
   uint2 *d_pinv = nullptr;                             // [L] P^-1 mod q_i
   uint32_t *d_mdT = nullptr;                           // [L][K] (P/p_k) mod q_i
   int2 *d_mdmap = nullptr;                             // [L] (i, i)
-  uint16_t *d_md_Btc = nullptr;
+  uint16_t *d_md_Btc = nullptr;                        // tensor-core table of the ModDown conversion
   unsigned int *d_gbar = nullptr;                      // grid-barrier counters of the persistent NTT
-  uint2 *d_pmod = nullptr;                             // [L] Shoup pairs of P mod q_i                        // tensor-core table of the ModDown conversion
+  uint2 *d_pmod = nullptr;                             // [L] Shoup pairs of P mod q_i
   unsigned int *d_status = nullptr;                    // device status word (expired waits)
   uint2 *d_rs_qinv = nullptr;                          // [L][L]
   // fhe_bconv: the tables of each (input primes, output primes, kernel) combination, built and
@@ -66,7 +66,7 @@ struct fhe_ctx {
     uint32_t *U = nullptr;    // [2][L+K][N]   inner product
     uint32_t *UC = nullptr;   // [2][K][N]     special limbs in coefficient form
     uint32_t *R = nullptr;    // [2][L][N]     ModDown base conversion
-    uint32_t *D = nullptr;    // [3][L][N]     HMult tensor
+    uint32_t *D = nullptr;    // [3][L][N]     HMult tensor (plain pipeline and NTT variants)
     uint32_t *TMP = nullptr;  // [2][L][N]     plain-pipeline gather
     uint32_t *V = nullptr;    // [2][N]        rescale
   };

@@ -260,9 +260,7 @@ static cudaError_t launch_diag(fhe_ctx *c, const DiagArgs &da, cudaStream_t s) {
 // The baby rotations and the diagonals in one kernel (ip_diag.cuh), up to the kBdGiant giant steps
 // whose sums a warp holds in registers: every further group would read the keys again (1.9 GB of a
 // CoeffToSlot level at L = 48) to spare the baby rotations' 0.9 GB, so more keep the two kernels.
-static bool baby_diag_fits(const fhe_ctx *c, int level, int n_giant) {
-  return c->tabs.ip_staged && n_giant <= kBdGiant && c->beta(level) <= 4 && c->N % kIpChunk == 0;
-}
+static bool baby_diag_fits(const fhe_ctx *c, int n_giant) { return c->tabs.ip_staged && n_giant <= kBdGiant; }
 
 static cudaError_t launch_baby_diag(fhe_ctx *c, const BabyDiagArgs &a, cudaStream_t s) {
   static PerDeviceOnce configured;
@@ -284,11 +282,8 @@ static cudaError_t launch_baby_diag(fhe_ctx *c, const BabyDiagArgs &a, cudaStrea
 }
 
 // The key switches of the giant steps and their sum in one kernel (ip_diag.cuh), wherever the staged
-// gather is on and the digits fit its rows; else IT_IPX items and k_gsum, which also sums a
-// transform without rotating giant steps (nothing to key-switch).
-static bool giant_ip_fits(const fhe_ctx *c, int level) {
-  return c->tabs.ip_staged && c->beta(level) <= 4 && c->N % kIpChunk == 0;
-}
+// gather is on; else IT_IPX items and k_gsum, which also sums a transform without rotating giant
+// steps (nothing to key-switch).
 
 static cudaError_t launch_giant_ip(fhe_ctx *c, const GiantIpArgs &a, cudaStream_t s) {
   static PerDeviceOnce configured;
@@ -588,7 +583,7 @@ extern "C" int fhe_linear_transform_dh(fhe_ctx *c, const uint32_t *ct, int level
     if (gb[b] != 1u) rb.push_back(b);
   for (int g = 0; g < n_giant; g++)
     if (gg[g] != 1u) rg.push_back(g);
-  const bool fused = !rb.empty() && baby_diag_fits(c, level, n_giant), gip = giant_ip_fits(c, level);
+  const bool fused = !rb.empty() && baby_diag_fits(c, n_giant), gip = c->tabs.ip_staged != 0;
   // scratch: inner sums and the accumulator (extended basis, two halves each), the rotating giant
   // steps' c1 halves in Q_l and, where the kernels that use them do not form them, the rotating
   // baby steps and the giant key switches

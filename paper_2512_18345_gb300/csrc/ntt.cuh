@@ -46,7 +46,7 @@ struct NttTables {
 enum : int {
   PRO_PLAIN = 0,   // src[j]
   PRO_GATHER = 1,  // src[sigma(j)], sigma = the limb's galois (NTT form input)
-  PRO_REDUCE = 2,  // src[j] reduced from another prime (rescale: src_prime)
+  PRO_REDUCE = 2,  // src[j] reduced from another prime (rescale)
   PRO_BCONV = 3,   // base conversion of n_in limbs at src (small ring)
   PRO_SUM = 5,     // sum over the list's items at src's place in each item's r (merged ModDowns)
   PRO_MUL = 4,     // src[j] src2[j] where the limb has a src2 (HMult's d2), else as PRO_GATHER
@@ -69,13 +69,10 @@ struct NttGeom {
   static constexpr int C = kTile / S;              // sub-transforms per tile
   static constexpr int LOGD = COLUMN ? LOGN - R : 0;
   static constexpr int TILES = N / kTile;
-  static constexpr int SMEM = (COLUMN && R == 4) ? kTile : kTile + 256;
+  static constexpr int SMEM = kTile + 256;
   // shared-memory address of element k of sub-transform c (bank-conflict free for the rounds)
   static __device__ __forceinline__ int addr(int c, int k) {
-    if (COLUMN) {
-      if (R == 4) return k * 256 + c;
-      return k * 16 + c + ((k >> 4) << 4);
-    }
+    if (COLUMN) return k * 16 + c + ((k >> 4) << 4);
     return c * 272 + ((k >> 4) << 4) + ((k & 15) ^ (k >> 4));
   }
   // index within the limb of element k of sub-transform c in tile `tile`
@@ -138,6 +135,7 @@ __device__ __forceinline__ void ntt_pass(const Limb &lb, const NttTables &tb, in
                                          uint32_t *sm, uint2 *tws, uint32_t *xfer) {
   using G = NttGeom<LOGN, COLUMN>;
   constexpr int R = G::R, N = G::N, S0 = COLUMN ? 0 : LOGN - 8;
+  static_assert(R == 8, "block passes, and column passes of a 2^16 limb: two rounds");
   const int prime = lb.prime;
   const PrimeC P = tb.pc[prime];
   const uint32_t q = P.q;
@@ -159,20 +157,9 @@ __device__ __forceinline__ void ntt_pass(const Limb &lb, const NttTables &tb, in
     if (OTF && tid < kOtfSmall) tws[240 + tid] = __ldg(tw + tid);
   }
 
-  int c, tau;
-  if (COLUMN && R == 4) {
-    c = tid;
-    tau = 0;
-  } else if (COLUMN) {
-    c = tid & 15;
-    tau = tid >> 4;
-  } else {
-    c = tid >> 4;
-    tau = tid & 15;
-  }
-  constexpr int ROUNDS = R / 4;
+  const int c = COLUMN ? tid & 15 : tid >> 4, tau = COLUMN ? tid >> 4 : tid & 15;
   // round 0 is the hi round going forward (large distances first), lo going backward
-  const bool hi0 = (R == 8) && FWD;
+  const bool hi0 = FWD;
 
   // block pass, lo round (stages sigma = 4 + m, m = 0..3): thread (c, tau) uses the 2^m
   // consecutive twiddles 2^(S0+sigma) + ((blk0 + c) << sigma) + (tau << m) + [0, 2^m), each
@@ -267,8 +254,8 @@ __device__ __forceinline__ void ntt_pass(const Limb &lb, const NttTables &tb, in
   }
 
 #pragma unroll
-  for (int rho = 0; rho < ROUNDS; rho++) {
-    const bool hi = (R == 8) && (FWD ? rho == 0 : rho == 1);
+  for (int rho = 0; rho < 2; rho++) {
+    const bool hi = FWD ? rho == 0 : rho == 1;
     if (rho > 0) {  // exchange through shared memory between the rounds
 #pragma unroll
       for (int e = 0; e < 16; e++) sm[G::addr(c, kmap<R>(!hi, e, tau))] = x[e];
@@ -284,7 +271,7 @@ __device__ __forceinline__ void ntt_pass(const Limb &lb, const NttTables &tb, in
       int base;
       if (COLUMN) {
         const int s = R - 1 - kbit;  // Cooley-Tukey stage: psi^brv(2^s + (k_lo >> (kbit + 1)))
-        base = (1 << s) + ((R == 8 && !hi) ? (tau << (3 - bit)) : 0);
+        base = (1 << s) + (!hi ? (tau << (3 - bit)) : 0);
       } else {
         const int sig = 7 - kbit;    // stage within the pass; local index (c << sig) + (k_lo >> (kbit + 1))
         base = 16 * ((1 << sig) - 1) + (c << sig);  // hi round only (sig < 4)
@@ -327,7 +314,7 @@ __device__ __forceinline__ void ntt_pass(const Limb &lb, const NttTables &tb, in
   }
 
   // ---- epilogue straight from registers
-  const bool hiL = (R == 8) && !FWD;  // the last round
+  const bool hiL = !FWD;  // the last round
   if constexpr (DSTM == DST_LOCAL) {  // single-pass kernel: the tile stays in shared memory (lazy values)
     static_assert(LOGN == 16, "the single-pass kernel splits a 2^16 limb into 16 tiles");
 #pragma unroll

@@ -39,8 +39,6 @@ static Seg mkseg(const uint32_t *src, uint32_t *dst, int n, int prime) {
   s.n = n;
   s.prime = prime;
   s.src_stride = 1;
-  s.src_prime = -1;
-
   return s;
 }
 
@@ -230,7 +228,6 @@ extern "C" int fhe_rescale(fhe_ctx *c, const uint32_t *ct, int level, uint32_t *
     uint32_t *o = out + (size_t)cc * (level - 1) * N;
     Seg a = mkseg(V + cc * N, o, level - 1, 0);
     a.src_stride = 0;
-    a.src_prime = level - 1;
     g1.add(a);
     Seg b = mkseg(o, o, level - 1, 0);
     b.src2 = ct + cc * poly;

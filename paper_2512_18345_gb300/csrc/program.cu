@@ -16,7 +16,6 @@ static Seg seg(const uint32_t *src, uint32_t *dst, int n, int prime, int item) {
   s.n = n;
   s.prime = prime;
   s.src_stride = 1;
-  s.src_prime = -1;
   s.item = item;
   s.galois = 1;
   return s;

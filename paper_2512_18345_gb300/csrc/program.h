@@ -62,9 +62,9 @@ struct DevProgram {
 };
 
 int ensure_slots(fhe_ctx *c, int n);
-// fork: the inner product of the ciphertext limbs on an auxiliary branch (complementary pipelining)
 // whether programs may merge the ModDowns of summed rotations (Item::sum)
 bool merge_moddowns(const fhe_ctx *c);
+// fork: the inner product of the ciphertext limbs on an auxiliary branch (complementary pipelining)
 int build_program(fhe_ctx *c, const std::vector<Item> &items, bool fused, bool fork, Program &P);
 // whether the items' program fits by-value launch arguments (program_fits_inline of it, without
 // building it or growing the workspace)
