@@ -170,7 +170,7 @@ def check(rc: int) -> None:
 # integers for pointers and streams, torch looked up once, the current stream's handle without a
 # Stream object, devices by their cached torch.device (11 -> 4 us a call).
 _torch = None
-_devices: dict = {}  # by name
+_devices: dict = {}
 
 
 def _cuda():
@@ -215,10 +215,9 @@ def to_numpy(t) -> np.ndarray:
 
 def empty(shape, device: int = 0):
     torch = _cuda()
-    name = f"cuda:{device}"
-    dev = _devices.get(name)
+    dev = _devices.get(device) if type(device) is int else torch.device(f"cuda:{device}")
     if dev is None:
-        dev = _devices[name] = torch.device(name)
+        dev = _devices[device] = torch.device(f"cuda:{device}")
     return torch.empty(tuple(shape), dtype=torch.int32, device=dev)
 
 
