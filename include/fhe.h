@@ -81,9 +81,11 @@ typedef struct {
   size_t limb_bytes;      /* 4 N */
   size_t key_bytes;       /* dnum * 2 * (L + K) * limb_bytes, one switching key */
   size_t workspace_bytes; /* device scratch the context owns */
-  size_t table_bytes;     /* device twiddle / base-conversion tables */
+  size_t table_bytes;     /* device twiddle / base-conversion tables; the twiddles take 32 N bytes a prime
+                             (both directions, in index order and again in the block passes' thread
+                             order: 126 MB at N = 2^16 with 60 primes), not counted by a memory limit */
   int n_rot_keys;         /* rotation keys currently set */
-  int bconv_mode;         /* FHE_BCONV_SCALAR or FHE_BCONV_TC */
+  int bconv_mode;         /* FHE_BCONV_SCALAR or FHE_BCONV_TC, as selected */
   uint32_t psi[FHE_MAX_PRIMES]; /* psi of q_0..q_{L-1}, p_0..p_{K-1} */
 } fhe_info;
 
@@ -109,7 +111,10 @@ FHE_API int fhe_ctx_info(const fhe_ctx *ctx, fhe_info *out);
  * The tensor-core digit split is exact for at most 12 inputs per conversion: a
  * K = 48 contraction when alpha and K are at most 8, a K = 64 one (signed offset
  * pieces) when they are at most 12.  FHE_EUNSUPPORTED for FHE_BCONV_TC when alpha
- * > 12 or K > 12. */
+ * > 12 or K > 12.  At N = 2^12 the fused calls (every operation and plan but
+ * fhe_bconv; not the plain pipeline nor FHE_NTT_OTF) convert inside their
+ * transforms on CUDA cores whatever is selected: same bits, and a launch less per
+ * conversion; fhe_info.bconv_mode is the selection. */
 FHE_API int fhe_ctx_set_bconv(fhe_ctx *ctx, int mode);
 /*
  * Synchronize the context's device and report device-side failures: returns
